@@ -60,7 +60,7 @@ __global__ void k_lbm_stream(const float *__restrict__ pop, float *__restrict__ 
 __global__ void k_lbm_bouzidi(const int32_t *__restrict__ cell, const uint8_t *__restrict__ dir,
                               const float *__restrict__ q, int64_t n, const float *__restrict__ pop,
                               float *__restrict__ pre, int64_t stride, int64_t ncell, int lattice,
-                              const int32_t *__restrict__ nbr, const uint64_t *__restrict__ mask, int *st)
+                              const int32_t *__restrict__ nbr, const uint64_t *__restrict__ mask, uint32_t *bits, int *st)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -83,26 +83,18 @@ __global__ void k_lbm_bouzidi(const int32_t *__restrict__ cell, const uint8_t *_
         g = f_d / (2.0f * qq) + (2.0f * qq - 1.0f) / (2.0f * qq) * f_o;
     }
     pre[(int64_t)o * stride + c] = g;
+    if (bits) atomicOr(bits + c, 1u << o);
 }
 
+// BGK relaxation of the populations f[0, Q) of a fluid cell, in place.
 template <int Q>
-__global__ void k_lbm_collide(const float *__restrict__ pre, float *__restrict__ out, int64_t stride, int64_t ncell,
-                              const uint64_t *__restrict__ mask, float omega)
+__device__ __forceinline__ void lbm_bgk(float (&f)[Q], float omega)
 {
-    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= ncell) return;
-    if ((mask[x >> 6] >> (x & 63)) & 1ull) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) out[(int64_t)i * stride + x] = 0.0f;
-        return;
-    }
-    float f[Q];
     float rho = 0.0f, jx = 0.0f, jy = 0.0f, jz = 0.0f;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         int cx, cy, cz;
         emb_dir(i, cx, cy, cz);
-        f[i] = pre[(int64_t)i * stride + x];
         rho += f[i];
         jx += cx * f[i];
         jy += cy * f[i];
@@ -120,8 +112,83 @@ __global__ void k_lbm_collide(const float *__restrict__ pre, float *__restrict__
                                 : (kind == 0 ? 8.0f / 27 : (kind == 1 ? 2.0f / 27 : (kind == 2 ? 1.0f / 54 : 1.0f / 216)));
         const float cu = cx * ux + cy * uy + cz * uz;
         const float feq = w * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * usq);
-        out[(int64_t)i * stride + x] = f[i] - omega * (f[i] - feq);
+        f[i] = f[i] - omega * (f[i] - feq);
     }
+}
+
+template <int Q>
+__global__ void k_lbm_collide(const float *__restrict__ pre, float *__restrict__ out, int64_t stride, int64_t ncell,
+                              const uint64_t *__restrict__ mask, float omega)
+{
+    const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= ncell) return;
+    if ((mask[x >> 6] >> (x & 63)) & 1ull) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) out[(int64_t)i * stride + x] = 0.0f;
+        return;
+    }
+    float f[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) f[i] = pre[(int64_t)i * stride + x];
+    lbm_bgk<Q>(f, omega);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) out[(int64_t)i * stride + x] = f[i];
+}
+
+// The whole step in one pass over the cells: the populations are pulled, relaxed in
+// registers and stored, so that each is read once and written once (streaming into
+// `pre` and colliding from it moves them twice).  k_lbm_bouzidi has run before and left
+// the population entering link cell c against c_d in pre[i * stride + c] and bit i in
+// word c of `bits` (row 0 of pre, which no link direction uses); bits is NULL without
+// links.  A CTA holds LBM_BLOCKS blocks, one thread a cell; their 27 neighbour ids and
+// masks are staged in shared memory, so the Q pulls of a cell wait on nothing but each
+// other.  Bound by HBM: 8 Q bytes a cell.
+#define LBM_BLOCKS 4
+template <int Q>
+__global__ void __launch_bounds__(64 * LBM_BLOCKS) k_lbm_step(const float *__restrict__ pop, const float *__restrict__ pre,
+                                                              const uint32_t *__restrict__ bits, float *__restrict__ out,
+                                                              int64_t stride, int64_t nblk,
+                                                              const int32_t *__restrict__ nbr,
+                                                              const uint64_t *__restrict__ mask, float omega)
+{
+    __shared__ uint64_t s_mask[LBM_BLOCKS * 27];
+    __shared__ int32_t s_id[LBM_BLOCKS * 27];
+    const int64_t b0 = (int64_t)blockIdx.x * LBM_BLOCKS;
+    if (threadIdx.x < LBM_BLOCKS * 27) {
+        const int j = threadIdx.x / 27, code = threadIdx.x - 27 * j;
+        int32_t id = -1;
+        if (b0 + j < nblk) id = code == 13 ? (int32_t)(b0 + j) : nbr[(b0 + j) * 26 + c_lbm_dir_of_offset[code] - 1];
+        s_id[threadIdx.x] = id;
+        s_mask[threadIdx.x] = id >= 0 ? mask[id] : 0ull;
+    }
+    __syncthreads();
+    const int j = threadIdx.x >> 6, t = threadIdx.x & 63;
+    const int64_t b = b0 + j;
+    if (b >= nblk) return;
+    const int64_t c = b * 64 + t;
+    if ((s_mask[27 * j + 13] >> t) & 1ull) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) out[(int64_t)i * stride + c] = 0.0f;
+        return;
+    }
+    const uint32_t lk = bits ? bits[c] : 0u;
+    const int x = t & 3, y = (t >> 2) & 3, z = t >> 4;
+    float f[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        int cx, cy, cz;
+        emb_dir(i, cx, cy, cz);
+        const int sx = x - cx, sy = y - cy, sz = z - cz;  // in [-1, 4]
+        const int code = 27 * j + 13 + (cx ? sx >> 2 : 0) + (cy ? 3 * (sy >> 2) : 0) + (cz ? 9 * (sz >> 2) : 0);
+        const int32_t id = s_id[code];
+        const int lt = (sx & 3) + 4 * (sy & 3) + 16 * (sz & 3);
+        const bool linked = (lk >> i) & 1u, solid = (s_mask[code] >> lt) & 1ull;
+        const float *src = linked ? pre + c : pop + (id >= 0 ? (int64_t)id * 64 + lt : c);
+        f[i] = linked || !solid ? src[(int64_t)i * stride] : 0.0f;
+    }
+    lbm_bgk<Q>(f, omega);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) out[(int64_t)i * stride + c] = f[i];
 }
 
 extern "C" emb_status emb_lbm_step(emb_forest f, int32_t lattice, const int32_t *d_cell, const uint8_t *d_dir,
@@ -144,16 +211,35 @@ extern "C" emb_status emb_lbm_step(emb_forest f, int32_t lattice, const int32_t 
     cudaStream_t s = emb_stream(stream);
     emb_status rc = emb_build_neighbors(lv, s);
     if (rc != EMB_OK) return rc;
+    int *st = emb_status_word();
+    if (!st) return EMB_ERR_CUDA;
+    if (phases == 7) {
+        // the boundary populations first, then streaming and collision in one pass
+        uint32_t *bits = n_links > 0 ? (uint32_t *)d_pre : nullptr;
+        if (bits) {
+            EMB_CUDA_TRY(cudaMemsetAsync(bits, 0, ncell * sizeof(uint32_t), s));
+            EMB_LAUNCH((k_lbm_bouzidi), emb_grid(n_links, 256), 256, 0, s)(d_cell, d_dir, d_q, n_links, d_pop, d_pre,
+                                                                           pop_stride, ncell, lattice, lv.nbr, lv.mask,
+                                                                           bits, st);
+        }
+        const int grid = emb_grid(lv.n, LBM_BLOCKS);
+        if (lattice == 19)
+            EMB_LAUNCH((k_lbm_step<19>), grid, 64 * LBM_BLOCKS, 0, s)(d_pop, d_pre, bits, d_pop_out, pop_stride, lv.n,
+                                                                      lv.nbr, lv.mask, omega);
+        else
+            EMB_LAUNCH((k_lbm_step<27>), grid, 64 * LBM_BLOCKS, 0, s)(d_pop, d_pre, bits, d_pop_out, pop_stride, lv.n,
+                                                                      lv.nbr, lv.mask, omega);
+        EMB_CUDA_TRY(cudaGetLastError());
+        return EMB_OK;
+    }
     const int grid = emb_grid(ncell, 256);
     if (phases & 1) {
         if (lattice == 19) EMB_LAUNCH((k_lbm_stream<19>), grid, 256, 0, s)(d_pop, d_pre, pop_stride, ncell, lv.nbr, lv.mask);
         else EMB_LAUNCH((k_lbm_stream<27>), grid, 256, 0, s)(d_pop, d_pre, pop_stride, ncell, lv.nbr, lv.mask);
     }
-    int *st = emb_status_word();
-    if (!st) return EMB_ERR_CUDA;
     if ((phases & 2) && n_links > 0)
         EMB_LAUNCH((k_lbm_bouzidi), emb_grid(n_links, 256), 256, 0, s)(d_cell, d_dir, d_q, n_links, d_pop, d_pre, pop_stride,
-                                                                       ncell, lattice, lv.nbr, lv.mask, st);
+                                                                       ncell, lattice, lv.nbr, lv.mask, nullptr, st);
     if (phases & 4) {
         if (lattice == 19)
             EMB_LAUNCH((k_lbm_collide<19>), grid, 256, 0, s)(d_pre, d_pop_out, pop_stride, ncell, lv.mask, omega);
