@@ -34,27 +34,87 @@ __device__ __forceinline__ int64_t partner_cell(int64_t cell, int cx, int cy, in
     return nb * 64 + lt;
 }
 
-struct LinkTerm {
-    double f_i, f_o, f_p;
+// The cell's populations that the Bouzidi rule of link k reads: f_i, and f_p (below
+// q = 1/2, when the partner cell exists) or f_o (from 1/2 on); the others stay 0.
+struct LinkPops {
+    float q, f_i, f_o, f_p;
     bool has;
     int cx, cy, cz;
 };
 
-__device__ __forceinline__ LinkTerm link_term(int64_t k, const int32_t *__restrict__ cell, const uint8_t *__restrict__ dir,
-                                              const float *__restrict__ pop, int64_t stride,
+__device__ __forceinline__ LinkPops link_pops(int64_t k, const int32_t *__restrict__ cell, const uint8_t *__restrict__ dir,
+                                              const float *__restrict__ q, const float *__restrict__ pop, int64_t stride,
                                               const int32_t *__restrict__ nbr, const uint64_t *__restrict__ mask)
 {
-    LinkTerm L;
-    int64_t c = cell[k];
-    int d = dir[k];
-    int o = (d & 1) ? d + 1 : d - 1;
+    LinkPops L;
+    const int64_t c = cell[k];
+    const int d = dir[k];
+    L.q = q[k];
     emb_dir(d, L.cx, L.cy, L.cz);
     L.f_i = pop[(int64_t)d * stride + c];
-    L.f_o = pop[(int64_t)o * stride + c];
-    int64_t p = partner_cell(c, L.cx, L.cy, L.cz, nbr, mask);
-    L.has = p >= 0;
-    L.f_p = L.has ? (double)pop[(int64_t)d * stride + p] : 0.0;
+    L.f_o = L.f_p = 0.0f;
+    L.has = false;
+    if (L.q < 0.5f) {
+        const int64_t p = partner_cell(c, L.cx, L.cy, L.cz, nbr, mask);
+        L.has = p >= 0;
+        if (L.has) L.f_p = pop[(int64_t)d * stride + p];
+    } else {
+        L.f_o = pop[(int64_t)((d & 1) ? d + 1 : d - 1) * stride + c];
+    }
     return L;
+}
+
+// Pairs of floats (h + l, l below half an ulp of h): the terms below carry about 46 bits
+// with them, at FP32 rate.  This chip has two FP64 lanes a clock and SM against 128 FP32
+// ones: with the same terms in FP64 both kernels were bound by them (1.72 M links, D3Q19:
+// force 120 -> 14 us with the link's cells in L2, 42 us from HBM; dF/dq 92 -> 9 us).
+// Bound now by the gathers of the populations.
+struct F2 {
+    float h, l;
+};
+__device__ __forceinline__ F2 two_sum(float a, float b)
+{
+    const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+    return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ F2 two_prod(float a, float b)
+{
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ F2 f2_norm(float h, float l)  // |h| >= |l|
+{
+    const float s = __fadd_rn(h, l);
+    return {s, __fsub_rn(l, __fsub_rn(s, h))};
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b)
+{
+    const F2 s = two_sum(a.h, b.h);
+    return f2_norm(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b)
+{
+    const F2 p = two_prod(a.h, b.h);
+    return f2_norm(p.h, __fadd_rn(p.l, __fmaf_rn(a.h, b.l, __fmul_rn(a.l, b.h))));
+}
+__device__ __forceinline__ F2 f2_div(F2 a, F2 b)
+{
+    const float x = __fdiv_rn(a.h, b.h);
+    const float r = __fadd_rn(__fmaf_rn(-x, b.h, a.h), __fmaf_rn(-x, b.l, a.l));
+    return f2_norm(x, __fdiv_rn(r, b.h));
+}
+__device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
+
+// Zero, or a magnitude in [2^-40, 2^41): sums, products and quotients of a few such values
+// neither overflow nor lose low parts to underflow.
+__device__ __forceinline__ bool f2_safe(float a)
+{
+    const uint32_t e = (__float_as_uint(a) >> 23) & 255u;
+    return e - 87u <= 80u || a == 0.0f;
+}
+__device__ __forceinline__ bool link_safe(const LinkPops &L)
+{
+    return L.q >= 0.0f && L.q <= 1.0f && f2_safe(L.f_i) && f2_safe(L.f_o) && f2_safe(L.f_p);
 }
 
 // Fixed-order block reduction of three doubles; thread 0 receives the sums.
@@ -84,22 +144,61 @@ __global__ void __launch_bounds__(MEX_BLOCK) k_mex_partial(const int32_t *__rest
                                                            const int32_t *__restrict__ nbr,
                                                            const uint64_t *__restrict__ mask, double *__restrict__ part)
 {
-    double fx = 0, fy = 0, fz = 0;
+    F2 ax = {0.0f, 0.0f}, ay = ax, az = ax;
+    double fx = 0, fy = 0, fz = 0;  // links outside the pairs' range (NaN and infinities too)
+    bool wild = false;
     for (int64_t k = (int64_t)blockIdx.x * MEX_BLOCK + threadIdx.x; k < n; k += (int64_t)gridDim.x * MEX_BLOCK) {
-        LinkTerm L = link_term(k, cell, dir, pop, stride, nbr, mask);
-        double qq = q[k], g;
-        if (qq < 0.5) g = L.has ? 2.0 * qq * L.f_i + (1.0 - 2.0 * qq) * L.f_p : L.f_i;
-        else g = L.f_i / (2.0 * qq) + (2.0 * qq - 1.0) / (2.0 * qq) * L.f_o;
-        double m = L.f_i + g;
-        fx += L.cx * m;
-        fy += L.cy * m;
-        fz += L.cz * m;
+        const LinkPops L = link_pops(k, cell, dir, q, pop, stride, nbr, mask);
+        if (link_safe(L)) {
+            const float q2 = 2.0f * L.q;
+            F2 m;  // f_i plus the population returned against it
+            if (L.q < 0.5f) {
+                // 2 f_i, or f_i + 2q f_i + (1 - 2q) f_p
+                m = {2.0f * L.f_i, 0.0f};
+                if (L.has) {
+                    const F2 w = two_sum(1.0f, -q2);
+                    F2 b = two_prod(w.h, L.f_p);
+                    b.l = __fmaf_rn(w.l, L.f_p, b.l);
+                    m = f2_add(f2_add(two_prod(q2, L.f_i), b), {L.f_i, 0.0f});
+                }
+            } else {
+                // f_i + (f_i + (2q - 1) f_o) / 2q; 2q - 1 is exact on [1/2, 1]
+                const F2 N = f2_add(two_prod(__fsub_rn(q2, 1.0f), L.f_o), {L.f_i, 0.0f});
+                m = f2_add(f2_div(N, {q2, 0.0f}), {L.f_i, 0.0f});
+            }
+            if (L.cx) ax = f2_add(ax, L.cx > 0 ? m : f2_neg(m));
+            if (L.cy) ay = f2_add(ay, L.cy > 0 ? m : f2_neg(m));
+            if (L.cz) az = f2_add(az, L.cz > 0 ? m : f2_neg(m));
+        } else {
+            const double qq = L.q, f_i = L.f_i;
+            double g;
+            if (qq < 0.5) g = L.has ? 2.0 * qq * f_i + (1.0 - 2.0 * qq) * (double)L.f_p : f_i;
+            else g = f_i / (2.0 * qq) + (2.0 * qq - 1.0) / (2.0 * qq) * (double)L.f_o;
+            const double m = f_i + g;
+            fx += L.cx * m;
+            fy += L.cy * m;
+            fz += L.cz * m;
+            wild = true;
+        }
     }
-    block_sum3(fx, fy, fz);
-    if (threadIdx.x == 0) {
-        part[3 * blockIdx.x + 0] = fx;
-        part[3 * blockIdx.x + 1] = fy;
-        part[3 * blockIdx.x + 2] = fz;
+    // the warps' pairs first (FP32), then one FP64 value a warp
+    __shared__ double s_warp[3][MEX_BLOCK / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ax = f2_add(ax, {__shfl_xor_sync(0xffffffffu, ax.h, o), __shfl_xor_sync(0xffffffffu, ax.l, o)});
+        ay = f2_add(ay, {__shfl_xor_sync(0xffffffffu, ay.h, o), __shfl_xor_sync(0xffffffffu, ay.l, o)});
+        az = f2_add(az, {__shfl_xor_sync(0xffffffffu, az.h, o), __shfl_xor_sync(0xffffffffu, az.l, o)});
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s_warp[0][threadIdx.x >> 5] = (double)ax.h + (double)ax.l;
+        s_warp[1][threadIdx.x >> 5] = (double)ay.h + (double)ay.l;
+        s_warp[2][threadIdx.x >> 5] = (double)az.h + (double)az.l;
+    }
+    if (__syncthreads_or(wild)) block_sum3(fx, fy, fz);
+    if (threadIdx.x < 3) {
+        double v = threadIdx.x == 0 ? s_warp[0][0] : (threadIdx.x == 1 ? s_warp[1][0] : s_warp[2][0]);
+        for (int w = 1; w < MEX_BLOCK / 32; ++w) v += s_warp[threadIdx.x][w];
+        part[3 * blockIdx.x + threadIdx.x] = v + (threadIdx.x == 0 ? fx : (threadIdx.x == 1 ? fy : fz));
     }
 }
 
@@ -125,11 +224,24 @@ __global__ void k_mex_bwd(const int32_t *__restrict__ cell, const uint8_t *__res
 {
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    LinkTerm L = link_term(k, cell, dir, pop, stride, nbr, mask);
-    double qq = q[k], g;
-    if (qq < 0.5) g = L.has ? 2.0 * (L.f_i - L.f_p) : 0.0;
-    else g = (L.f_o - L.f_i) / (2.0 * qq * qq);
-    double s = (double)gF[0] * L.cx + (double)gF[1] * L.cy + (double)gF[2] * L.cz;
+    const LinkPops L = link_pops(k, cell, dir, q, pop, stride, nbr, mask);
+    const float gx = gF[0], gy = gF[1], gz = gF[2];
+    if (link_safe(L) && f2_safe(gx) && f2_safe(gy) && f2_safe(gz)) {
+        const F2 s = f2_add(two_sum(L.cx * gx, L.cy * gy), {L.cz * gz, 0.0f});
+        F2 r = {0.0f, 0.0f};
+        if (L.q < 0.5f) {
+            if (L.has) r = f2_mul(s, two_sum(2.0f * L.f_i, -2.0f * L.f_p));
+        } else {
+            r = f2_div(f2_mul(s, two_sum(L.f_o, -L.f_i)), two_prod(2.0f * L.q, L.q));
+        }
+        gq[k] = r.h;
+        return;
+    }
+    const double qq = L.q, f_i = L.f_i;
+    double g;
+    if (qq < 0.5) g = L.has ? 2.0 * (f_i - (double)L.f_p) : 0.0;
+    else g = ((double)L.f_o - f_i) / (2.0 * qq * qq);
+    const double s = (double)gx * L.cx + (double)gy * L.cy + (double)gz * L.cz;
     gq[k] = (float)(s * g);
 }
 
