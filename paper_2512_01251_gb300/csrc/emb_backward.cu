@@ -2,9 +2,10 @@
 // derivative with respect to q, and the adjoint of q with respect to the
 // vertices (Sec. 2.2 cites both methods; Sec. 3.4 builds the q table they use).
 //
-// All reductions have a fixed order: per-CTA trees in FP64 followed by one CTA
-// summing the partials in index order, and per-vertex sums taken in ascending
-// (link, corner) order.  No floating-point atomics are used.
+// All reductions are independent of the order in which the GPU runs: the force takes
+// per-thread and per-warp sums of float pairs, per-CTA sums in FP64 and one CTA over the
+// partials in index order; the per-vertex sums are integers.  No floating-point atomics
+// are used.
 #include <mutex>
 
 #include "emb_internal.cuh"
@@ -392,107 +393,305 @@ extern "C" emb_status emb_mex_force_noalloc(emb_forest f, int32_t lattice, const
 // ---------------------------------------------------------------------------
 // dq/dV adjoint
 // ---------------------------------------------------------------------------
-// Per link k and corner j of its triangle: gq_k lambda_j n / (h n.c), world units.
-__global__ void k_qbwd_terms(const uint64_t *__restrict__ key, LevelGeom g, double scale, const int32_t *__restrict__ cell,
-                             const uint8_t *__restrict__ dir, const float *__restrict__ q, const int32_t *__restrict__ tri,
-                             const float *__restrict__ gq, int64_t n, const int4 *__restrict__ rec, int64_t T,
-                             float *__restrict__ val, int32_t *__restrict__ vid, uint32_t *__restrict__ vcnt, int *st)
+// Link k adds gq_k lambda_j n / (h n.c) to vertex j of its triangle (world units).  With
+// the vertices relative to the cell centre, V_A = c . (B x C) and so on are integers and
+// lambda_j = V_j / (c . n), c . n = V_A + V_B + V_C: the sum over a triangle's links
+// needs one scalar S_j = sum gq_k K V_j / (c . n)^2 per vertex (K = 2^20 r_o / h), and
+// the normal n multiplies it once.
+//
+// Sums are taken in integers, so that their order does not matter and the atomics that
+// form them give the same result every time:
+//   k_qbwd_tile    a CTA takes QB_TILE consecutive links (neighbours in space, so they
+//                  share triangles); per (tile, triangle) it finds the largest exponent
+//                  of each of the three terms, then adds the terms as multiples of 2^-41
+//                  of it.  One entry per (tile, triangle) is written, and the exponent
+//                  bound of its nine products S_j n_d is raised into the vertices';
+//   k_qbwd_scatter one thread per entry adds the nine products to the vertices, as
+//                  multiples of the vertex component's own quantum;
+//   k_qbwd_write   the sums as floats.
+// Listing every (link, vertex) term and ranking a vertex's list against itself (the
+// earlier form) costs c^2 for c terms at a vertex: 8.9 ms on a body of 999 triangles whose
+// vertices meet 3,600 links each, and 560 us on 111 K triangles with 1.72 M links, most of
+// it FP64 terms.  Now 53 us on the first, bound by the shared-memory atomics and the gathers
+// of the tile kernel.  A tile of 512 links keeps three CTAs an SM (29 KB, 80 registers).
+#define QB_BLOCK 256
+#define QB_PER 2
+#define QB_TILE (QB_BLOCK * QB_PER)
+#define QB_HASH (2 * QB_TILE)
+#define QB_BITS 42  // a term is less than 2^QB_BITS quanta of its entry: two limbs of 21 bits
+#define QB_NONE (-(1 << 30))
+#define QB_NAN 1u
+#define QB_PINF 2u
+#define QB_NINF 4u
+
+// S_j = m[j] 2^e[j] of one triangle over one tile; bits 3j .. 3j + 2 of `flag` hold
+// QB_NAN, QB_PINF and QB_NINF if a term was not finite.
+struct __align__(16) QbEntry {
+    int tri;
+    uint32_t flag;
+    int e[3];
+    int pad;
+    long long m[3];
+};
+
+__device__ __forceinline__ float exp2i(int e) { return __int_as_float((127 + e) << 23); }  // e in [-126, 127]
+
+// v 2^-k as a pair (|v| < 2^62)
+__device__ __forceinline__ F2 f2_of_ll(long long v, float scale)
 {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    int64_t tr = tri[k];
-    if (tr < 0 || tr >= T) {
-        emb_set_status(st, EMB_ERR_BAD_INPUT);
-        for (int j = 0; j < 3; ++j) vid[3 * k + j] = -1;
-        return;
-    }
-    int4 A = rec[3 * tr], B = rec[3 * tr + 1], C = rec[3 * tr + 2];
-    int64_t c = cell[k];
-    uint64_t bk = key[c >> 6];
-    int t = (int)(c & 63);
-    long long gx = 4 * (long long)(bk & EMB_KEY_MASK) + (t & 3);
-    long long gy = 4 * (long long)((bk >> EMB_KEY_BITS) & EMB_KEY_MASK) + ((t >> 2) & 3);
-    long long gz = 4 * (long long)(bk >> (2 * EMB_KEY_BITS)) + (t >> 4);
-    int cx, cy, cz;
-    emb_dir(dir[k], cx, cy, cz);
-    // coordinates relative to A (exact integers in double)
-    double bx = (double)B.x - A.x, by = (double)B.y - A.y, bz = (double)B.z - A.z;
-    double qx = (double)C.x - A.x, qy = (double)C.y - A.y, qz = (double)C.z - A.z;
-    double s_ = (double)q[k] * (double)g.h;
-    double xx = (double)((2 * gx + 1) * g.half - A.x) + s_ * cx;
-    double xy = (double)((2 * gy + 1) * g.half - A.y) + s_ * cy;
-    double xz = (double)((2 * gz + 1) * g.half - A.z) + s_ * cz;
-    double nx = by * qz - bz * qy, ny = bz * qx - bx * qz, nz = bx * qy - by * qx;
-    double nn = nx * nx + ny * ny + nz * nz;
-    double nc = nx * cx + ny * cy + nz * cz;
+    const float h = (float)v;
+    return {h * scale, (float)(v - (long long)h) * scale};
+}
+
+__device__ __forceinline__ void tri_normal(const int4 &A, const int4 &B, const int4 &C, long long n[3])
+{
+    const int ux = B.x - A.x, uy = B.y - A.y, uz = B.z - A.z, vx = C.x - A.x, vy = C.y - A.y, vz = C.z - A.z;
+    n[0] = (long long)uy * vz - (long long)uz * vy;
+    n[1] = (long long)uz * vx - (long long)ux * vz;
+    n[2] = (long long)ux * vy - (long long)uy * vx;
+}
+
+// a . (b x c) for a lattice direction c: |b x c| < 2^27, |a . (b x c)| < 2^55
+__device__ __forceinline__ long long lat_det(const int a[3], const int b[3], int cx, int cy, int cz)
+{
+    return (long long)a[0] * (b[1] * cz - b[2] * cy) + (long long)a[1] * (b[2] * cx - b[0] * cz) +
+           (long long)a[2] * (b[0] * cy - b[1] * cx);
+}
+
+// The three terms of one link in FP64 with the hit point taken at the given q, for a q
+// that is not the link's crossing, a line parallel to its triangle, and a gq that is no
+// normal number; non-finite terms come back as flags.
+__device__ __noinline__ uint32_t qb_terms_wide(const int a[3], const int b[3], const int c3[3], const long long n[3],
+                                               int cx, int cy, int cz, double s_, double f, F2 t[3], int &ex)
+{
+    const double bx = (double)b[0] - a[0], by = (double)b[1] - a[1], bz = (double)b[2] - a[2];
+    const double qx = (double)c3[0] - a[0], qy = (double)c3[1] - a[1], qz = (double)c3[2] - a[2];
+    const double xx = s_ * cx - a[0], xy = s_ * cy - a[1], xz = s_ * cz - a[2];
+    const double nx = (double)n[0], ny = (double)n[1], nz = (double)n[2];
+    const double nn = nx * nx + ny * ny + nz * nz;
     // X = lB B' + lC C':  X x C' = lB n,  B' x X = lC n
-    double lB = (nx * (xy * qz - xz * qy) + ny * (xz * qx - xx * qz) + nz * (xx * qy - xy * qx)) / nn;
-    double lC = (nx * (by * xz - bz * xy) + ny * (bz * xx - bx * xz) + nz * (bx * xy - by * xx)) / nn;
-    double lA = 1.0 - lB - lC;
-    double f = (double)gq[k] * scale / ((double)g.h * nc);
-    double lam[3] = {lA, lB, lC};
-    int ids[3] = {A.w, B.w, C.w};
+    const double lB = (nx * (xy * qz - xz * qy) + ny * (xz * qx - xx * qz) + nz * (xx * qy - xy * qx)) / nn;
+    const double lC = (nx * (by * xz - bz * xy) + ny * (bz * xx - bx * xz) + nz * (bx * xy - by * xx)) / nn;
+    f /= nx * cx + ny * cy + nz * cz;
+    const double w[3] = {f * (1.0 - lB - lC), f * lB, f * lC};
+    uint32_t flag = 0;
+    ex = QB_NONE;
     for (int j = 0; j < 3; ++j) {
-        double w = f * lam[j];
-        val[3 * (3 * k + j) + 0] = (float)(w * nx);
-        val[3 * (3 * k + j) + 1] = (float)(w * ny);
-        val[3 * (3 * k + j) + 2] = (float)(w * nz);
-        vid[3 * k + j] = ids[j];
-        atomicAdd(vcnt + ids[j], 1u);
+        if (isnan(w[j])) flag |= QB_NAN << (3 * j);
+        else if (isinf(w[j])) flag |= (w[j] > 0 ? QB_PINF : QB_NINF) << (3 * j);
+        else if (w[j] != 0.0) ex = max(ex, ilogb(w[j]));
     }
+    for (int j = 0; j < 3; ++j) {
+        t[j] = {0.0f, 0.0f};
+        if (!isfinite(w[j]) || w[j] == 0.0) continue;
+        const double m = scalbn(w[j], -ex);
+        if (fabs(m) < 0x1p-100) continue;  // its scale would leave the float range
+        t[j].h = (float)m;
+        t[j].l = (float)(m - (double)t[j].h);
+    }
+    return flag;
 }
 
-__global__ void k_qbwd_fill(const int32_t *__restrict__ vid, int64_t m, const uint32_t *__restrict__ voff,
-                            uint32_t *__restrict__ cur, uint32_t *__restrict__ slot)
+__global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restrict__ key, LevelGeom g, int r_o,
+                                                         const int32_t *__restrict__ cell, const uint8_t *__restrict__ dir,
+                                                         const float *__restrict__ q, const int32_t *__restrict__ tri,
+                                                         const float *__restrict__ gq, int64_t n,
+                                                         const int4 *__restrict__ rec, int64_t T,
+                                                         QbEntry *__restrict__ ent, int *__restrict__ tile_n,
+                                                         int *__restrict__ vexp, uint32_t *__restrict__ vflag, int *st)
 {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m) return;
-    int32_t v = vid[e];
-    if (v < 0) return;
-    uint32_t p = atomicAdd(cur + v, 1u);
-    slot[voff[v] + p] = (uint32_t)e;
-}
-
-// One warp per vertex.  The fill left a vertex's entries unordered in slot[a, b);
-// each lane ranks its entries among all of them (entry ids are distinct) and
-// stores them at their rank in `sorted`, so sorted[a, b) ascends.  After a warp
-// barrier lane l sums the entries of ranks l, l + 32, l + 64, ... in that order
-// and the 32 lane sums meet in a fixed butterfly: the result does not depend on
-// the order the atomics of the fill happened to take.  Work per vertex is
-// c^2 / 32 comparisons per lane for c entries.
-__global__ void k_qbwd_reduce(const uint32_t *__restrict__ voff, const uint32_t *__restrict__ slot,
-                              uint32_t *__restrict__ sorted, const float *__restrict__ val, int64_t V,
-                              float *__restrict__ gv)
-{
-    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (v >= V) return;  // uniform per warp
-    const uint32_t a = voff[v], b = voff[v + 1];
-    for (uint32_t i = a + lane; i < b; i += 32) {
-        const uint32_t e = slot[i];
-        uint32_t r = 0;
-        for (uint32_t j = a; j < b; ++j) r += slot[j] < e;
-        sorted[a + r] = e;
-    }
-    __syncwarp();
-    double sx = 0, sy = 0, sz = 0;
-    for (uint32_t i = a + lane; i < b; i += 32) {
-        const int64_t e = sorted[i];
-        sx += val[3 * e];
-        sy += val[3 * e + 1];
-        sz += val[3 * e + 2];
-    }
+    __shared__ int s_key[QB_HASH];                     // triangle of a hash slot (-1: free)
+    __shared__ uint16_t s_idx[QB_HASH];                // its entry
+    __shared__ int s_tri[QB_TILE], s_emax[3][QB_TILE];
+    __shared__ int s_hi[3][QB_TILE], s_lo[3][QB_TILE];
+    __shared__ uint32_t s_flag[QB_TILE];
+    __shared__ int s_n;
+    for (int i = threadIdx.x; i < QB_HASH; i += QB_BLOCK) s_key[i] = -1;
+    for (int i = threadIdx.x; i < QB_TILE; i += QB_BLOCK) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        sx += __shfl_xor_sync(0xffffffffu, sx, o);
-        sy += __shfl_xor_sync(0xffffffffu, sy, o);
-        sz += __shfl_xor_sync(0xffffffffu, sz, o);
+        for (int j = 0; j < 3; ++j) {
+            s_emax[j][i] = QB_NONE;
+            s_hi[j][i] = s_lo[j][i] = 0;
+        }
+        s_flag[i] = 0;
     }
-    if (lane == 0) {
-        gv[3 * v] = (float)sx;
-        gv[3 * v + 1] = (float)sy;
-        gv[3 * v + 2] = (float)sz;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    const int64_t k0 = (int64_t)blockIdx.x * QB_TILE;
+    F2 t[QB_PER][3];
+    int ea[QB_PER], slot[QB_PER];
+    uint32_t flag[QB_PER];
+#pragma unroll
+    for (int u = 0; u < QB_PER; ++u) {
+        const int64_t k = k0 + u * QB_BLOCK + threadIdx.x;
+        slot[u] = -1;
+        flag[u] = 0;
+        ea[u] = 0;
+        if (k >= n) continue;
+        const int64_t tr = tri[k];
+        if (tr < 0 || tr >= T) {
+            emb_set_status(st, EMB_ERR_BAD_INPUT);
+            continue;
+        }
+        // the triangle's slot: at most QB_TILE of the QB_HASH slots are taken
+        int s = (int)((uint32_t)tr * 2654435761u >> 16) & (QB_HASH - 1);
+        for (;;) {
+            int have = *(volatile int *)&s_key[s];
+            if (have == -1) {
+                have = atomicCAS(&s_key[s], -1, (int)tr);
+                if (have == -1) {
+                    const int e = atomicAdd(&s_n, 1);
+                    s_idx[s] = (uint16_t)e;
+                    s_tri[e] = (int)tr;
+                    have = (int)tr;
+                }
+            }
+            if (have == (int)tr) break;
+            s = (s + 1) & (QB_HASH - 1);
+        }
+        slot[u] = s;
+        const int4 A = rec[3 * tr], B = rec[3 * tr + 1], C = rec[3 * tr + 2];
+        const int64_t c = cell[k];
+        const uint64_t bk = key[c >> 6];
+        const int tc = (int)(c & 63), half = (int)g.half;
+        const int px = (2 * (4 * (int)(bk & EMB_KEY_MASK) + (tc & 3)) + 1) * half;
+        const int py = (2 * (4 * (int)((bk >> EMB_KEY_BITS) & EMB_KEY_MASK) + ((tc >> 2) & 3)) + 1) * half;
+        const int pz = (2 * (4 * (int)(bk >> (2 * EMB_KEY_BITS)) + (tc >> 4)) + 1) * half;
+        int cx, cy, cz;
+        emb_dir(dir[k], cx, cy, cz);
+        const int a[3] = {A.x - px, A.y - py, A.z - pz}, b[3] = {B.x - px, B.y - py, B.z - pz},
+                  d[3] = {C.x - px, C.y - py, C.z - pz};
+        const long long V[3] = {lat_det(b, d, cx, cy, cz), lat_det(d, a, cx, cy, cz), lat_det(a, b, cx, cy, cz)};
+        const long long nc = V[0] + V[1] + V[2];  // c . n
+        long long nn[3];
+        tri_normal(A, B, C, nn);
+        const float qk = q[k], gk = gq[k];
+        // the crossing of the link's line with the plane, D / (h c.n) in steps of the link: a
+        // q that is not it (within 2^-20, rounding included) takes the general path
+        const i128 D = mul128(nn[0], a[0]) + mul128(nn[1], a[1]) + mul128(nn[2], a[2]);
+        const long long M = nc < 0 ? -nc : nc;
+        const float Nf = D < 0 ? -i128_to_float(-D) : i128_to_float(D), Mh = (float)M * (float)g.h;
+        const uint32_t ge = (__float_as_uint(gk) >> 23) & 255u;
+        const bool usual = M != 0 && fabsf(qk * Mh - (nc < 0 ? -Nf : Nf)) <= 0x1p-20f * Mh &&
+                           (gk == 0.0f || ge - 1u < 254u);
+        if (usual) {
+            const int kb = 63 - __clzll(M);
+            const float sc = exp2i(-kb);
+            const F2 m = f2_of_ll(M, sc);
+            // 1 / m to second order, squared; times the mantissa of gq and r_o
+            const float r1 = __frcp_rn(m.h);
+            const F2 r = f2_norm(r1, r1 * __fadd_rn(__fmaf_rn(-r1, m.h, 1.0f), -r1 * m.l));
+            const float gm = gk == 0.0f ? 0.0f : __uint_as_float((__float_as_uint(gk) & 0x807FFFFFu) | 0x3F800000u);
+            const F2 w = f2_mul(two_prod(gm, (float)r_o), f2_mul(r, r));
+#pragma unroll
+            for (int j = 0; j < 3; ++j) t[u][j] = f2_mul(f2_of_ll(V[j], sc), w);
+            ea[u] = (int)ge - 127 + (20 - g.lh) - kb;
+        } else {
+            flag[u] = qb_terms_wide(a, b, d, nn, cx, cy, cz, (double)qk * (double)g.h,
+                                    (double)gk * (1048576.0 * (double)r_o) / (double)g.h, t[u], ea[u]);
+        }
     }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < QB_PER; ++u) {
+        if (slot[u] < 0) continue;
+        const int e = s_idx[slot[u]];
+        slot[u] = e;
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+            if (t[u][j].h != 0.0f)
+                atomicMax(&s_emax[j][e], (int)((__float_as_uint(t[u][j].h) >> 23) & 255u) - 127 + ea[u]);
+        if (flag[u]) atomicOr(&s_flag[e], flag[u]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < QB_PER; ++u) {
+        if (slot[u] < 0) continue;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            // |term| 2^ea < 2^(emax + 1): below 2^21 in units of 2^(emax + 1 - 21), the high limb
+            const int sh = ea[u] - s_emax[j][slot[u]] + QB_BITS / 2 - 1;
+            if (t[u][j].h == 0.0f || sh < -100) continue;
+            const float f = exp2i(sh), x = t[u][j].h * f, hi = floorf(x);
+            const int lo = __float2int_rn(__fmaf_rn(t[u][j].l, f, x - hi) * (float)(1 << (QB_BITS / 2)));
+            atomicAdd(&s_hi[j][slot[u]], (int)hi);
+            atomicAdd(&s_lo[j][slot[u]], lo);
+        }
+    }
+    __syncthreads();
+    const int cnt = s_n;
+    for (int i = threadIdx.x; i < cnt; i += QB_BLOCK) {
+        QbEntry E;
+        E.tri = s_tri[i];
+        E.flag = s_flag[i];
+        E.pad = 0;
+        const int4 A = rec[3 * (int64_t)E.tri], B = rec[3 * (int64_t)E.tri + 1], C = rec[3 * (int64_t)E.tri + 2];
+        const int vid[3] = {A.w, B.w, C.w};
+        long long nn[3];
+        tri_normal(A, B, C, nn);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            E.m[j] = ((long long)s_hi[j][i] << (QB_BITS / 2)) + s_lo[j][i];
+            E.e[j] = s_emax[j][i] + 1 - QB_BITS;
+            const uint32_t fl = (E.flag >> (3 * j)) & 7u;
+            if (E.m[j] == 0 && !fl) continue;
+            const int mb = 64 - __clzll(E.m[j] < 0 ? -E.m[j] : E.m[j]);
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                const int64_t at = 3 * (int64_t)vid[j] + x;
+                if (E.m[j] != 0 && nn[x] != 0)
+                    atomicMax(vexp + at, E.e[j] + mb + 64 - __clzll(nn[x] < 0 ? -nn[x] : nn[x]));
+                // an infinite term times a component of n: its sign, or NaN where that is 0
+                if (fl)
+                    atomicOr(vflag + at, nn[x] == 0 ? QB_NAN
+                                                    : (nn[x] > 0 ? fl : (fl & QB_NAN) | ((fl & QB_PINF) << 1) | ((fl & QB_NINF) >> 1)));
+            }
+        }
+        ent[k0 + i] = E;
+    }
+    if (threadIdx.x == 0) tile_n[blockIdx.x] = cnt;
+}
+
+// A vertex component's quantum is 2^(vexp - qbits): 3n terms of less than 2^vexp each stay
+// below 2^63 in it.
+__global__ void __launch_bounds__(QB_BLOCK) k_qbwd_scatter(const QbEntry *__restrict__ ent, const int *__restrict__ tile_n,
+                                                            const int4 *__restrict__ rec, const int *__restrict__ vexp,
+                                                            int qbits, unsigned long long *__restrict__ vacc)
+{
+    const int cnt = tile_n[blockIdx.x];
+    for (int i = threadIdx.x; i < cnt; i += QB_BLOCK) {
+        const QbEntry E = ent[(int64_t)blockIdx.x * QB_TILE + i];
+        const int4 A = rec[3 * (int64_t)E.tri], B = rec[3 * (int64_t)E.tri + 1], C = rec[3 * (int64_t)E.tri + 2];
+        const int vid[3] = {A.w, B.w, C.w};
+        long long nn[3];
+        tri_normal(A, B, C, nn);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+#pragma unroll
+            for (int x = 0; x < 3; ++x) {
+                if (E.m[j] == 0 || nn[x] == 0) continue;
+                const int64_t at = 3 * (int64_t)vid[j] + x;
+                const int sh = vexp[at] - qbits - E.e[j];  // quanta of E.e per quantum of the vertex, log2
+                const i128 P = mul128(E.m[j], nn[x]);
+                if (sh > 120) continue;
+                const long long v = sh > 0 ? (long long)((P + ((i128)1 << (sh - 1))) >> sh) : (long long)(P << -sh);
+                if (v) atomicAdd(vacc + at, (unsigned long long)v);
+            }
+        }
+    }
+}
+
+__global__ void k_qbwd_write(const int *__restrict__ vexp, const uint32_t *__restrict__ vflag,
+                             const unsigned long long *__restrict__ vacc, int64_t m, int qbits, float *__restrict__ gv)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    const long long v = (long long)vacc[i];
+    const uint32_t fl = vflag[i];
+    float r = 0.0f;
+    if (v) r = (float)scalbn((double)v, vexp[i] - qbits);
+    if (fl) r = fl == QB_PINF ? INFINITY : (fl == QB_NINF ? -INFINITY : NAN);
+    gv[i] = r;
 }
 
 extern "C" emb_status emb_cutlinks_backward(emb_mesh m, emb_forest f, const int32_t *d_cell, const uint8_t *d_dir,
@@ -509,32 +708,29 @@ extern "C" emb_status emb_cutlinks_backward(emb_mesh m, emb_forest f, const int3
     if (!st) return EMB_ERR_CUDA;
     const EmbLevel &lv = f->lv[f->max_level];
     LevelGeom g = level_geom(f, f->max_level);
-    double scale = (double)(1ll << 20) * (double)f->r_o;
-    // one scratch allocation: val (9n floats), vid (3n), slot (3n), vcnt and voff (V + 1 each), scan scratch
-    const size_t a_val = (size_t)(9 * n + 1) * sizeof(float), a_ent = (size_t)(3 * n + 1) * sizeof(uint32_t),
-                 a_v = (size_t)(m->V + 1) * sizeof(uint32_t), a_tmp = emb_scan_tmp_words(m->V) * sizeof(uint64_t);
+    // one scratch allocation: vertex sums and flags (3V each, zeroed), their exponents (3V,
+    // 0x80 bytes), the entries (QB_TILE a tile) and their counts
+    const int64_t nt = (n + QB_TILE - 1) / QB_TILE, m3 = 3 * m->V;
+    const size_t a_acc = (size_t)m3 * sizeof(uint64_t), a_v = (size_t)m3 * sizeof(uint32_t),
+                 a_tn = (size_t)(nt + 1) * sizeof(int), a_ent = (size_t)(nt * QB_TILE) * sizeof(QbEntry);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     char *scratch = nullptr;
-    EMB_CUDA_TRY(emb_malloc_async((void **)&scratch, up(a_val) + 2 * up(a_ent) + 2 * up(a_v) + up(a_tmp), s));
-    float *val = (float *)scratch;
-    int32_t *vid = (int32_t *)(scratch + up(a_val));
-    uint32_t *slot = (uint32_t *)(scratch + up(a_val) + up(a_ent));
-    uint32_t *vcnt = (uint32_t *)(scratch + up(a_val) + 2 * up(a_ent));
-    uint32_t *voff = (uint32_t *)(scratch + up(a_val) + 2 * up(a_ent) + up(a_v));
-    uint64_t *tmp = (uint64_t *)(scratch + up(a_val) + 2 * up(a_ent) + 2 * up(a_v));
-    EMB_CUDA_TRY(cudaMemsetAsync(vcnt, 0, (m->V + 1) * sizeof(uint32_t), s));
-    if (n > 0)
-        EMB_LAUNCH((k_qbwd_terms), emb_grid(n, 256), 256, 0, s)(lv.key, g, scale, d_cell, d_dir, d_q, d_tri, d_gq, n, m->rec, m->T,
-                                                      val, vid, vcnt, st);
-    emb_status rc = emb_scan_into(vcnt, voff, m->V, tmp, s);
-    if (rc != EMB_OK) {
-        cudaFreeAsync(scratch, s);
-        return rc;
+    EMB_CUDA_TRY(emb_malloc_async((void **)&scratch, up(a_acc) + 2 * up(a_v) + up(a_tn) + a_ent, s));
+    unsigned long long *vacc = (unsigned long long *)scratch;
+    uint32_t *vflag = (uint32_t *)(scratch + up(a_acc));
+    int *vexp = (int *)(scratch + up(a_acc) + up(a_v));
+    int *tile_n = (int *)(scratch + up(a_acc) + 2 * up(a_v));
+    QbEntry *ent = (QbEntry *)(scratch + up(a_acc) + 2 * up(a_v) + up(a_tn));
+    int qbits = 61;
+    while (((3 * n) >> (61 - qbits)) != 0) --qbits;
+    EMB_CUDA_TRY(cudaMemsetAsync(vacc, 0, up(a_acc) + a_v, s));
+    EMB_CUDA_TRY(cudaMemsetAsync(vexp, 0x80, a_v, s));
+    if (n > 0) {
+        EMB_LAUNCH((k_qbwd_tile), (int)nt, QB_BLOCK, 0, s)(lv.key, g, m->r_o, d_cell, d_dir, d_q, d_tri, d_gq, n, m->rec,
+                                                           m->T, ent, tile_n, vexp, vflag, st);
+        EMB_LAUNCH((k_qbwd_scatter), (int)nt, QB_BLOCK, 0, s)(ent, tile_n, m->rec, vexp, qbits, vacc);
     }
-    EMB_CUDA_TRY(cudaMemsetAsync(vcnt, 0, (m->V + 1) * sizeof(uint32_t), s));
-    if (n > 0) EMB_LAUNCH((k_qbwd_fill), emb_grid(3 * n, 256), 256, 0, s)(vid, 3 * n, voff, vcnt, slot);
-    // vid is spent after the fill and holds the sorted entries of each vertex
-    EMB_LAUNCH((k_qbwd_reduce), emb_grid(32 * m->V, 256), 256, 0, s)(voff, slot, (uint32_t *)vid, val, m->V, d_gverts);
+    EMB_LAUNCH((k_qbwd_write), emb_grid(m3, 256), 256, 0, s)(vexp, vflag, vacc, m3, qbits, d_gverts);
     EMB_CUDA_TRY(cudaGetLastError());
     EMB_CUDA_TRY(cudaFreeAsync(scratch, s));
     return EMB_OK;

@@ -1,13 +1,17 @@
-"""The force and dF/dq where their fast arithmetic ends: populations of any magnitude
-(zeros, infinities and NaN among them).  References in FP64."""
+"""The force, dF/dq and the vertex gradient where their fast arithmetic ends: populations
+and weights of any magnitude (zeros, infinities and NaN among them), a q that is not the
+link's crossing, thousands of links at one vertex, link counts around a tile, and the same
+bits from run to run.  References in FP64."""
 from __future__ import annotations
 
 import numpy as np
 import pytest
 
 from synth import workload
+from synth.meshes import octahedron
 
 pytestmark = pytest.mark.gpu
+G = 1 << 20
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -86,3 +90,91 @@ def test_force_not_finite(orc, body):
     F, gq = _call(E, torch.from_numpy(pop).cuda(), gF)
     np.testing.assert_allclose(gq, ref, rtol=1e-6, atol=1e-6)
     assert np.all(np.isnan(F))
+
+
+def _grad(E, gq, q=None, n=None):
+    import torch
+
+    import paper_2512_01251_gb300 as P
+    L = E.links
+    q = L["q"] if q is None else torch.from_numpy(q).cuda()
+    cut = [x[:n].contiguous() for x in (L["cell"], L["dir"], q, L["tri"], torch.from_numpy(gq).cuda())]
+    g = P.emb_cutlinks_backward(E.mesh, E.forest, *cut)
+    assert torch.equal(torch.nan_to_num(g), torch.nan_to_num(P.emb_cutlinks_backward(E.mesh, E.forest, *cut)))
+    assert P.emb_status_get() == P.EMB_OK
+    return g.cpu().numpy().astype(np.float64)
+
+
+def _ref(orc, lk, gq, o, t, R, levels, nv, n=None):
+    lk = {k: np.asarray(x)[:n] for k, x in lk.items() if k in ("cell", "dir", "q", "tri")}
+    gq = gq.astype(np.float64)[:n]
+    ref = orc.grad_verts_from_gq(lk, gq, o["X"], t, R, levels, o["blocks"][-1], nv)
+    # the size of the summed terms: one link at a time would be |gq| |dq/dV|
+    _, nrm, _, _, _, _, c, h = orc.dq_dverts(lk, o["X"], t, R, levels)
+    size = np.zeros((nv, 3))
+    b = np.abs(gq[:, None] * nrm / (h * np.einsum("ij,ij->i", nrm, c))[:, None])
+    for j in range(3):
+        np.add.at(size, t[lk["tri"], j], b)
+    return ref, size
+
+
+@pytest.mark.parametrize("spread", [0, 20, 60])
+def test_gradient_over_magnitudes(orc, body, spread):
+    w, v, t, E, o, partner = body
+    rng = np.random.default_rng(spread + 5)
+    n = len(o["links"]["q"])
+    gq = (rng.standard_normal(n) * np.exp2(rng.uniform(-spread, spread, n))).astype(np.float32)
+    gq[::7] = 0.0
+    ref, size = _ref(orc, o["links"], gq, o, t, w.R, w.levels, len(v))
+    g = _grad(E, gq)
+    assert np.all(np.abs(g - ref) <= 2.0 ** -23 * np.abs(ref) + 2.0 ** -22 * size)
+
+
+@pytest.mark.parametrize("n", [0, 1, 31, 256, 511, 512, 513, 1024, 1025])
+def test_gradient_link_counts(orc, body, n):
+    w, v, t, E, o, partner = body
+    gq = np.random.default_rng(n).standard_normal(len(o["links"]["q"])).astype(np.float32)
+    ref, size = _ref(orc, o["links"], gq, o, t, w.R, w.levels, len(v), n)
+    assert np.all(np.abs(_grad(E, gq, n=n) - ref) <= 2.0 ** -23 * np.abs(ref) + 2.0 ** -22 * size)
+
+
+def test_gradient_at_another_q(orc, body):
+    """A q that is not the link's crossing moves the hit point along the link."""
+    w, v, t, E, o, partner = body
+    rng = np.random.default_rng(9)
+    n = len(o["links"]["q"])
+    gq = rng.standard_normal(n).astype(np.float32)
+    q = rng.uniform(0.0, 1.0, n).astype(np.float32)
+    ref, size = _ref(orc, dict(o["links"], q=q.astype(np.float64)), gq, o, t, w.R, w.levels, len(v))
+    # barycentric weights reach the link's length over the triangle's height here
+    assert np.all(np.abs(_grad(E, gq, q=q) - ref) <= 1e-5 * (np.abs(ref) + size))
+
+
+def test_gradient_not_finite(orc, body):
+    w, v, t, E, o, partner = body
+    n = len(o["links"]["q"])
+    gq = np.zeros(n, dtype=np.float32)
+    k = np.random.default_rng(3).integers(0, n, 3)
+    gq[k] = [np.nan, np.inf, -np.inf]
+    g = _grad(E, gq)
+    touched = np.zeros(len(v), dtype=bool)
+    touched[t[o["links"]["tri"][k]].reshape(-1)] = True
+    assert not np.any(np.isfinite(g[touched])) and np.all(g[~touched] == 0.0)
+
+
+def test_gradient_many_links_per_vertex(orc):
+    """Eight faces on a fine grid: every vertex takes a third of the terms of four faces."""
+    import torch
+
+    import paper_2512_01251_gb300 as P
+    v, t = octahedron([G // 2 + 3, G // 2 - 5, G // 2 + 1], [G // 4 + 11, G // 5, G // 3 - 7])
+    v, t = np.asarray(v, dtype=np.float32), np.asarray(t, dtype=np.int32)
+    E = P.embed(torch.from_numpy(v), torch.from_numpy(t), 4, 3, 2, 27)
+    o = orc.embed_lines(v, t, 4, 3, 2, 27)
+    n = len(o["links"]["q"])
+    assert n > 20000
+    gq = np.random.default_rng(8).standard_normal(n).astype(np.float32)
+    ref, size = _ref(orc, o["links"], gq, o, t, 4, 3, len(v))
+    g = _grad(E, gq)
+    # each term's own error is FP32-sized; independent, they add up to far less than this
+    assert np.all(np.abs(g - ref) <= 2.0 ** -23 * np.abs(ref) + 2.0 ** -24 * size)
