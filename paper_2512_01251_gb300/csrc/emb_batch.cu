@@ -44,11 +44,12 @@ struct BMesh {
     emb_forest_s geo;                // frame and level geometry (no buffers)
     BLevel L[EMB_MAX_LEVELS];
     // scratch sized for the largest level / the triangle count
-    uint32_t *flag = nullptr, *pos = nullptr;       // T + 1
+    uint32_t *nf = nullptr;                         // filtered triangles of the level
+    uint32_t *fword = nullptr;                      // filter words
+    uint64_t *fstate = nullptr;                     // scan state of the filter
     unsigned long long *s_acc = nullptr;            // max blocks
     unsigned int *p_acc = nullptr, *t_acc = nullptr;
     uint32_t *cnt = nullptr, *rank = nullptr;       // max blocks + 1
-    uint32_t *pc = nullptr;                         // max bitmap words + 1
     uint64_t *tmp = nullptr;                        // scan scratch
     // finest level
     uint32_t *bin_off = nullptr, *bin_ent = nullptr;
@@ -213,14 +214,14 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     BTRY(balloc(B, &B.fbits, fw));
     EmbLevel &fin = B.L[B.Lf].lv;
     BTRY(balloc(B, &fin.nbr, fin.n * 26 + 1));
-    BTRY(balloc(B, &B.flag, T + 1));
-    BTRY(balloc(B, &B.pos, T + 1));
+    BTRY(balloc(B, &B.nf, 1));
+    BTRY(balloc(B, &B.fword, (size_t)(T + 31) / 32));
+    BTRY(balloc(B, &B.fstate, (size_t)emb_filter_state_words(T)));
     BTRY(balloc(B, &B.s_acc, nmax));
     BTRY(balloc(B, &B.p_acc, nmax));
     BTRY(balloc(B, &B.t_acc, nmax));
     BTRY(balloc(B, &B.cnt, nmax + 1));
     BTRY(balloc(B, &B.rank, nmax + 1));
-    BTRY(balloc(B, &B.pc, wmax + 1));
     const int64_t sw = emb_scan_tmp_words(T > nmax ? (T > wmax ? T : wmax) : (nmax > wmax ? nmax : wmax));
     BTRY(balloc(B, &B.tmp, sw));
     BTRY(balloc(B, &B.bin_off, fin.n + 1));
@@ -246,16 +247,6 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     return EMB_OK;
 }
 
-// d_n = 8 x the flagged count of the parent level, capped at the level's capacity
-// (EMB_ERR_CAPACITY when the flagged blocks need more).
-__global__ void k_level_count(const uint32_t *__restrict__ nflags, int64_t cap, uint32_t *__restrict__ d_n, int *st)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const uint64_t n = 8ull * *nflags;
-    if (n > (uint64_t)cap) emb_set_status(st, EMB_ERR_CAPACITY);
-    *d_n = (uint32_t)(n < (uint64_t)cap ? n : (uint64_t)cap);
-}
-
 // EMB_ERR_CAPACITY when the pair list asked for more entries than it holds.
 __global__ void k_list_check(const unsigned long long *__restrict__ list_n, uint64_t cap, int *st)
 {
@@ -270,24 +261,22 @@ static emb_status enqueue_mesh(BMesh &B, int tri_block, cudaStream_t s)
     const bool hr = B.d_n != nullptr;  // headroom: counts up to capacity, read on the device
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
-    BTRY(emb_enq_root_keys(B.R, B.L[0].lv.key, s));
-    BTRY(emb_enq_level_index(B.L[0].lv, B.pc, B.tmp, s));
+    BTRY(emb_enq_root(B.L[0].lv, s));
     for (int L = 0; L <= B.Lf; ++L) {
         BLevel &BL = B.L[L];
         EmbLevel &lv = BL.lv;
         const LevelGeom g = level_geom(&B.geo, L);
-        BTRY(emb_enq_filter(rec, T, g, B.flag, B.pos, BL.flist, B.tmp, tri_block, s, hr ? EMB_NO_EXPECT : (uint64_t)BL.nf));
-        BTRY(emb_enq_voxelize(rec, T, BL.flist, hr ? T : BL.nf, B.pos + T, nullptr, g, lv, B.s_acc, B.p_acc, B.t_acc, B.bq,
+        BTRY(emb_enq_filter(rec, T, g, BL.flist, B.nf, B.fword, B.fstate, false, tri_block, s,
+                            hr ? EMB_NO_EXPECT : (uint64_t)BL.nf));
+        BTRY(emb_enq_voxelize(rec, T, BL.flist, hr ? T : BL.nf, B.nf, nullptr, g, lv, B.s_acc, B.p_acc, B.t_acc, B.bq,
                               tri_block, s));
         if (L < B.Lf) {
             const long long dil = emb_refine_dilation(&B.geo, L, B.band);
             if (dil < 0) return EMB_ERR_RANGE;
             BTRY(emb_enq_refine(rec, T, g, dil, lv, BL.flags, B.fbits, B.bq, s));
-            BTRY(emb_enq_flag_ranks(lv, BL.flags, B.cnt, B.rank, B.tmp, s, hr ? EMB_NO_EXPECT : (uint64_t)BL.F));
+            BTRY(emb_enq_flag_ranks(lv, BL.flags, B.rank, B.tmp, false, s, hr ? EMB_NO_EXPECT : (uint64_t)BL.F));
             EmbLevel &C = B.L[L + 1].lv;
-            if (hr) EMB_LAUNCH((k_level_count), 1, 32, 0, s)(B.rank + lv.n, C.n, B.d_n + L + 1, st);
-            BTRY(emb_enq_children(lv, BL.flags, B.rank, C.key, C.n, true, s));
-            BTRY(emb_enq_level_index(C, B.pc, B.tmp, s));
+            BTRY(emb_enq_child_level(lv, BL.flags, B.rank, C, C.n, true, hr ? B.d_n + L + 1 : nullptr, B.tmp, false, s));
         } else {
             BTRY(emb_enq_bin_pairs(rec, T, g, lv, B.cnt, B.bin_off, B.list_bs, B.list_tri, B.list_n, (uint64_t)B.pairs,
                                    B.tmp, B.bq, s, hr ? EMB_NO_EXPECT : (uint64_t)B.pairs));

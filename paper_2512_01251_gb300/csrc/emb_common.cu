@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "emb_internal.cuh"
+#include "emb_scan.cuh"
 
 // ---------------------------------------------------------------------------
 // status word and error notes
@@ -127,150 +128,134 @@ extern "C" emb_status emb_directions(int32_t *h_out)
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of uint32 values (three phases: tile sums, scan of sums, apply)
+// exclusive scan of uint32 values (one launch)
 // ---------------------------------------------------------------------------
 #define SCAN_BLOCK 512
 #define SCAN_ITEMS 8
 #define SCAN_TILE (SCAN_BLOCK * SCAN_ITEMS)
 
-// Block-wide exclusive scan of one uint64 per thread; returns the block total in *total.
-__device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t *total)
+// What is summed: SCAN_ITEMS consecutive values from base (0 past n).
+struct ScanU32 {
+    const uint32_t *p;
+    __device__ __forceinline__ void load(int64_t base, int64_t n, uint32_t v[SCAN_ITEMS]) const
+    {
+        if (base + SCAN_ITEMS <= n && !((uintptr_t)p & 15)) {
+            const uint4 a = *(const uint4 *)(p + base), b = *(const uint4 *)(p + base + 4);
+            v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < n ? p[base + i] : 0u;
+    }
+};
+struct ScanFlags {  // bytes: 1 where not zero
+    const uint8_t *p;
+    __device__ __forceinline__ void load(int64_t base, int64_t n, uint32_t v[SCAN_ITEMS]) const
+    {
+        if (base + SCAN_ITEMS <= n && !((uintptr_t)p & 7)) {
+            const uint2 a = *(const uint2 *)(p + base);
+#pragma unroll
+            for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = ((i < 4 ? a.x : a.y) >> (8 * (i & 3))) & 255u ? 1u : 0u;
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < n && p[base + i] ? 1u : 0u;
+    }
+};
+struct ScanPopc {  // set bits of 64-bit words
+    const uint64_t *p;
+    __device__ __forceinline__ void load(int64_t base, int64_t n, uint32_t v[SCAN_ITEMS]) const
+    {
+        if (base + SCAN_ITEMS <= n && !((uintptr_t)p & 15)) {
+#pragma unroll
+            for (int i = 0; i < SCAN_ITEMS; i += 2) {
+                const ulonglong2 a = *(const ulonglong2 *)(p + base + i);
+                v[i] = (uint32_t)__popcll(a.x);
+                v[i + 1] = (uint32_t)__popcll(a.y);
+            }
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) v[i] = base + i < n ? (uint32_t)__popcll(p[base + i]) : 0u;
+    }
+};
+
+// out[0, n]: exclusive sums and, at n, the total (also in *total when given), which is
+// checked against `expect` unless that is EMB_NO_EXPECT.  state: NULL for a single tile.
+// Latency-bound up to about a million values: 2 launches a scan were 2 + 5 us.
+template <class In>
+__global__ void __launch_bounds__(SCAN_BLOCK) k_scan(In in, int64_t n, uint32_t *__restrict__ out,
+                                                     uint64_t *__restrict__ state, uint64_t expect,
+                                                     uint32_t *__restrict__ total, int *st)
 {
-    __shared__ uint64_t warp_sums[SCAN_BLOCK / 32];
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint64_t inc = v;
+    __shared__ uint32_t s_tile;
+    __shared__ uint64_t s_warp[SCAN_BLOCK / 32 + 1];  // exclusive sums of the warps; last: the tiles before
+    const uint32_t tile = state ? scan_ticket(state, &s_tile) : 0u;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = (int64_t)tile * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
+    uint32_t v[SCAN_ITEMS];
+    in.load(base, n, v);
+    uint64_t own = 0;
+#pragma unroll
+    for (int i = 0; i < SCAN_ITEMS; ++i) own += v[i];
+    uint64_t incl = own;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        uint64_t t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
+        const uint64_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
-    if (lane == 31) warp_sums[w] = inc;
+    if (lane == 31) s_warp[w] = incl;
     __syncthreads();
     if (w == 0) {
-        uint64_t s = lane < SCAN_BLOCK / 32 ? warp_sums[lane] : 0;
-        uint64_t si = s;
+        const uint64_t x = lane < SCAN_BLOCK / 32 ? s_warp[lane] : 0;
+        uint64_t xi = x;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            uint64_t t = __shfl_up_sync(0xffffffffu, si, o);
-            if (lane >= o) si += t;
+            const uint64_t t = __shfl_up_sync(0xffffffffu, xi, o);
+            if (lane >= o) xi += t;
         }
-        if (lane < SCAN_BLOCK / 32) warp_sums[lane] = si - s;  // exclusive warp offsets
-        if (lane == SCAN_BLOCK / 32 - 1) *total = si;
+        const uint64_t sum = __shfl_sync(0xffffffffu, xi, 31);
+        const uint64_t before = state ? scan_lookback(state, tile, sum, st) : 0;
+        if (lane < SCAN_BLOCK / 32) s_warp[lane] = xi - x;
+        if (lane == 0) s_warp[SCAN_BLOCK / 32] = before;
     }
     __syncthreads();
-    uint64_t r = warp_sums[w] + inc - v;
-    __syncthreads();
-    return r;
-}
-
-__global__ void k_scan_tile_sums(const uint32_t *__restrict__ in, int64_t n, uint64_t *__restrict__ tile_sum)
-{
-    __shared__ uint64_t tot;
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    uint64_t s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i)
-        if (base + i < n) s += in[base + i];
-    block_excl_scan(s, &tot);
-    if (threadIdx.x == 0) tile_sum[blockIdx.x] = tot;
-}
-
-__global__ void k_scan_sums(uint64_t *__restrict__ tile_sum, int64_t ntiles, uint64_t *__restrict__ total)
-{
-    __shared__ uint64_t tot;
-    uint64_t carry = 0;
-    for (int64_t b = 0; b < ntiles; b += SCAN_BLOCK) {
-        int64_t i = b + threadIdx.x;
-        uint64_t v = i < ntiles ? tile_sum[i] : 0;
-        uint64_t ex = block_excl_scan(v, &tot);
-        if (i < ntiles) tile_sum[i] = carry + ex;
-        carry += tot;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) *total = carry;
-}
-
-// Writes the tile's exclusive sums from its offset `run`; entry n receives the total,
-// which is checked against `expect` unless that is EMB_NO_EXPECT.
-__device__ __forceinline__ void scan_write_tile(const uint32_t v[SCAN_ITEMS], int64_t base, int64_t n, uint64_t run,
-                                                uint32_t *__restrict__ out, uint64_t expect, int *st)
-{
+    uint64_t run = s_warp[SCAN_BLOCK / 32] + s_warp[w] + incl - own;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         if (base + i <= n) {  // entry n receives the total
             if (run > 0xFFFFFFFFull) emb_set_status(st, EMB_ERR_CAPACITY);
             out[base + i] = (uint32_t)run;
-            if (base + i == n && expect != EMB_NO_EXPECT && run != expect) emb_set_status(st, EMB_ERR_STATE);
+            if (base + i == n) {
+                if (expect != EMB_NO_EXPECT && run != expect) emb_set_status(st, EMB_ERR_STATE);
+                if (total) *total = (uint32_t)run;
+            }
         }
         run += v[i];
     }
 }
 
-__global__ void k_scan_apply(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int64_t n,
-                             const uint64_t *__restrict__ tile_off, uint64_t expect, int *st)
-{
-    __shared__ uint64_t tot;
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    uint32_t v[SCAN_ITEMS];
-    uint64_t s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        v[i] = base + i < n ? in[base + i] : 0u;
-        s += v[i];
-    }
-    const uint64_t run = tile_off[blockIdx.x] + block_excl_scan(s, &tot);
-    scan_write_tile(v, base, n, run, out, expect, st);
-}
+int64_t emb_scan_tmp_words(int64_t n) { return scan_state_words((n + SCAN_TILE) / SCAN_TILE); }
 
-// Apply with the scan of the tile sums folded in: each tile adds up the sums of the
-// tiles before it (few enough to read them all), and the last tile stores the total
-// after the sums.  With one tile it is the whole scan in one launch.
-__global__ void k_scan_apply_fused(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, int64_t n,
-                                   uint64_t *__restrict__ tile_sum, int64_t ntiles, uint64_t expect, int *st)
-{
-    __shared__ uint64_t tot, before;
-    uint64_t part = 0;
-    for (int64_t i = threadIdx.x; i < (int64_t)blockIdx.x; i += SCAN_BLOCK) part += tile_sum[i];
-    block_excl_scan(part, &before);
-    const uint64_t off = before;
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
-    uint32_t v[SCAN_ITEMS];
-    uint64_t s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        v[i] = base + i < n ? in[base + i] : 0u;
-        s += v[i];
-    }
-    const uint64_t run = off + block_excl_scan(s, &tot);
-    if (threadIdx.x == 0 && (int64_t)blockIdx.x == ntiles - 1) tile_sum[ntiles] = off + tot;
-    scan_write_tile(v, base, n, run, out, expect, st);
-}
-
-int64_t emb_scan_tmp_words(int64_t n) { return (n + 1 + SCAN_TILE - 1) / SCAN_TILE + 1; }
-
-// Above this many tiles the tile sums get a scan of their own.
-#define SCAN_FUSE_TILES 1024
-
-// d_out gets n + 1 entries: exclusive prefix sums and, at index n, the total (also in
-// tmp[ntiles]); a total other than `expect` raises EMB_ERR_STATE on the device.
-// tmp: emb_scan_tmp_words(n) uint64 words of scratch.  Enqueues only: one launch up
-// to SCAN_TILE entries, two up to SCAN_FUSE_TILES tiles, three beyond.
-emb_status emb_scan_into_expect(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
-                                cudaStream_t s)
+// tmp: emb_scan_tmp_words(n) uint64 words of scratch, zeroed here unless the caller has
+// (`zeroed`: one memset can then serve several scans); one tile needs none.
+template <class In>
+static emb_status enq_scan(In in, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect, uint32_t *d_total,
+                           bool zeroed, cudaStream_t s)
 {
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
-    int64_t ntiles = (n + 1 + SCAN_TILE - 1) / SCAN_TILE;
-    if (ntiles <= SCAN_FUSE_TILES) {
-        if (ntiles > 1) EMB_LAUNCH((k_scan_tile_sums), (int)ntiles, SCAN_BLOCK, 0, s)(d_in, n, tmp);
-        EMB_LAUNCH((k_scan_apply_fused), (int)ntiles, SCAN_BLOCK, 0, s)(d_in, d_out, n, tmp, ntiles, expect, st);
-    } else {
-        EMB_LAUNCH((k_scan_tile_sums), (int)ntiles, SCAN_BLOCK, 0, s)(d_in, n, tmp);
-        EMB_LAUNCH((k_scan_sums), 1, SCAN_BLOCK, 0, s)(tmp, ntiles, tmp + ntiles);
-        EMB_LAUNCH((k_scan_apply), (int)ntiles, SCAN_BLOCK, 0, s)(d_in, d_out, n, tmp, expect, st);
-    }
+    const int64_t ntiles = (n + SCAN_TILE) / SCAN_TILE;
+    if (ntiles > 1 && !zeroed) EMB_CUDA_TRY(cudaMemsetAsync(tmp, 0, scan_state_words(ntiles) * sizeof(uint64_t), s));
+    EMB_LAUNCH((k_scan<In>), (int)ntiles, SCAN_BLOCK, 0, s)(in, n, d_out, ntiles > 1 ? tmp : nullptr, expect, d_total, st);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
+}
+
+emb_status emb_scan_into_expect(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
+                                cudaStream_t s, uint32_t *d_total, bool zeroed)
+{
+    return enq_scan(ScanU32{d_in}, d_out, n, tmp, expect, d_total, zeroed, s);
 }
 
 emb_status emb_scan_into(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, cudaStream_t s)
@@ -278,19 +263,15 @@ emb_status emb_scan_into(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint6
     return emb_scan_into_expect(d_in, d_out, n, tmp, EMB_NO_EXPECT, s);
 }
 
-emb_status emb_scan_u32(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *h_total, cudaStream_t s)
+emb_status emb_scan_flags(const uint8_t *d_flags, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
+                          bool zeroed, cudaStream_t s)
 {
-    uint64_t *tmp = nullptr;
-    int64_t ntiles = (n + 1 + SCAN_TILE - 1) / SCAN_TILE;
-    EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(n) * sizeof(uint64_t), s));
-    emb_status rc = emb_scan_into(d_in, d_out, n, tmp, s);
-    if (rc != EMB_OK) return rc;
-    if (h_total) {
-        EMB_CUDA_TRY(cudaMemcpyAsync(h_total, tmp + ntiles, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-        EMB_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-    EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
-    return EMB_OK;
+    return enq_scan(ScanFlags{d_flags}, d_out, n, tmp, expect, nullptr, zeroed, s);
+}
+
+emb_status emb_scan_popc(const uint64_t *d_words, uint32_t *d_out, int64_t n, uint64_t *tmp, bool zeroed, cudaStream_t s)
+{
+    return enq_scan(ScanPopc{d_words}, d_out, n, tmp, EMB_NO_EXPECT, nullptr, zeroed, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -328,28 +309,6 @@ __global__ void k_bits_set(const uint64_t *__restrict__ key, int64_t n, int64_t 
     atomicOr(bits + (lin >> 6), 1ull << (lin & 63));
 }
 
-// The bits of a child level whose block count, 8 x *nflags (at most cap), is still on
-// the device: threads past the count leave the bitmap alone.
-__global__ void k_bits_set_counted(const uint64_t *__restrict__ key, const uint32_t *__restrict__ nflags, int64_t cap,
-                                   int64_t nb, unsigned long long *__restrict__ bits)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t n = 8 * (int64_t)*nflags;
-    if (i >= n || i >= cap) return;
-    uint64_t k = key[i];
-    int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
-            bz = (int64_t)(k >> (2 * EMB_KEY_BITS));
-    if (bx >= nb || by >= nb || bz >= nb) return;
-    int64_t lin = (bz * nb + by) * nb + bx;
-    atomicOr(bits + (lin >> 6), 1ull << (lin & 63));
-}
-
-__global__ void k_word_popc(const uint64_t *__restrict__ bits, int64_t nw, uint32_t *__restrict__ out)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nw) out[i] = (uint32_t)__popcll(bits[i]);
-}
-
 int64_t emb_hash_capacity(int64_t n)
 {
     int64_t cap = 1024;
@@ -365,8 +324,8 @@ int64_t emb_bitmap_words(int64_t nb)
 
 // Rank bitmap of a level whose keys are in place or, where the level's dense positions
 // exceed EMB_BITMAP_MAX_BITS, its hash (lookups use whichever exists); buffers sized by
-// emb_bitmap_words / emb_hash_capacity; pc: words + 1 uint32, tmp: scan scratch.
-emb_status emb_enq_level_index(EmbLevel &lv, uint32_t *pc, uint64_t *tmp, cudaStream_t s)
+// emb_bitmap_words / emb_hash_capacity; tmp: scan scratch.
+emb_status emb_enq_level_index(EmbLevel &lv, uint64_t *tmp, cudaStream_t s)
 {
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
@@ -380,43 +339,9 @@ emb_status emb_enq_level_index(EmbLevel &lv, uint32_t *pc, uint64_t *tmp, cudaSt
         if (lv.n > 0)
             EMB_LAUNCH((k_bits_set), emb_grid(lv.n, 256), 256, 0, s)(lv.key, lv.n, lv.nb_axis, (unsigned long long *)lv.bits,
                                                                      lv.d_n);
-        EMB_LAUNCH((k_word_popc), emb_grid(nw, 256), 256, 0, s)(lv.bits, nw, pc);
-        emb_status rc = emb_scan_into(pc, lv.wpre, nw, tmp, s);
+        emb_status rc = emb_scan_popc(lv.bits, lv.wpre, nw, tmp, false, s);
         if (rc != EMB_OK) return rc;
     }
-    EMB_CUDA_TRY(cudaGetLastError());
-    return EMB_OK;
-}
-
-// The rank bitmap of level lv (which must have one) from keys whose count, 8 x *nflags
-// with at most cap keys, is read on the device: lets the host read the count back while
-// the index is being built.
-emb_status emb_build_index_counted(EmbLevel &lv, const uint32_t *nflags, int64_t cap, cudaStream_t s)
-{
-    const int64_t nw = emb_bitmap_words(lv.nb_axis);
-    if (nw == 0) return EMB_ERR_STATE;
-    if (lv.hkey) EMB_CUDA_TRY(cudaFreeAsync(lv.hkey, s));
-    if (lv.hval) EMB_CUDA_TRY(cudaFreeAsync(lv.hval, s));
-    if (lv.bits) EMB_CUDA_TRY(cudaFreeAsync(lv.bits, s));
-    if (lv.wpre) EMB_CUDA_TRY(cudaFreeAsync(lv.wpre, s));
-    lv.hkey = nullptr;
-    lv.hval = nullptr;
-    lv.hcap = 0;
-    uint32_t *pc = nullptr;
-    uint64_t *tmp = nullptr;
-    EMB_CUDA_TRY(emb_malloc_async(&lv.bits, nw * sizeof(uint64_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&lv.wpre, (nw + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&pc, (nw + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(nw) * sizeof(uint64_t), s));
-    EMB_CUDA_TRY(cudaMemsetAsync(lv.bits, 0, nw * sizeof(uint64_t), s));
-    if (cap > 0)
-        EMB_LAUNCH((k_bits_set_counted), emb_grid(cap, 256), 256, 0, s)(lv.key, nflags, cap, lv.nb_axis,
-                                                                           (unsigned long long *)lv.bits);
-    EMB_LAUNCH((k_word_popc), emb_grid(nw, 256), 256, 0, s)(lv.bits, nw, pc);
-    emb_status rc = emb_scan_into(pc, lv.wpre, nw, tmp, s);
-    EMB_CUDA_TRY(cudaFreeAsync(pc, s));
-    EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
-    if (rc != EMB_OK) return rc;
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
@@ -522,16 +447,13 @@ emb_status emb_build_hash(EmbLevel &lv, cudaStream_t s)
         EMB_CUDA_TRY(emb_malloc_async(&lv.hkey, lv.hcap * sizeof(uint64_t), s));
         EMB_CUDA_TRY(emb_malloc_async(&lv.hval, lv.hcap * sizeof(int32_t), s));
     }
-    uint32_t *pc = nullptr;
     uint64_t *tmp = nullptr;
     if (nw > 0) {
         EMB_CUDA_TRY(emb_malloc_async(&lv.bits, nw * sizeof(uint64_t), s));
         EMB_CUDA_TRY(emb_malloc_async(&lv.wpre, (nw + 1) * sizeof(uint32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&pc, (nw + 1) * sizeof(uint32_t), s));
         EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(nw) * sizeof(uint64_t), s));
     }
-    emb_status rc = emb_enq_level_index(lv, pc, tmp, s);
-    if (pc) EMB_CUDA_TRY(cudaFreeAsync(pc, s));
+    emb_status rc = emb_enq_level_index(lv, tmp, s);
     if (tmp) EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
     return rc;
 }

@@ -10,40 +10,92 @@
 
 #include "emb_internal.cuh"
 
-__global__ void k_root_keys(int64_t R, uint64_t *__restrict__ key)
+// The root level in one launch: every position holds a block, so the bitmap is full and
+// the prefix of word w is 64 w.
+__global__ void k_root(int64_t R, uint64_t *__restrict__ key, uint64_t *__restrict__ bits, uint32_t *__restrict__ wpre,
+                       int64_t nw)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= R * R * R) return;
-    key[i] = emb_key(i % R, (i / R) % R, i / (R * R));
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = R * R * R;
+    if (i < n) key[i] = emb_key(i % R, (i / R) % R, i / (R * R));
+    if (i < nw) bits[i] = n - 64 * i >= 64 ? ~0ull : (1ull << (n - 64 * i)) - 1ull;
+    if (i <= nw) wpre[i] = (uint32_t)(64 * i < n ? 64 * i : n);
 }
 
-__global__ void k_flags_u32(const uint8_t *__restrict__ f, int64_t n, uint32_t *__restrict__ out)
+// Blocks of a level at dense positions below lin (at most nb^3).
+__device__ __forceinline__ int64_t rank_below(const uint64_t *__restrict__ bits, const uint32_t *__restrict__ wpre,
+                                              int64_t lin)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = f[i] ? 1u : 0u;
+    const int sh = (int)(lin & 63);
+    const int64_t r = wpre[lin >> 6];
+    return sh ? r + __popcll(bits[lin >> 6] & ((1ull << sh) - 1ull)) : r;
 }
 
+// Keys past the count in a planned replay that flagged fewer blocks than its buffers hold
+// (a replay with headroom, or one whose counts left its plan): a key above every real
+// key, so that the level's keys stay sorted for the binary searches over all Cn of
+// them; its coordinates (2^21 - 1 on every axis) fail the range checks of the passes
+// that decode keys, and the passes over blocks stop at the device count where there
+// is one.
+#define EMB_KEY_TAIL 0x7FFFFFFFFFFFFFFFull
 
-__global__ void k_make_children(const uint64_t *__restrict__ key, int64_t n, const uint8_t *__restrict__ flags,
-                                const uint32_t *__restrict__ rank, uint64_t *__restrict__ ckey, int64_t Cn)
+// The children of the flagged blocks, in order, and their bits in the child level's bitmap
+// (cbits, zeroed before; NULL for a level with a hash).  The parents before a block's row
+// and plane are counted with the parent's rank bitmap (two loads each) where it has one,
+// else by binary search.  A planned replay also fills the keys past the count and stores
+// the level's block count at d_n.  (With the bits, the tail and the count in launches of
+// their own and the binary searches always: 12 us a level instead of 5.)
+__global__ void k_make_children(const EmbLevel P, const uint8_t *__restrict__ flags, const uint32_t *__restrict__ rank,
+                                uint64_t *__restrict__ ckey, int64_t Cn, unsigned long long *__restrict__ cbits,
+                                bool planned, uint32_t *__restrict__ d_n, int *st)
 {
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t *__restrict__ key = P.key;
+    const int64_t n = P.n, nb = P.nb_axis;
+    if (planned) {
+        const int64_t m = 8 * (int64_t)rank[n];
+        for (int64_t i = m + p; i < Cn; i += (int64_t)gridDim.x * blockDim.x) ckey[i] = EMB_KEY_TAIL;
+        if (p == 0 && d_n) {
+            if (m > Cn) emb_set_status(st, EMB_ERR_CAPACITY);
+            *d_n = (uint32_t)(m < Cn ? m : Cn);
+        }
+    }
     if (p >= n || !flags[p]) return;
-    uint64_t k = key[p];
-    int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
-            bz = (int64_t)(k >> (2 * EMB_KEY_BITS));
-    uint64_t row0 = k & ~EMB_KEY_MASK, row1 = row0 + (1ull << EMB_KEY_BITS);
-    uint64_t pl0 = k & ~((1ull << (2 * EMB_KEY_BITS)) - 1ull), pl1 = pl0 + (1ull << (2 * EMB_KEY_BITS));
-    int64_t rl = lower_bound_u64(key, n, row0), rh = lower_bound_u64(key, n, row1);
-    int64_t pll = lower_bound_u64(key, n, pl0), plh = lower_bound_u64(key, n, pl1);
-    int64_t r_p = rank[p], r_row = rank[rl], F_row = (int64_t)rank[rh] - r_row;
-    int64_t r_pl = rank[pll], F_pl = (int64_t)rank[plh] - r_pl;
+    const uint64_t k = key[p];
+    const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
+                  bz = (int64_t)(k >> (2 * EMB_KEY_BITS));
+    int64_t rl, rh, pll, plh;
+    if (P.bits) {
+        if (bx >= nb || by >= nb || bz >= nb) return;  // only a replay whose counts left its plan gets here
+        const int64_t row = (bz * nb + by) * nb, plane = bz * nb * nb;
+        rl = rank_below(P.bits, P.wpre, row);
+        rh = rank_below(P.bits, P.wpre, row + nb);
+        pll = rank_below(P.bits, P.wpre, plane);
+        plh = rank_below(P.bits, P.wpre, plane + nb * nb);
+    } else {
+        const uint64_t row0 = k & ~EMB_KEY_MASK, row1 = row0 + (1ull << EMB_KEY_BITS);
+        const uint64_t pl0 = k & ~((1ull << (2 * EMB_KEY_BITS)) - 1ull), pl1 = pl0 + (1ull << (2 * EMB_KEY_BITS));
+        rl = lower_bound_u64(key, n, row0);
+        rh = lower_bound_u64(key, n, row1);
+        pll = lower_bound_u64(key, n, pl0);
+        plh = lower_bound_u64(key, n, pl1);
+    }
+    const int64_t r_p = rank[p], r_row = rank[rl], F_row = (int64_t)rank[rh] - r_row;
+    const int64_t r_pl = rank[pll], F_pl = (int64_t)rank[plh] - r_pl;
     for (int dz = 0; dz < 2; ++dz)
-        for (int dy = 0; dy < 2; ++dy)
-            for (int dx = 0; dx < 2; ++dx) {
-                int64_t pos = 8 * r_pl + dz * 4 * F_pl + 4 * (r_row - r_pl) + dy * 2 * F_row + 2 * (r_p - r_row) + dx;
-                if (pos >= 0 && pos < Cn) ckey[pos] = emb_key(2 * bx + dx, 2 * by + dy, 2 * bz + dz);
+        for (int dy = 0; dy < 2; ++dy) {
+            const int64_t pos = 8 * r_pl + dz * 4 * F_pl + 4 * (r_row - r_pl) + dy * 2 * F_row + 2 * (r_p - r_row);
+            const int64_t cy = 2 * by + dy, cz = 2 * bz + dz;
+            unsigned long long pair = 0;  // the two children along x: neighbours in a word, 2 bx is even
+            for (int dx = 0; dx < 2; ++dx)
+                if (pos + dx >= 0 && pos + dx < Cn) {
+                    ckey[pos + dx] = emb_key(2 * bx + dx, cy, cz);
+                    pair |= 1ull << dx;
+                }
+            if (cbits && pair) {
+                const int64_t lin = (cz * (2 * nb) + cy) * (2 * nb) + 2 * bx;
+                atomicOr(cbits + (lin >> 6), pair << (lin & 63));
             }
+        }
 }
 
 __global__ void k_unpack_keys(const uint64_t *__restrict__ key, int64_t n, int32_t *__restrict__ out)
@@ -91,12 +143,14 @@ extern "C" emb_status emb_forest_root(int32_t R, int32_t max_level, void *stream
     EmbLevel &lv = f->lv[0];
     lv.n = (int64_t)R * R * R;
     lv.nb_axis = R;
-    if (emb_malloc_async(&lv.key, lv.n * sizeof(uint64_t), s) != cudaSuccess) {
+    const int64_t nw = emb_bitmap_words(R);
+    if (emb_malloc_async(&lv.key, lv.n * sizeof(uint64_t), s) != cudaSuccess ||
+        emb_malloc_async(&lv.bits, nw * sizeof(uint64_t), s) != cudaSuccess ||
+        emb_malloc_async(&lv.wpre, (nw + 1) * sizeof(uint32_t), s) != cudaSuccess) {
         emb_forest_destroy(f);
         return EMB_ERR_CUDA;
     }
-    emb_status rc = emb_enq_root_keys(R, lv.key, s);
-    if (rc == EMB_OK) rc = emb_build_hash(lv, s);
+    const emb_status rc = emb_enq_root(lv, s);
     if (rc != EMB_OK) {
         emb_forest_destroy(f);
         return rc;
@@ -122,41 +176,37 @@ extern "C" void emb_forest_destroy(emb_forest f)
 }
 
 // Refinement in two enqueue-only halves (buffers supplied by the caller):
-//  (1) ranks of the flagged blocks of P: cnt, rank hold P.n + 1 uint32; the number
-//      of flagged blocks F ends at rank[P.n]; tmp is scan scratch for P.n entries;
-//  (2) the 8 F children keys, written in (z, y, x) order into ckey.
-emb_status emb_enq_flag_ranks(const EmbLevel &P, const uint8_t *d_flags, uint32_t *cnt, uint32_t *rank, uint64_t *tmp,
+//  (1) ranks of the flagged blocks of P: rank holds P.n + 1 uint32; the number of
+//      flagged blocks F ends at rank[P.n]; tmp is scan scratch for P.n entries;
+//  (2) level C: its first min(8 F, Cn) keys in (z, y, x) order and its index (rank bitmap,
+//      or the hash over C.n keys where it has none); tmp is scan scratch for its bitmap.
+//      `zeroed`: the caller has cleared the bitmap and tmp.  planned: see k_make_children.
+emb_status emb_enq_flag_ranks(const EmbLevel &P, const uint8_t *d_flags, uint32_t *rank, uint64_t *tmp, bool zeroed,
                               cudaStream_t s, uint64_t expect)
 {
-    if (P.n > 0) EMB_LAUNCH((k_flags_u32), emb_grid(P.n, 256), 256, 0, s)(d_flags, P.n, cnt);
-    return emb_scan_into_expect(cnt, rank, P.n, tmp, expect, s);
+    return emb_scan_flags(d_flags, rank, P.n, tmp, expect, zeroed, s);
 }
 
-// Keys [8 F, Cn) of a planned replay that flagged fewer blocks than its buffers hold
-// (a replay with headroom, or one whose counts left its plan): a key above every real
-// key, so that the level's keys stay sorted for the binary searches over all Cn of
-// them; its coordinates (2^21 - 1 on every axis) fail the range checks of the passes
-// that decode keys, and the passes over blocks stop at the device count where there
-// is one.
-#define EMB_KEY_TAIL 0x7FFFFFFFFFFFFFFFull
-__global__ void k_key_tail(uint64_t *__restrict__ ckey, int64_t Cn, const uint32_t *__restrict__ nflags)
+emb_status emb_enq_child_level(const EmbLevel &P, const uint8_t *d_flags, const uint32_t *rank, EmbLevel &C, int64_t Cn,
+                               bool planned, uint32_t *d_n, uint64_t *tmp, bool zeroed, cudaStream_t s)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < Cn && i >= 8 * (int64_t)*nflags) ckey[i] = EMB_KEY_TAIL;
-}
-
-emb_status emb_enq_children(const EmbLevel &P, const uint8_t *d_flags, const uint32_t *rank, uint64_t *ckey, int64_t Cn,
-                            bool planned, cudaStream_t s)
-{
-    if (P.n > 0 && Cn > 0) EMB_LAUNCH((k_make_children), emb_grid(P.n, 256), 256, 0, s)(P.key, P.n, d_flags, rank, ckey, Cn);
-    if (planned && Cn > 0) EMB_LAUNCH((k_key_tail), emb_grid(Cn, 256), 256, 0, s)(ckey, Cn, rank + P.n);
+    int *st = emb_status_word();
+    if (!st) return EMB_ERR_CUDA;
+    const int64_t nw = C.bits ? emb_bitmap_words(C.nb_axis) : 0;
+    if (nw > 0 && !zeroed) EMB_CUDA_TRY(cudaMemsetAsync(C.bits, 0, nw * sizeof(uint64_t), s));
+    if (P.n > 0 && (Cn > 0 || d_n))
+        EMB_LAUNCH((k_make_children), emb_grid(P.n, 256), 256, 0, s)(P, d_flags, rank, C.key, Cn,
+                                                                     (unsigned long long *)(nw > 0 ? C.bits : nullptr),
+                                                                     planned, d_n, st);
     EMB_CUDA_TRY(cudaGetLastError());
-    return EMB_OK;
+    if (nw > 0) return emb_scan_popc(C.bits, C.wpre, nw, tmp, zeroed, s);
+    return emb_enq_level_index(C, tmp, s);
 }
 
-emb_status emb_enq_root_keys(int64_t R, uint64_t *key, cudaStream_t s)
+emb_status emb_enq_root(EmbLevel &lv, cudaStream_t s)
 {
-    EMB_LAUNCH((k_root_keys), emb_grid(R * R * R, 256), 256, 0, s)(R, key);
+    const int64_t R = lv.nb_axis, nw = emb_bitmap_words(R), n = R * R * R;
+    EMB_LAUNCH((k_root), emb_grid(n > nw + 1 ? n : nw + 1, 256), 256, 0, s)(R, lv.key, lv.bits, lv.wpre, nw);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
@@ -180,28 +230,28 @@ extern "C" emb_status emb_forest_refine(emb_forest f, int32_t level, const uint8
     EmbLevel &P = f->lv[level];
     EmbLevel &C = f->lv[level + 1];
     free_level(C);
-    uint32_t *cnt = nullptr, *rank = nullptr;
-    uint64_t *tmp = nullptr;
-    EMB_CUDA_TRY(emb_malloc_async(&cnt, (P.n + 1) * sizeof(uint32_t), s));
+    uint32_t *rank = nullptr;
     EMB_CUDA_TRY(emb_malloc_async(&rank, (P.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(P.n) * sizeof(uint64_t), s));
-    emb_status rc = emb_enq_flag_ranks(P, d_flags, cnt, rank, tmp, s);
-    if (rc != EMB_OK) return rc;
     C.nb_axis = P.nb_axis * 2;
+    const int64_t nw = emb_bitmap_words(C.nb_axis), sp = emb_scan_tmp_words(P.n);
+    emb_status rc = EMB_OK;
     if (f->rb_slot < 0) f->rb_slot = emb_readback_acquire(&f->rb_h, &f->rb_ev);
-    if (emb_bitmap_words(C.nb_axis) > 0 && f->rb_slot >= 0) {
+    if (nw > 0 && f->rb_slot >= 0) {
         // The child level takes the rank bitmap: its keys (room for 8 per parent) and
         // index are built from the flagged count on the device while that count comes
-        // back to the host, so the GPU is not left idle during the read-back.
+        // back to the host, so the GPU is not left idle during the read-back.  The two
+        // scans' states lie behind the bitmap, cleared with it.
+        const int64_t cap = 8 * P.n, zw = nw + sp + emb_scan_tmp_words(nw);
+        EMB_CUDA_TRY(emb_malloc_async(&C.bits, zw * sizeof(uint64_t), s));
+        EMB_CUDA_TRY(emb_malloc_async(&C.wpre, (nw + 1) * sizeof(uint32_t), s));
+        EMB_CUDA_TRY(emb_malloc_async(&C.key, (cap + 1) * sizeof(uint64_t), s));
+        EMB_CUDA_TRY(cudaMemsetAsync(C.bits, 0, zw * sizeof(uint64_t), s));
+        rc = emb_enq_flag_ranks(P, d_flags, rank, C.bits + nw, true, s);
+        if (rc != EMB_OK) return rc;
         EMB_CUDA_TRY(cudaMemcpyAsync(f->rb_h, rank + P.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         EMB_CUDA_TRY(cudaEventRecord(f->rb_ev, s));
-        const int64_t cap = 8 * P.n;
-        EMB_CUDA_TRY(emb_malloc_async(&C.key, (cap + 1) * sizeof(uint64_t), s));
-        rc = emb_enq_children(P, d_flags, rank, C.key, cap, false, s);
-        if (rc == EMB_OK) rc = emb_build_index_counted(C, rank + P.n, cap, s);
-        EMB_CUDA_TRY(cudaFreeAsync(cnt, s));
+        rc = emb_enq_child_level(P, d_flags, rank, C, cap, false, nullptr, C.bits + nw + sp, true, s);
         EMB_CUDA_TRY(cudaFreeAsync(rank, s));
-        EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
         if (rc != EMB_OK) return rc;
         // the count is stored when a call first needs it (emb_forest_settle): work that
         // does not need it, such as the next level's x-line filter, is queued first, so
@@ -209,17 +259,27 @@ extern "C" emb_status emb_forest_refine(emb_forest f, int32_t level, const uint8
         C.n = 0;
         f->n_pending = level + 1;
     } else {
+        uint64_t *tmp = nullptr;
+        const int64_t sc = nw > 0 ? emb_scan_tmp_words(nw) : 1;
+        EMB_CUDA_TRY(emb_malloc_async(&tmp, (sp > sc ? sp : sc) * sizeof(uint64_t), s));
+        rc = emb_enq_flag_ranks(P, d_flags, rank, tmp, false, s);
+        if (rc != EMB_OK) return rc;
         uint32_t F = 0;
         EMB_CUDA_TRY(cudaMemcpyAsync(&F, rank + P.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
         EMB_CUDA_TRY(cudaStreamSynchronize(s));
         C.n = 8 * (int64_t)F;
         EMB_CUDA_TRY(emb_malloc_async(&C.key, (C.n + 1) * sizeof(uint64_t), s));
-        rc = emb_enq_children(P, d_flags, rank, C.key, C.n, false, s);
-        if (rc != EMB_OK) return rc;
-        EMB_CUDA_TRY(cudaFreeAsync(cnt, s));
+        if (nw > 0) {
+            EMB_CUDA_TRY(emb_malloc_async(&C.bits, nw * sizeof(uint64_t), s));
+            EMB_CUDA_TRY(emb_malloc_async(&C.wpre, (nw + 1) * sizeof(uint32_t), s));
+        } else {
+            C.hcap = emb_hash_capacity(C.n);
+            EMB_CUDA_TRY(emb_malloc_async(&C.hkey, C.hcap * sizeof(uint64_t), s));
+            EMB_CUDA_TRY(emb_malloc_async(&C.hval, C.hcap * sizeof(int32_t), s));
+        }
+        rc = emb_enq_child_level(P, d_flags, rank, C, C.n, false, nullptr, tmp, false, s);
         EMB_CUDA_TRY(cudaFreeAsync(rank, s));
         EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
-        rc = emb_build_hash(C, s);
         if (rc != EMB_OK) return rc;
     }
     f->top = level + 1;

@@ -211,23 +211,24 @@ emb_status emb_forest_settle(emb_forest f);
         const emb_status rs_ = emb_forest_settle(f_);          \
         if (rs_ != EMB_OK) return rs_;                         \
     } while (0)
-// Scans: d_out gets n + 1 entries (exclusive sums, total at n).  emb_scan_u32
-// allocates its scratch and can read the total back (synchronising); emb_scan_into
-// only enqueues, with emb_scan_tmp_words(n) words of caller scratch.
-emb_status emb_scan_u32(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *h_total, cudaStream_t s);
-emb_status emb_scan_into(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, cudaStream_t s);
-// emb_scan_into that also checks the total against a planned count (EMB_ERR_STATE on the
-// device when they differ), for planned replays; EMB_NO_EXPECT skips the check.
+// Scans (enqueue only): d_out gets n + 1 entries (exclusive sums, total at n) of uint32
+// values, of bytes counted as 1 where not zero, or of the set bits of 64-bit words; tmp is
+// emb_scan_tmp_words(n) words of scratch, zeroed by the call unless `zeroed`.  A total other
+// than `expect` raises EMB_ERR_STATE on the device (planned replays); EMB_NO_EXPECT skips the
+// check.  d_total, when given, gets the total too.
 #define EMB_NO_EXPECT 0xFFFFFFFFFFFFFFFFull
-emb_status emb_scan_into_expect(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
-                                cudaStream_t s);
 int64_t emb_scan_tmp_words(int64_t n);
+emb_status emb_scan_into(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, cudaStream_t s);
+emb_status emb_scan_into_expect(const uint32_t *d_in, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
+                                cudaStream_t s, uint32_t *d_total = nullptr, bool zeroed = false);
+emb_status emb_scan_flags(const uint8_t *d_flags, uint32_t *d_out, int64_t n, uint64_t *tmp, uint64_t expect,
+                          bool zeroed, cudaStream_t s);
+emb_status emb_scan_popc(const uint64_t *d_words, uint32_t *d_out, int64_t n, uint64_t *tmp, bool zeroed, cudaStream_t s);
 // Level index (hash + rank bitmap) and neighbour table.
 int64_t emb_hash_capacity(int64_t n);
 int64_t emb_bitmap_words(int64_t nb);
-emb_status emb_enq_level_index(EmbLevel &lv, uint32_t *pc, uint64_t *tmp, cudaStream_t s);
+emb_status emb_enq_level_index(EmbLevel &lv, uint64_t *tmp, cudaStream_t s);
 emb_status emb_build_hash(EmbLevel &lv, cudaStream_t s);
-emb_status emb_build_index_counted(EmbLevel &lv, const uint32_t *nflags, int64_t cap, cudaStream_t s);
 // Device address of a caller output buffer (device memory, or page-locked host memory
 // through its mapping); EMB_ERR_BAD_INPUT for pageable memory.  NULL stays NULL.
 emb_status emb_device_view(void *p, void **dp);
@@ -239,15 +240,16 @@ emb_status emb_build_neighbors(EmbLevel &lv, cudaStream_t s);
 int emb_grid(int64_t n, int block);
 int emb_sm_count();
 // Forest steps (enqueue only; buffers supplied by the caller).
-emb_status emb_enq_root_keys(int64_t R, uint64_t *key, cudaStream_t s);
-emb_status emb_enq_flag_ranks(const EmbLevel &P, const uint8_t *d_flags, uint32_t *cnt, uint32_t *rank, uint64_t *tmp,
+emb_status emb_enq_root(EmbLevel &lv, cudaStream_t s);
+emb_status emb_enq_flag_ranks(const EmbLevel &P, const uint8_t *d_flags, uint32_t *rank, uint64_t *tmp, bool zeroed,
                               cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
-emb_status emb_enq_children(const EmbLevel &P, const uint8_t *d_flags, const uint32_t *rank, uint64_t *ckey, int64_t Cn,
-                            bool planned, cudaStream_t s);
+emb_status emb_enq_child_level(const EmbLevel &P, const uint8_t *d_flags, const uint32_t *rank, EmbLevel &C, int64_t Cn,
+                               bool planned, uint32_t *d_n, uint64_t *tmp, bool zeroed, cudaStream_t s);
 // Binning, voxelization and refine flags (enqueue only).
 struct LevelGeom;
-emb_status emb_enq_filter(const int4 *rec, int64_t T, LevelGeom g, uint32_t *flag, uint32_t *pos, uint32_t *flist,
-                          uint64_t *tmp, int block, cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
+int64_t emb_filter_state_words(int64_t T);
+emb_status emb_enq_filter(const int4 *rec, int64_t T, LevelGeom g, uint32_t *flist, uint32_t *count, uint32_t *word,
+                          uint64_t *state, bool zeroed, int block, cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
 struct EmbBigQ;
 emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbLevel &lv, uint32_t *cnt, uint32_t *off,
                              uint2 *list_bs, uint32_t *list_tri, unsigned long long *list_n, uint64_t list_cap,
