@@ -47,8 +47,7 @@ struct BMesh {
     uint32_t *nf = nullptr;                         // filtered triangles of the level
     uint32_t *fword = nullptr;                      // filter words
     uint64_t *fstate = nullptr;                     // scan state of the filter
-    unsigned long long *s_acc = nullptr;            // max blocks
-    unsigned int *p_acc = nullptr, *t_acc = nullptr;
+    uint64_t *acc = nullptr;                        // voxelizer scratch (max blocks)
     uint32_t *cnt = nullptr, *rank = nullptr;       // max blocks + 1
     uint64_t *tmp = nullptr;                        // scan scratch
     // finest level
@@ -211,15 +210,13 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
         const int64_t nw = emb_bitmap_words(B.L[L].lv.nb_axis);
         fw = nw > fw ? nw : fw;
     }
-    BTRY(balloc(B, &B.fbits, fw));
+    BTRY(balloc(B, &B.fbits, fw + 1));
     EmbLevel &fin = B.L[B.Lf].lv;
     BTRY(balloc(B, &fin.nbr, fin.n * 26 + 1));
     BTRY(balloc(B, &B.nf, 1));
     BTRY(balloc(B, &B.fword, (size_t)(T + 31) / 32));
     BTRY(balloc(B, &B.fstate, (size_t)emb_filter_state_words(T)));
-    BTRY(balloc(B, &B.s_acc, nmax));
-    BTRY(balloc(B, &B.p_acc, nmax));
-    BTRY(balloc(B, &B.t_acc, nmax));
+    BTRY(balloc(B, &B.acc, (size_t)emb_vox_words(nmax)));
     BTRY(balloc(B, &B.cnt, nmax + 1));
     BTRY(balloc(B, &B.rank, nmax + 1));
     const int64_t sw = emb_scan_tmp_words(T > nmax ? (T > wmax ? T : wmax) : (nmax > wmax ? nmax : wmax));
@@ -268,7 +265,7 @@ static emb_status enqueue_mesh(BMesh &B, int tri_block, cudaStream_t s)
         const LevelGeom g = level_geom(&B.geo, L);
         BTRY(emb_enq_filter(rec, T, g, BL.flist, B.nf, B.fword, B.fstate, false, tri_block, s,
                             hr ? EMB_NO_EXPECT : (uint64_t)BL.nf));
-        BTRY(emb_enq_voxelize(rec, T, BL.flist, hr ? T : BL.nf, B.nf, nullptr, g, lv, B.s_acc, B.p_acc, B.t_acc, B.bq,
+        BTRY(emb_enq_voxelize(rec, T, BL.flist, hr ? T : BL.nf, B.nf, nullptr, g, lv, B.acc, nullptr, B.bq,
                               tri_block, s));
         if (L < B.Lf) {
             const long long dil = emb_refine_dilation(&B.geo, L, B.band);

@@ -350,9 +350,10 @@ emb_status emb_enq_level_index(EmbLevel &lv, uint64_t *tmp, cudaStream_t s)
 // it is, page-locked host memory through its device mapping (the kernel then writes
 // over the host link); pageable host memory, or an address the runtime does not know,
 // is refused before anything is enqueued.
-emb_status emb_device_view(void *p, void **dp)
+emb_status emb_device_view(void *p, void **dp, bool *device)
 {
     *dp = nullptr;
+    if (device) *device = false;
     if (!p) return EMB_OK;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -361,6 +362,7 @@ emb_status emb_device_view(void *p, void **dp)
     }
     if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) {
         *dp = p;
+        if (device) *device = a.type == cudaMemoryTypeDevice;
         return EMB_OK;
     }
     if (a.type == cudaMemoryTypeHost && a.devicePointer) {

@@ -77,6 +77,10 @@ struct emb_mesh_s {
     int64_t V, T;
     int4 *rec;      // T x 3 records {X, Y, Z, vertex id}
     int device;
+    // largest extent of a triangle per axis (frame units); not known once the vertices
+    // have moved (emb_mesh_update)
+    int32_t ext[3];
+    bool ext_known;
 };
 
 struct EmbLevel {
@@ -230,8 +234,9 @@ int64_t emb_bitmap_words(int64_t nb);
 emb_status emb_enq_level_index(EmbLevel &lv, uint64_t *tmp, cudaStream_t s);
 emb_status emb_build_hash(EmbLevel &lv, cudaStream_t s);
 // Device address of a caller output buffer (device memory, or page-locked host memory
-// through its mapping); EMB_ERR_BAD_INPUT for pageable memory.  NULL stays NULL.
-emb_status emb_device_view(void *p, void **dp);
+// through its mapping); EMB_ERR_BAD_INPUT for pageable memory.  NULL stays NULL.  *device:
+// plain device memory.
+emb_status emb_device_view(void *p, void **dp, bool *device = nullptr);
 // A pinned host slot (8 words) and its event for a count read-back; -1 when none is free.
 int emb_readback_acquire(uint64_t **h, cudaEvent_t *ev);
 void emb_readback_release(int slot);
@@ -256,9 +261,10 @@ emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbL
                              uint64_t *tmp, const EmbBigQ &Q, cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
 emb_status emb_enq_bin_scatter(const uint2 *list_bs, const uint32_t *list_tri, const unsigned long long *list_n,
                                uint64_t list_cap, const uint32_t *off, uint32_t *ent, uint64_t ent_cap, cudaStream_t s);
+int64_t emb_vox_words(int64_t n);
 emb_status emb_enq_voxelize(const int4 *rec, int64_t T, const uint32_t *flist, int64_t nf, const uint32_t *d_nf,
-                            const uint32_t *keep, LevelGeom g, const EmbLevel &lv, unsigned long long *s_acc,
-                            unsigned int *p_acc, unsigned int *t_acc, const EmbBigQ &Q, int block, cudaStream_t s);
+                            const uint32_t *keep, LevelGeom g, const EmbLevel &lv, uint64_t *acc, uint64_t *mask_out,
+                            const EmbBigQ &Q, int block, cudaStream_t s);
 emb_status emb_enq_refine(const int4 *rec, int64_t T, LevelGeom g, long long dil, const EmbLevel &lv, uint8_t *flags,
                           unsigned long long *fbits, const EmbBigQ &Q, cudaStream_t s);
 long long emb_refine_dilation(const emb_forest_s *f, int L, int band);
@@ -604,7 +610,13 @@ __device__ __forceinline__ unsigned long long emb_bigq_count(const EmbBigQ &Q)
     return n < Q.cap ? n : Q.cap;
 }
 
-// Host side (emb_common.cu): capacity for T triangles, allocation, per-launch reset.
+// Host side (emb_common.cu): capacity for T triangles (0 when no triangle can have more than
+// EMB_BIG_ITEMS items, `items` being the most one can have: no queue and no chunk kernel),
+// allocation, per-launch reset.
+static inline long long emb_mesh_items(const emb_mesh_s *m, long long a, long long b, long long c)
+{
+    return m->ext_known ? a * b * c : EMB_BIG_ITEMS + 1;
+}
 int64_t emb_bigq_capacity(int64_t T);
 emb_status emb_bigq_alloc(EmbBigQ &Q, int64_t T, cudaStream_t s);  // stream-ordered
 void emb_bigq_free(EmbBigQ &Q, cudaStream_t s);

@@ -1,6 +1,8 @@
 // Geometry input (Sec. 3.1): snapped vertex check, integer frame, 48-byte
 // triangle records, and the watertightness check on the GPU.
+#include <limits.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include "emb_internal.cuh"
 
@@ -73,13 +75,14 @@ __device__ __forceinline__ bool edge_enter(const EdgeTable &E, uint32_t a, uint3
     return false;
 }
 
-// Records, and with E.done the edges (a thread per triangle).
+// Records, the largest extents, and with E.done the edges (a thread per triangle).
 __global__ void k_mesh_records(const float *__restrict__ verts, const int32_t *__restrict__ tris, int64_t V, int64_t T,
-                               int32_t r_o, int4 *__restrict__ rec, EdgeTable E, int *err)
+                               int32_t r_o, int4 *__restrict__ rec, EdgeTable E, int *ext, int *err)
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int bad = 0;
     uint32_t done = 0;
+    int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {0, 0, 0};
     if (t < T) {
         int32_t vid[3];
 #pragma unroll
@@ -96,6 +99,8 @@ __global__ void k_mesh_records(const float *__restrict__ verts, const int32_t *_
                 float m = verts[3 * (int64_t)id + d] * 1048576.0f;  // exact: power-of-two scaling
                 if (!(m > 0.0f && m < 1048576.0f && m == truncf(m))) bad |= MESH_ERR_SNAP;
                 c[d] = (int)m * r_o;
+                lo[d] = min(lo[d], c[d]);
+                hi[d] = max(hi[d], c[d]);
             }
             rec[3 * t + k] = make_int4(c[0], c[1], c[2], id);
         }
@@ -108,6 +113,12 @@ __global__ void k_mesh_records(const float *__restrict__ verts, const int32_t *_
             }
         }
         if (bad) atomicOr(err, bad);
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int e = __reduce_max_sync(0xffffffffu, hi[d] >= lo[d] ? hi[d] - lo[d] : 0);
+        // few warps raise it: a read first
+        if ((threadIdx.x & 31) == 0 && e > *(volatile int *)(ext + d)) atomicMax(ext + d, e);
     }
     if (E.done) {
         done = __reduce_add_sync(0xffffffffu, done);
@@ -165,10 +176,10 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
     m->V = V;
     m->T = T;
     cudaGetDevice(&m->device);
-    // error word and completion counters, then the edge table: cleared together
+    // error word, completion counters and extents, then the edge table: cleared together
     char *scratch = nullptr;
     emb_status rc = EMB_OK;
-    uint32_t head[1 + EDGE_COUNTERS] = {0};
+    uint32_t head[1 + EDGE_COUNTERS + 3] = {0};
     const size_t a_head = 512;
     // room for every edge in a small mesh's overflow table (a triangle has 3/2); in a large
     // one for a third of them (a few percent overflow, more where a few vertices have many
@@ -195,7 +206,8 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
         const EdgeTable E = {slots ? (unsigned long long *)(scratch + a_head) : nullptr,
                              (unsigned long long *)(scratch + a_head + a_slot), cap, want >= 2 * T ? cap : 128,
                              check_watertight ? (uint32_t *)scratch + 1 : nullptr};
-        EMB_LAUNCH((k_mesh_records), emb_grid(T, 256), 256, 0, s)(d_verts, d_tris, V, T, r_o, m->rec, E, (int *)scratch);
+        EMB_LAUNCH((k_mesh_records), emb_grid(T, 256), 256, 0, s)(d_verts, d_tris, V, T, r_o, m->rec, E,
+                                                                      (int *)scratch + 1 + EDGE_COUNTERS, (int *)scratch);
         if (cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(head, scratch, sizeof(head), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) {
@@ -212,6 +224,8 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
         for (int i = 0; i < EDGE_COUNTERS; ++i) closed += head[1 + i];
         if (2 * closed != 3 * T) head[0] |= MESH_ERR_OPEN_EDGE;
     }
+    memcpy(m->ext, head + 1 + EDGE_COUNTERS, sizeof(m->ext));
+    m->ext_known = true;
     if (head[0] & (MESH_ERR_ID | MESH_ERR_SNAP)) rc = EMB_ERR_BAD_INPUT;
     else if (head[0]) rc = EMB_ERR_NOT_WATERTIGHT;
 done:
@@ -237,6 +251,7 @@ extern "C" emb_status emb_mesh_update(emb_mesh m, const float *d_verts, int64_t 
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
     cudaStream_t s = emb_stream(stream);
+    m->ext_known = false;
     EMB_LAUNCH((k_mesh_move), emb_grid(3 * m->T, 256), 256, 0, s)(d_verts, V, m->T, m->r_o, m->rec, st);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;

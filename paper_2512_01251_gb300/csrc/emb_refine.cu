@@ -334,7 +334,9 @@ long long emb_refine_dilation(const emb_forest_s *f, int L, int band)
     return num >> sh;
 }
 
-// Enqueue only: flags (lv.n bytes) are cleared and set.
+// Enqueue only: flags (lv.n bytes) are cleared and set; fbits (NULL for a level without a
+// bitmap) is scratch of a word more than the level's bitmap has, the last one the count of
+// the chunk queue.
 emb_status emb_enq_refine(const int4 *rec, int64_t T, LevelGeom g, long long dil, const EmbLevel &lv, uint8_t *flags,
                           unsigned long long *fbits, const EmbBigQ &Q, cudaStream_t s)
 {
@@ -342,18 +344,19 @@ emb_status emb_enq_refine(const int4 *rec, int64_t T, LevelGeom g, long long dil
     EMB_CUDA_TRY(cudaMemsetAsync(flags, 0, lv.n, s));
     const EmbLookup lk = emb_lookup_of(lv);
     FlagBits fb = {nullptr, g.nb};
+    EmbBigQ q = Q;
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
     if (fbits && nw > 0) {
-        EMB_CUDA_TRY(cudaMemsetAsync(fbits, 0, nw * sizeof(unsigned long long), s));
+        EMB_CUDA_TRY(cudaMemsetAsync(fbits, 0, (nw + 1) * sizeof(unsigned long long), s));
         fb.w = fbits;
-    }
-    if (Q.cap) EMB_CUDA_TRY(cudaMemsetAsync(Q.n, 0, sizeof(unsigned long long), s));
+        q.n = fbits + nw;
+    } else if (Q.cap) EMB_CUDA_TRY(cudaMemsetAsync(Q.n, 0, sizeof(unsigned long long), s));
     int64_t grid = (T + 32 * EMB_WU_WARPS - 1) / (32 * EMB_WU_WARPS);
     const int64_t resident = (int64_t)emb_sm_count() * REFINE_MINB;
     if (grid > resident) grid = resident;
     if (grid < 1) grid = 1;
-    EMB_LAUNCH((k_refine), (int)grid, 32 * EMB_WU_WARPS, 0, s)(rec, T, g, dil, lk, flags, fb, Q);
-    if (Q.cap) EMB_LAUNCH((k_refine_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, dil, lk, flags, fb, Q);
+    EMB_LAUNCH((k_refine), (int)grid, 32 * EMB_WU_WARPS, 0, s)(rec, T, g, dil, lk, flags, fb, q);
+    if (q.cap) EMB_LAUNCH((k_refine_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, dil, lk, flags, fb, q);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
@@ -370,15 +373,22 @@ extern "C" emb_status emb_refine_flags(emb_forest f, emb_bins b, int32_t level, 
     long long dil = emb_refine_dilation(f, level, band);
     if (dil < 0) return EMB_ERR_RANGE;
     cudaStream_t s = emb_stream(stream);
-    EmbBigQ Q;
-    emb_status rc = emb_bigq_alloc(Q, b->m->T, s);
-    if (rc != EMB_OK) return rc;
-    unsigned long long *fbits = nullptr;
+    // the flagged bits, and the chunk queue where a triangle may meet more than
+    // EMB_BIG_ITEMS dilated blocks: [-dil, extent + dil] spans at most this many an axis
+    const emb_mesh m = b->m;
+    const LevelGeom g = level_geom(f, level);
+    auto span = [&](int d) { return ((m->ext[d] + 2 * dil) >> g.lW) + 2; };
+    EmbBigQ Q = {nullptr, nullptr, 0};
+    if (emb_mesh_items(m, span(0), span(1), span(2)) > EMB_BIG_ITEMS) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
-    if (nw > 0 && emb_malloc_async(&fbits, nw * sizeof(unsigned long long), s) != cudaSuccess) fbits = nullptr;
-    rc = emb_enq_refine(b->m->rec, b->m->T, level_geom(f, level), dil, lv, d_flags, fbits, Q, s);
-    if (fbits) cudaFreeAsync(fbits, s);
-    emb_bigq_free(Q, s);
+    const size_t a_bits = ((size_t)(nw + 1) * sizeof(unsigned long long) + 255) & ~(size_t)255;
+    char *scratch = nullptr;
+    EMB_CUDA_TRY(emb_malloc_async(&scratch, a_bits + (size_t)Q.cap * sizeof(uint2), s));
+    Q.n = (unsigned long long *)scratch + nw;
+    Q.q = (uint2 *)(scratch + a_bits);
+    const emb_status rc = emb_enq_refine(m->rec, m->T, g, dil, lv, d_flags,
+                                         nw > 0 ? (unsigned long long *)scratch : nullptr, Q, s);
+    cudaFreeAsync(scratch, s);
     return rc;
 }
 
