@@ -48,19 +48,18 @@ struct BMesh {
     uint32_t *fword = nullptr;                      // filter words
     uint64_t *fstate = nullptr;                     // scan state of the filter
     uint64_t *acc = nullptr;                        // voxelizer scratch (max blocks)
-    uint32_t *cnt = nullptr, *rank = nullptr;       // max blocks + 1
+    uint32_t *rank = nullptr;                       // max blocks + 1
+    uint64_t *bin_z = nullptr;                      // cleared scratch of the binning pass
     uint64_t *tmp = nullptr;                        // scan scratch
     // finest level
     uint32_t *bin_off = nullptr, *bin_ent = nullptr;
     uint2 *list_bs = nullptr;                       // pair list of the binning pass (planned pairs)
     uint32_t *list_tri = nullptr;
-    unsigned long long *list_n = nullptr;
     uint64_t *cand = nullptr;
     uint32_t *work_n = nullptr, *work = nullptr, *blk_off = nullptr;
-    unsigned int *next = nullptr;                   // queue cursor of a per-mesh link launch
     uint2 *witem = nullptr;                         // link work items
     uint2 *extra = nullptr;                         // extra parts of split blocks
-    unsigned long long *extra_n = nullptr;
+    unsigned long long *queue = nullptr;            // extra parts asked for, cursor of a per-mesh link launch
     EmbBigQ bq = {nullptr, nullptr, 0};             // chunk queue of large triangles
     unsigned long long *fbits = nullptr;            // dense flagged bits (largest refined level)
     int32_t *o_cell = nullptr, *o_tri = nullptr;
@@ -137,7 +136,7 @@ static emb_status plan_mesh(BMesh &B, cudaStream_t s)
             B.links = nl;
             if (rc == EMB_OK) {
                 uint32_t nw = 0;
-                if (cudaMemcpyAsync(&nw, f->work_n + f->lv[L].n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) !=
+                if (cudaMemcpyAsync(&nw, f->work_n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s) !=
                         cudaSuccess ||
                     cudaStreamSynchronize(s) != cudaSuccess)
                     rc = EMB_ERR_CUDA;
@@ -217,7 +216,6 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     BTRY(balloc(B, &B.fword, (size_t)(T + 31) / 32));
     BTRY(balloc(B, &B.fstate, (size_t)emb_filter_state_words(T)));
     BTRY(balloc(B, &B.acc, (size_t)emb_vox_words(nmax)));
-    BTRY(balloc(B, &B.cnt, nmax + 1));
     BTRY(balloc(B, &B.rank, nmax + 1));
     const int64_t sw = emb_scan_tmp_words(T > nmax ? (T > wmax ? T : wmax) : (nmax > wmax ? nmax : wmax));
     BTRY(balloc(B, &B.tmp, sw));
@@ -225,15 +223,14 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     BTRY(balloc(B, &B.bin_ent, B.pairs + 1));
     BTRY(balloc(B, &B.list_bs, B.pairs + 1));
     BTRY(balloc(B, &B.list_tri, B.pairs + 1));
-    BTRY(balloc(B, &B.list_n, 1));
+    BTRY(balloc(B, &B.bin_z, (size_t)emb_bin_words(fin.n)));
     BTRY(balloc(B, &B.cand, fin.n * 26 + 1));
-    BTRY(balloc(B, &B.work_n, fin.n + 1));
+    BTRY(balloc(B, &B.work_n, 1));
     BTRY(balloc(B, &B.work, fin.n + 1));
     BTRY(balloc(B, &B.blk_off, fin.n + 1));
-    BTRY(balloc(B, &B.next, 1));
     BTRY(balloc(B, &B.witem, fin.n + 1));
     BTRY(balloc(B, &B.extra, (size_t)emb_link_extra_capacity(fin.n)));
-    BTRY(balloc(B, &B.extra_n, 1));
+    BTRY(balloc(B, &B.queue, 2));
     BTRY(balloc(B, &B.bq.n, 1));
     BTRY(balloc(B, &B.bq.q, (size_t)emb_bigq_capacity(T)));
     B.bq.cap = (uint32_t)emb_bigq_capacity(T);
@@ -242,12 +239,6 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     BTRY(balloc(B, &B.o_q, B.links + 1));
     BTRY(balloc(B, &B.o_tri, B.links + 1));
     return EMB_OK;
-}
-
-// EMB_ERR_CAPACITY when the pair list asked for more entries than it holds.
-__global__ void k_list_check(const unsigned long long *__restrict__ list_n, uint64_t cap, int *st)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0 && *list_n > cap) emb_set_status(st, EMB_ERR_CAPACITY);
 }
 
 // Enqueues the pipeline of mesh B up to (not including) the link kernel, on stream s.
@@ -275,16 +266,15 @@ static emb_status enqueue_mesh(BMesh &B, int tri_block, cudaStream_t s)
             EmbLevel &C = B.L[L + 1].lv;
             BTRY(emb_enq_child_level(lv, BL.flags, B.rank, C, C.n, true, hr ? B.d_n + L + 1 : nullptr, B.tmp, false, s));
         } else {
-            BTRY(emb_enq_bin_pairs(rec, T, g, lv, B.cnt, B.bin_off, B.list_bs, B.list_tri, B.list_n, (uint64_t)B.pairs,
-                                   B.tmp, B.bq, s, hr ? EMB_NO_EXPECT : (uint64_t)B.pairs));
-            if (hr) EMB_LAUNCH((k_list_check), 1, 32, 0, s)(B.list_n, (uint64_t)B.pairs, st);
-            BTRY(emb_enq_bin_scatter(B.list_bs, B.list_tri, B.list_n, (uint64_t)B.pairs, B.bin_off, B.bin_ent,
-                                     (uint64_t)B.pairs, s));
+            BTRY(emb_enq_bin_pairs(rec, T, g, lv, B.bin_z, B.bin_off, B.list_bs, B.list_tri, (uint64_t)B.pairs, B.bq, s,
+                                   hr ? EMB_NO_EXPECT : (uint64_t)B.pairs));
+            BTRY(emb_enq_bin_scatter(lv, B.bin_z, B.list_bs, B.list_tri, (uint64_t)B.pairs, B.bin_off, B.bin_ent,
+                                     (uint64_t)B.pairs, nullptr, hr, s));
             BTRY(emb_enq_neighbors(lv, s));
-            BTRY(emb_enq_link_prep(lv, B.lattice, B.cand, B.cnt, B.rank, B.work_n, B.work, B.blk_off, B.tmp, s,
+            BTRY(emb_enq_link_prep(lv, B.lattice, B.cand, B.rank, B.work_n, B.work, B.blk_off, B.tmp, s,
                                    hr ? EMB_NO_EXPECT : (uint64_t)B.nwork, hr ? EMB_NO_EXPECT : (uint64_t)B.links));
-            BTRY(emb_enq_link_split(lv, B.work, B.work_n + lv.n, B.cand, B.blk_off, B.bin_off, B.witem, B.extra,
-                                    B.extra_n, (uint32_t)emb_link_extra_capacity(lv.n), s));
+            BTRY(emb_enq_link_split(lv, B.work, B.work_n, B.cand, B.blk_off, B.bin_off, B.witem, B.extra, B.queue,
+                                    (uint32_t)emb_link_extra_capacity(lv.n), nullptr, s));
         }
     }
     return EMB_OK;
@@ -398,10 +388,10 @@ static LinkMesh link_mesh(BMesh &B)
     M.ent_cap = (uint64_t)B.pairs;
     M.rec = B.m->rec;
     M.T = (uint32_t)B.m->T;
-    M.work_n = B.work_n + fin.n;
+    M.work_n = B.work_n;
     M.witem = B.witem;
     M.extra = B.extra;
-    M.extra_n = B.extra_n;
+    M.extra_n = B.queue;
     M.extra_cap = (uint32_t)emb_link_extra_capacity(fin.n);
     M.o_cell = B.o_cell;
     M.o_dir = B.o_dir;
@@ -449,7 +439,7 @@ static emb_status batch_enqueue(emb_batch b, cudaStream_t s)
                 EMB_CUDA_TRY(cudaEventRecord(b->ev_mesh[order[q]], b->st[k]));
                 EMB_CUDA_TRY(cudaStreamWaitEvent(ls, b->ev_mesh[order[q]], 0));
             }
-            BTRY(emb_enq_link_emit(one, B.next, b->link_ctas, ls, B.nwork > 0 ? B.nwork : 1));
+            BTRY(emb_enq_link_emit(one, (unsigned int *)(B.queue + 1), true, b->link_ctas, ls, B.nwork > 0 ? B.nwork : 1));
         }
     }
     for (int i = 0; i < K; ++i) {
@@ -464,7 +454,7 @@ static emb_status batch_enqueue(emb_batch b, cudaStream_t s)
     LinkTable tab;
     tab.n = (int)b->m.size();
     for (int j = 0; j < tab.n; ++j) tab.m[j] = link_mesh(b->m[j]);
-    return emb_enq_link_emit(tab, b->next, b->link_ctas, s, 0);
+    return emb_enq_link_emit(tab, b->next, false, b->link_ctas, s, 0);
 }
 
 extern "C" emb_status emb_batch_run(emb_batch b, void *stream)

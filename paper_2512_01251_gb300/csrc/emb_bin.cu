@@ -509,12 +509,19 @@ static emb_status enq_filter_flags(const int4 *rec, int64_t T, LevelGeom g, uint
     return EMB_OK;
 }
 
-// The pair list into the CSR bins: entry e goes to off[block] + slot (below ent_cap).
+// The pair list into the CSR bins: entry e goes to off[block] + slot (below ent_cap).  The
+// number of entries asked for goes to *req (when given), and one above cap raises
+// EMB_ERR_CAPACITY (`check`).
 __global__ void k_bin_scatter(const uint2 *__restrict__ bs, const uint32_t *__restrict__ tri,
                               const unsigned long long *__restrict__ n, uint64_t cap, const uint32_t *__restrict__ off,
-                              uint32_t *__restrict__ ent, uint64_t ent_cap)
+                              uint32_t *__restrict__ ent, uint64_t ent_cap, unsigned long long *__restrict__ req,
+                              bool check, int *st)
 {
     const unsigned long long m = *n < cap ? *n : cap;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (req) *req = *n;
+        if (check && *n > cap) emb_set_status(st, EMB_ERR_CAPACITY);
+    }
     for (unsigned long long e = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; e < m;
          e += (unsigned long long)gridDim.x * blockDim.x) {
         const uint2 v = bs[e];
@@ -523,33 +530,53 @@ __global__ void k_bin_scatter(const uint2 *__restrict__ bs, const uint32_t *__re
     }
 }
 
-// Steps 2-9 at the finest level, geometry half (enqueue only): cnt holds n + 1 uint32
-// and receives the pairs per block, off their n + 1 offsets (total at off[n]); the
-// list holds list_cap entries (list_n counts the requests); tmp: scan scratch for n.
-emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbLevel &lv, uint32_t *cnt, uint32_t *off,
-                             uint2 *list_bs, uint32_t *list_tri, unsigned long long *list_n, uint64_t list_cap,
-                             uint64_t *tmp, const EmbBigQ &Q, cudaStream_t s, uint64_t expect)
+// Scratch of the geometry half, cleared together: the pairs per block (n + 1 uint32), the
+// requests to the pair list, the count of the chunk queue, and the scan state.
+struct BinScratch {
+    uint32_t *cnt;
+    unsigned long long *list_n, *big_n;
+    uint64_t *state;
+};
+static BinScratch bin_scratch(uint64_t *z, int64_t n)
 {
-    EMB_CUDA_TRY(cudaMemsetAsync(cnt, 0, (lv.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(cudaMemsetAsync(list_n, 0, sizeof(unsigned long long), s));
+    const int64_t c = (n + 2) / 2;
+    return {(uint32_t *)z, (unsigned long long *)z + c, (unsigned long long *)z + c + 1, z + c + 2};
+}
+int64_t emb_bin_words(int64_t n) { return (n + 2) / 2 + 2 + emb_scan_tmp_words(n); }
+
+// Steps 2-9 at the finest level, geometry half (enqueue only): z is scratch of
+// emb_bin_words(lv.n) words; off receives the n + 1 offsets of the blocks' pairs (total at
+// off[n], and at *d_total when given); the list holds list_cap entries.
+emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbLevel &lv, uint64_t *z, uint32_t *off,
+                             uint2 *list_bs, uint32_t *list_tri, uint64_t list_cap, const EmbBigQ &Q, cudaStream_t s,
+                             uint64_t expect, uint32_t *d_total)
+{
+    const BinScratch S = bin_scratch(z, lv.n);
+    EMB_CUDA_TRY(cudaMemsetAsync(z, 0, emb_bin_words(lv.n) * sizeof(uint64_t), s));
     const EmbLookup lk = emb_lookup_of(lv);
-    const PairList PL = {list_bs, list_tri, list_n, list_cap};
-    if (Q.cap) EMB_CUDA_TRY(cudaMemsetAsync(Q.n, 0, sizeof(unsigned long long), s));
+    const PairList PL = {list_bs, list_tri, S.list_n, list_cap};
+    EmbBigQ q = Q;
+    q.n = S.big_n;
     if (T > 0)
-        EMB_LAUNCH((k_bin_pairs), emb_grid(T, 32 * EMB_WU_WARPS), 32 * EMB_WU_WARPS, 0, s)(rec, T, g, g.half, lk, cnt, PL,
-                                                                                           Q);
-    if (Q.cap) EMB_LAUNCH((k_bin_pairs_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, g.half, lk, cnt, PL, Q);
-    return emb_scan_into_expect(cnt, off, lv.n, tmp, expect, s);
+        EMB_LAUNCH((k_bin_pairs), emb_grid(T, 32 * EMB_WU_WARPS), 32 * EMB_WU_WARPS, 0, s)(rec, T, g, g.half, lk, S.cnt, PL,
+                                                                                           q);
+    if (q.cap) EMB_LAUNCH((k_bin_pairs_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, g.half, lk, S.cnt, PL, q);
+    return emb_scan_into_expect(S.cnt, off, lv.n, S.state, expect, s, d_total, true);
 }
 
-// Scatter half: ent holds ent_cap entries.
-emb_status emb_enq_bin_scatter(const uint2 *list_bs, const uint32_t *list_tri, const unsigned long long *list_n,
-                               uint64_t list_cap, const uint32_t *off, uint32_t *ent, uint64_t ent_cap, cudaStream_t s)
+// Scatter half: z as left by the geometry half; ent holds ent_cap entries.  `check` and
+// d_req: see k_bin_scatter.
+emb_status emb_enq_bin_scatter(const EmbLevel &lv, uint64_t *z, const uint2 *list_bs, const uint32_t *list_tri,
+                               uint64_t list_cap, const uint32_t *off, uint32_t *ent, uint64_t ent_cap,
+                               unsigned long long *d_req, bool check, cudaStream_t s)
 {
+    int *st = emb_status_word();
+    if (!st) return EMB_ERR_CUDA;
     int64_t grid = (int64_t)((list_cap + 255) / 256);
     if (grid > 152 * 16) grid = 152 * 16;
     if (grid < 1) grid = 1;
-    EMB_LAUNCH((k_bin_scatter), (int)grid, 256, 0, s)(list_bs, list_tri, list_n, list_cap, off, ent, ent_cap);
+    EMB_LAUNCH((k_bin_scatter), (int)grid, 256, 0, s)(list_bs, list_tri, bin_scratch(z, lv.n).list_n, list_cap, off, ent,
+                                                      ent_cap, d_req, check, st);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
@@ -562,15 +589,16 @@ static emb_status bin_finest(emb_bins b, uint64_t list_cap, uint64_t ent_cap, cu
     const EmbLevel &lv = b->f->lv[b->level];
     const LevelGeom g = level_geom(b->f, b->level);
     emb_status rc = EMB_OK;
-    uint32_t *cnt = nullptr;
-    uint64_t *tmp = nullptr;
-    char *list = nullptr;
+    // one scratch: the cleared words, the pair list, and the chunk queue where a triangle may
+    // meet more than EMB_BIG_ITEMS blocks dilated by half a cell
+    const long long span = ((m->ext + g.h) >> g.lW) + 2;
     EmbBigQ Q = {nullptr, nullptr, 0};
-    const size_t a_bs = ((size_t)list_cap * sizeof(uint2) + 255) & ~(size_t)255;
-    if (emb_malloc_async(&cnt, (lv.n + 1) * sizeof(uint32_t), s) != cudaSuccess ||
-        emb_malloc_async(&tmp, emb_scan_tmp_words(lv.n) * sizeof(uint64_t), s) != cudaSuccess ||
-        emb_malloc_async((void **)&list, 256 + a_bs + (size_t)list_cap * sizeof(uint32_t), s) != cudaSuccess)
-        rc = EMB_ERR_CUDA;
+    if (emb_mesh_big(m, span, span, span)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t a_z = up((size_t)emb_bin_words(lv.n) * sizeof(uint64_t)), a_bs = up((size_t)list_cap * sizeof(uint2)),
+                 a_tri = up((size_t)list_cap * sizeof(uint32_t));
+    char *scratch = nullptr;
+    if (emb_malloc_async(&scratch, a_z + a_bs + a_tri + (size_t)Q.cap * sizeof(uint2), s) != cudaSuccess) rc = EMB_ERR_CUDA;
     if (rc == EMB_OK && !b->off && emb_malloc_async(&b->off, (lv.n + 1) * sizeof(uint32_t), s) != cudaSuccess)
         rc = EMB_ERR_CUDA;
     if (rc == EMB_OK && b->ent_cap != ent_cap) {
@@ -579,21 +607,18 @@ static emb_status bin_finest(emb_bins b, uint64_t list_cap, uint64_t ent_cap, cu
         b->ent_cap = ent_cap;
         if (emb_malloc_async(&b->ent, ((size_t)ent_cap + 1) * sizeof(uint32_t), s) != cudaSuccess) rc = EMB_ERR_CUDA;
     }
-    if (rc == EMB_OK) rc = emb_bigq_alloc(Q, m->T, s);
-    unsigned long long *ln = (unsigned long long *)list;
-    uint2 *lbs = (uint2 *)(list + 256);
-    uint32_t *ltri = (uint32_t *)(list + 256 + a_bs);
-    if (rc == EMB_OK) rc = emb_enq_bin_pairs(m->rec, m->T, g, lv, cnt, b->off, lbs, ltri, ln, list_cap, tmp, Q, s);
-    if (rc == EMB_OK) rc = emb_enq_bin_scatter(lbs, ltri, ln, list_cap, b->off, b->ent, ent_cap, s);
-    if (rc == EMB_OK &&
-        (cudaMemcpyAsync(b->dcount + 4, b->off + lv.n, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-         cudaMemcpyAsync(b->dcount + 8, ln, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s) != cudaSuccess))
-        rc = EMB_ERR_CUDA;
+    uint64_t *z = (uint64_t *)scratch;
+    uint2 *lbs = (uint2 *)(scratch + a_z);
+    uint32_t *ltri = (uint32_t *)(scratch + a_z + a_bs);
+    Q.q = (uint2 *)(scratch + a_z + a_bs + a_tri);
+    if (rc == EMB_OK)
+        rc = emb_enq_bin_pairs(m->rec, m->T, g, lv, z, b->off, lbs, ltri, list_cap, Q, s, EMB_NO_EXPECT,
+                               (uint32_t *)(b->dcount + 4));
+    if (rc == EMB_OK)
+        rc = emb_enq_bin_scatter(lv, z, lbs, ltri, list_cap, b->off, b->ent, ent_cap, (unsigned long long *)(b->dcount + 8),
+                                 false, s);
     b->list_cap = list_cap;
-    emb_bigq_free(Q, s);
-    if (list) cudaFreeAsync(list, s);
-    if (cnt) cudaFreeAsync(cnt, s);
-    if (tmp) cudaFreeAsync(tmp, s);
+    if (scratch) cudaFreeAsync(scratch, s);
     return rc;
 }
 

@@ -555,26 +555,6 @@ int64_t emb_bigq_capacity(int64_t T)
     return c < (1 << 20) ? c : (1 << 20);
 }
 
-emb_status emb_bigq_alloc(EmbBigQ &Q, int64_t T, cudaStream_t s)
-{
-    Q.q = nullptr;
-    Q.n = nullptr;
-    Q.cap = (uint32_t)emb_bigq_capacity(T);
-    char *p = nullptr;
-    EMB_CUDA_TRY(emb_malloc_async((void **)&p, 256 + (size_t)Q.cap * sizeof(uint2), s));
-    Q.n = (unsigned long long *)p;
-    Q.q = (uint2 *)(p + 256);
-    return EMB_OK;
-}
-
-void emb_bigq_free(EmbBigQ &Q, cudaStream_t s)
-{
-    if (Q.n) cudaFreeAsync(Q.n, s);
-    Q.q = nullptr;
-    Q.n = nullptr;
-    Q.cap = 0;
-}
-
 // Multiprocessors of the current device (cached per device; persistent grids).
 int emb_sm_count()
 {

@@ -15,6 +15,7 @@
 //   t = N / (h M) between crossings (lowest triangle id on equality).  q = t is
 //   rounded to float once.
 #include "emb_internal.cuh"
+#include "emb_scan.cuh"
 
 #define LINK_TILE 64
 
@@ -909,24 +910,84 @@ __global__ void k_count_check(const uint32_t *__restrict__ blk_off, int64_t n, i
     if (threadIdx.x == 0 && blockIdx.x == 0 && blk_off[n] > 0) emb_set_status(st, EMB_ERR_CAPACITY);
 }
 
-__global__ void k_nonempty(const uint32_t *__restrict__ cnt, int64_t n, uint32_t *__restrict__ flag)
+// Link offsets and the list of blocks with links from the blocks' link counts, in one
+// launch: a block's links and whether it has any travel in one word (links << 26 |
+// blocks: a table's cell ids are 32-bit, so there are fewer than 2^25 blocks and 2^36
+// links), summed over the tiles by look-back.  Blocks past the level's count hold no links.
+// Totals: blk_off[n] and *work_n, checked against the planned ones.  (Flags, two scans and a
+// compaction were six launches, 18 us on 97K blocks without the gaps between them.)
+#define LISTS_BLOCK 512
+#define LISTS_ITEMS 8
+#define LISTS_TILE (LISTS_BLOCK * LISTS_ITEMS)
+#define LISTS_BITS 26
+__global__ void __launch_bounds__(LISTS_BLOCK) k_link_lists(const uint32_t *__restrict__ cnt, int64_t n,
+                                                            const uint32_t *d_n, uint32_t *__restrict__ blk_off,
+                                                            uint32_t *__restrict__ work, uint32_t *__restrict__ work_n,
+                                                            uint64_t *__restrict__ state, uint64_t expect_work,
+                                                            uint64_t expect_links, int *st)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = cnt[i] ? 1u : 0u;
+    __shared__ uint32_t s_tile;
+    __shared__ uint64_t s_warp[LISTS_BLOCK / 32 + 1];
+    const uint32_t tile = state ? scan_ticket(state, &s_tile) : 0u;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t base = (int64_t)tile * LISTS_TILE + (int64_t)threadIdx.x * LISTS_ITEMS, live = emb_count(n, d_n);
+    uint32_t v[LISTS_ITEMS];
+    uint64_t own = 0;
+#pragma unroll
+    for (int i = 0; i < LISTS_ITEMS; ++i) {
+        v[i] = base + i < live ? cnt[base + i] : 0u;
+        own += (uint64_t)v[i] << LISTS_BITS | (v[i] ? 1u : 0u);
+    }
+    uint64_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint64_t t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        const uint64_t x = lane < LISTS_BLOCK / 32 ? s_warp[lane] : 0;
+        uint64_t xi = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint64_t t = __shfl_up_sync(0xffffffffu, xi, o);
+            if (lane >= o) xi += t;
+        }
+        const uint64_t sum = __shfl_sync(0xffffffffu, xi, 31);
+        const uint64_t before = state ? scan_lookback(state, tile, sum, st) : 0;
+        if (lane < LISTS_BLOCK / 32) s_warp[lane] = xi - x;
+        if (lane == 0) s_warp[LISTS_BLOCK / 32] = before;
+    }
+    __syncthreads();
+    uint64_t run = s_warp[LISTS_BLOCK / 32] + s_warp[w] + incl - own;
+#pragma unroll
+    for (int i = 0; i < LISTS_ITEMS; ++i) {
+        const uint64_t links = run >> LISTS_BITS;
+        const uint32_t blocks = (uint32_t)run & ((1u << LISTS_BITS) - 1u);
+        if (base + i <= n) {
+            if (links > 0xFFFFFFFFull) emb_set_status(st, EMB_ERR_CAPACITY);
+            blk_off[base + i] = (uint32_t)links;
+            if (v[i]) work[blocks] = (uint32_t)(base + i);
+            if (base + i == n) {
+                *work_n = blocks;
+                if ((expect_work != EMB_NO_EXPECT && blocks != expect_work) ||
+                    (expect_links != EMB_NO_EXPECT && links != expect_links))
+                    emb_set_status(st, EMB_ERR_STATE);
+            }
+        }
+        run += (uint64_t)v[i] << LISTS_BITS | (v[i] ? 1u : 0u);
+    }
 }
 
-__global__ void k_compact_ids(const uint32_t *__restrict__ flag, const uint32_t *__restrict__ pos, int64_t n,
-                              uint32_t *__restrict__ out)
-{
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && flag[i]) out[pos[i]] = (uint32_t)i;
-}
+int64_t emb_link_state_words(int64_t n) { return scan_state_words((n + LISTS_TILE) / LISTS_TILE); }
 
 static void free_candidates(emb_forest f, cudaStream_t s)
 {
     if (f->cand) cudaFreeAsync(f->cand, s);
     f->cand = nullptr;
-    uint32_t **bufs[] = {&f->blk_off, &f->work, &f->work_n};
+    f->work_n = nullptr;
+    uint32_t **bufs[] = {&f->blk_off, &f->work};
     for (uint32_t **p : bufs) {
         if (*p) cudaFreeAsync(*p, s);
         *p = nullptr;
@@ -934,25 +995,24 @@ static void free_candidates(emb_forest f, cudaStream_t s)
 }
 
 // Link preparation for the finest level (enqueue only, neighbour table in place):
-// cand (26 n words), cnt and flag (n + 1 uint32, scratch), work_n (n + 1: the
-// work-list scan, count at work_n[n]), work (n), blk_off (n + 1: link offsets,
-// total at blk_off[n]), tmp (scan scratch for n).
-emb_status emb_enq_link_prep(const EmbLevel &lv, int lattice, uint64_t *cand, uint32_t *cnt, uint32_t *flag,
-                             uint32_t *work_n, uint32_t *work, uint32_t *blk_off, uint64_t *tmp, cudaStream_t s,
-                             uint64_t expect_work, uint64_t expect_links)
+// cand (26 n words), cnt (n uint32, scratch), work (n) and *work_n: the blocks with links
+// and their count, blk_off (n + 1: link offsets, total at blk_off[n]), state
+// (emb_link_state_words(n) words of scratch).
+emb_status emb_enq_link_prep(const EmbLevel &lv, int lattice, uint64_t *cand, uint32_t *cnt, uint32_t *work_n,
+                             uint32_t *work, uint32_t *blk_off, uint64_t *state, cudaStream_t s, uint64_t expect_work,
+                             uint64_t expect_links)
 {
-    EMB_CUDA_TRY(cudaMemsetAsync(cnt, 0, (lv.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(cudaMemsetAsync(flag, 0, (lv.n + 1) * sizeof(uint32_t), s));
-    if (lv.n > 0) {
-        EMB_LAUNCH((k_link_cand), emb_grid(lv.n, CAND_BLOCK), CAND_BLOCK, 0, s)(lv.mask, lv.nbr, lv.n, lattice, cand, cnt,
-                                                                  emb_status_word(), lv.d_n);
-        EMB_LAUNCH((k_nonempty), emb_grid(lv.n, 256), 256, 0, s)(cnt, lv.n, flag);
-    }
-    emb_status rc = emb_scan_into_expect(flag, work_n, lv.n, tmp, expect_work, s);
-    if (rc != EMB_OK) return rc;
-    if (lv.n > 0) EMB_LAUNCH((k_compact_ids), emb_grid(lv.n, 256), 256, 0, s)(flag, work_n, lv.n, work);
+    int *st = emb_status_word();
+    if (!st) return EMB_ERR_CUDA;
+    const int64_t tiles = (lv.n + LISTS_TILE) / LISTS_TILE;
+    if (tiles > 1) EMB_CUDA_TRY(cudaMemsetAsync(state, 0, scan_state_words(tiles) * sizeof(uint64_t), s));
+    if (lv.n > 0)
+        EMB_LAUNCH((k_link_cand), emb_grid(lv.n, CAND_BLOCK), CAND_BLOCK, 0, s)(lv.mask, lv.nbr, lv.n, lattice, cand, cnt, st,
+                                                                                  lv.d_n);
+    EMB_LAUNCH((k_link_lists), (int)tiles, LISTS_BLOCK, 0, s)(cnt, lv.n, lv.d_n, blk_off, work, work_n,
+                                                              tiles > 1 ? state : nullptr, expect_work, expect_links, st);
     EMB_CUDA_TRY(cudaGetLastError());
-    return emb_scan_into_expect(cnt, blk_off, lv.n, tmp, expect_links, s);
+    return EMB_OK;
 }
 
 // Work items (thread per block with links): block b with l links, a bin of nt
@@ -961,13 +1021,16 @@ emb_status emb_enq_link_prep(const EmbLevel &lv, int lattice, uint64_t *cand, ui
 // ceil(nbc / P) consecutive cells.  The first part is the block's own item; the
 // others are appended to `extra`, and when that is full the block stays whole,
 // which changes the speed only.  The lanes of a warp take their extra slots with one
-// atomic (a single counter taken once per heavy block serialised the kernel).
+// atomic (a single counter taken once per heavy block serialised the kernel).  d_count,
+// when given, receives the table's links.
 __global__ void k_link_split(const uint32_t *__restrict__ work, const uint32_t *__restrict__ work_n,
                              const uint64_t *__restrict__ cand, const uint32_t *__restrict__ blk_off,
                              const uint32_t *__restrict__ bin_off, int64_t n, uint2 *__restrict__ witem,
-                             uint2 *__restrict__ extra, unsigned long long *__restrict__ extra_n, uint32_t cap)
+                             uint2 *__restrict__ extra, unsigned long long *__restrict__ extra_n, uint32_t cap,
+                             int64_t *__restrict__ d_count)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && d_count) *d_count = (int64_t)blk_off[n];
     const int lane = threadIdx.x & 31;
     const bool live = i < n && i < (int64_t)*work_n;
     if (__ballot_sync(0xffffffffu, live) == 0u) return;  // the whole warp
@@ -1025,12 +1088,12 @@ int64_t emb_link_extra_capacity(int64_t n)
 // Enqueue only: after emb_enq_link_prep and the finest bins; witem holds n entries.
 emb_status emb_enq_link_split(const EmbLevel &lv, const uint32_t *work, const uint32_t *work_n, const uint64_t *cand,
                               const uint32_t *blk_off, const uint32_t *bin_off, uint2 *witem, uint2 *extra,
-                              unsigned long long *extra_n, uint32_t extra_cap, cudaStream_t s)
+                              unsigned long long *queue, uint32_t extra_cap, int64_t *d_count, cudaStream_t s)
 {
-    EMB_CUDA_TRY(cudaMemsetAsync(extra_n, 0, sizeof(unsigned long long), s));
+    EMB_CUDA_TRY(cudaMemsetAsync(queue, 0, 2 * sizeof(unsigned long long), s));
     if (lv.n > 0)
         EMB_LAUNCH((k_link_split), emb_grid(lv.n, 256), 256, 0, s)(work, work_n, cand, blk_off, bin_off, lv.n, witem,
-                                                                   extra, extra_n, extra_cap);
+                                                                   extra, queue, extra_cap, d_count);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
@@ -1054,12 +1117,14 @@ emb_status emb_link_emit_init()
     return EMB_OK;
 }
 
-// One persistent launch over the meshes of `tab`; `next` is the queue cursor.
+// One persistent launch over the meshes of `tab`; `next` is the queue cursor (cleared here
+// unless the caller has).
 // The grid fills every SM (ctas_per_sm resident CTAs each, 0 = as many as fit)
 // unless the work is smaller: with `items` > 0 (the blocks with links, known to
 // the caller) it stops at about items_per_warp items per warp, so that a small
 // mesh leaves SMs to the kernels of other streams.
-emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, int ctas_per_sm, cudaStream_t s, int64_t items)
+emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, bool zeroed, int ctas_per_sm, cudaStream_t s,
+                             int64_t items)
 {
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
@@ -1073,7 +1138,7 @@ emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, int ctas_
         const int64_t need = (items + LE_WARPS * items_per_warp - 1) / (LE_WARPS * items_per_warp);
         if (need < grid) grid = need;
     }
-    EMB_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(unsigned int), s));
+    if (!zeroed) EMB_CUDA_TRY(cudaMemsetAsync(next, 0, sizeof(unsigned int), s));
     EMB_LAUNCH((k_link_emit), (int)grid, LE_WARPS * 32, smem, s)(tab, next, st);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
@@ -1101,19 +1166,15 @@ static emb_status build_candidates(emb_forest f, int lattice, cudaStream_t s, bo
     free_candidates(f, s);
     EMB_CUDA_TRY(emb_malloc_async(&f->cand, (lv.n * 26 + 1) * sizeof(uint64_t), s));
     EMB_CUDA_TRY(emb_malloc_async(&f->blk_off, (lv.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&f->work_n, (lv.n + 1) * sizeof(uint32_t), s));
     EMB_CUDA_TRY(emb_malloc_async(&f->work, (lv.n + 1) * sizeof(uint32_t), s));
-    if (!f->next) EMB_CUDA_TRY(cudaMalloc(&f->next, sizeof(unsigned int)));
-    uint32_t *cnt = nullptr, *flag = nullptr;
-    uint64_t *tmp = nullptr;
-    EMB_CUDA_TRY(emb_malloc_async(&cnt, (lv.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&flag, (lv.n + 1) * sizeof(uint32_t), s));
-    EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(lv.n) * sizeof(uint64_t), s));
-    rc = emb_enq_link_prep(lv, lattice, f->cand, cnt, flag, f->work_n, f->work, f->blk_off, tmp, s);
+    f->work_n = f->work + lv.n;
+    const size_t a_state = (size_t)emb_link_state_words(lv.n) * sizeof(uint64_t);
+    char *scratch = nullptr;
+    EMB_CUDA_TRY(emb_malloc_async(&scratch, a_state + (lv.n + 1) * sizeof(uint32_t), s));
+    rc = emb_enq_link_prep(lv, lattice, f->cand, (uint32_t *)(scratch + a_state), f->work_n, f->work, f->blk_off,
+                           (uint64_t *)scratch, s);
     if (rc != EMB_OK) return rc;
-    EMB_CUDA_TRY(cudaFreeAsync(cnt, s));
-    EMB_CUDA_TRY(cudaFreeAsync(flag, s));
-    EMB_CUDA_TRY(cudaFreeAsync(tmp, s));
+    EMB_CUDA_TRY(cudaFreeAsync(scratch, s));
     f->cand_lattice = lattice;
     f->n_links = EMB_LINKS_ON_DEVICE;
     if (!read_count) return EMB_OK;
@@ -1181,7 +1242,10 @@ extern "C" emb_status emb_cutlinks(emb_forest f, emb_bins b, int32_t lattice, in
     emb_status rc = build_candidates(f, lattice, s, false);
     if (rc != EMB_OK) return rc;
     EmbLevel &lv = f->lv[f->max_level];
-    if (d_count) EMB_LAUNCH((k_store_count), 1, 32, 0, s)(f->blk_off, lv.n, d_count);
+    // the count: with the work items where there are any, else by itself
+    const bool split = !(f->n_links >= 0 && f->n_links > capacity) && f->n_links != 0 && capacity != 0;
+    if (d_count && !(split && d_cell && d_dir && d_q && d_tri))
+        EMB_LAUNCH((k_store_count), 1, 32, 0, s)(f->blk_off, lv.n, d_count);
     if (f->n_links >= 0 && f->n_links > capacity) {
         EMB_LAUNCH((k_set_status), 1, 1, 0, s)(st, EMB_ERR_CAPACITY);
         EMB_CUDA_TRY(cudaGetLastError());
@@ -1206,7 +1270,7 @@ extern "C" emb_status emb_cutlinks(emb_forest f, emb_bins b, int32_t lattice, in
     M.ent_cap = (uint64_t)b->npairs;  // complete after emb_bins_sync
     M.rec = b->m->rec;
     M.T = (uint32_t)b->m->T;
-    M.work_n = f->work_n + lv.n;
+    M.work_n = f->work_n;
     M.o_cell = d_cell;
     M.o_dir = d_dir;
     M.o_q = d_q;
@@ -1222,14 +1286,14 @@ extern "C" emb_status emb_cutlinks(emb_forest f, emb_bins b, int32_t lattice, in
     unsigned long long *xn = (unsigned long long *)sp;
     uint2 *witem = (uint2 *)(sp + 256);
     uint2 *extra = (uint2 *)(sp + 256 + a_w);
-    rc = emb_enq_link_split(lv, f->work, f->work_n + lv.n, f->cand, f->blk_off, b->off, witem, extra, xn, (uint32_t)xcap,
+    rc = emb_enq_link_split(lv, f->work, f->work_n, f->cand, f->blk_off, b->off, witem, extra, xn, (uint32_t)xcap, d_count,
                             s);
     if (rc == EMB_OK) {
         M.witem = witem;
         M.extra = extra;
         M.extra_n = xn;
         M.extra_cap = (uint32_t)xcap;
-        rc = emb_enq_link_emit(tab, f->next, 0, s, 0);
+        rc = emb_enq_link_emit(tab, (unsigned int *)(xn + 1), true, 0, s, 0);
     }
     cudaFreeAsync(sp, s);
     if (rc != EMB_OK) return rc;

@@ -169,8 +169,6 @@ extern "C" void emb_forest_destroy(emb_forest f)
     if (f->cand) cudaFree(f->cand);
     if (f->blk_off) cudaFree(f->blk_off);
     if (f->work) cudaFree(f->work);
-    if (f->work_n) cudaFree(f->work_n);
-    if (f->next) cudaFree(f->next);
     emb_readback_release(f->rb_slot);
     delete f;
 }
@@ -296,10 +294,7 @@ extern "C" emb_status emb_forest_refine(emb_forest f, int32_t level, const uint8
         cudaFreeAsync(f->work, s);
         f->work = nullptr;
     }
-    if (f->work_n) {
-        cudaFreeAsync(f->work_n, s);
-        f->work_n = nullptr;
-    }
+    f->work_n = nullptr;
     f->n_links = -1;
     return EMB_OK;
 }

@@ -77,9 +77,9 @@ struct emb_mesh_s {
     int64_t V, T;
     int4 *rec;      // T x 3 records {X, Y, Z, vertex id}
     int device;
-    // largest extent of a triangle per axis (frame units); not known once the vertices
+    // largest extent of a triangle along an axis (frame units); not known once the vertices
     // have moved (emb_mesh_update)
-    int32_t ext[3];
+    int32_t ext;
     bool ext_known;
 };
 
@@ -142,9 +142,8 @@ struct emb_forest_s {
     // cut-link candidates at the finest level (built by emb_cutlinks_count / emb_cutlinks)
     uint64_t *cand = nullptr;     // per finest block x 26 directions: fluid cells whose neighbour along c_d is solid
     uint32_t *blk_off = nullptr;  // per finest block: exclusive link offset (n+1 entries)
-    uint32_t *work = nullptr;     // ids of finest blocks with at least one link; count at work_n[0]
-    uint32_t *work_n = nullptr;
-    unsigned int *next = nullptr; // work-queue cursor of the persistent link kernel
+    uint32_t *work = nullptr;     // ids of finest blocks with at least one link; their count at work_n
+    uint32_t *work_n = nullptr;   // (inside the allocation of `work`)
     int32_t cand_lattice = 0;
     int64_t n_links = -1;
     int device;
@@ -256,11 +255,13 @@ int64_t emb_filter_state_words(int64_t T);
 emb_status emb_enq_filter(const int4 *rec, int64_t T, LevelGeom g, uint32_t *flist, uint32_t *count, uint32_t *word,
                           uint64_t *state, bool zeroed, int block, cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
 struct EmbBigQ;
-emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbLevel &lv, uint32_t *cnt, uint32_t *off,
-                             uint2 *list_bs, uint32_t *list_tri, unsigned long long *list_n, uint64_t list_cap,
-                             uint64_t *tmp, const EmbBigQ &Q, cudaStream_t s, uint64_t expect = EMB_NO_EXPECT);
-emb_status emb_enq_bin_scatter(const uint2 *list_bs, const uint32_t *list_tri, const unsigned long long *list_n,
-                               uint64_t list_cap, const uint32_t *off, uint32_t *ent, uint64_t ent_cap, cudaStream_t s);
+int64_t emb_bin_words(int64_t n);
+emb_status emb_enq_bin_pairs(const int4 *rec, int64_t T, LevelGeom g, const EmbLevel &lv, uint64_t *z, uint32_t *off,
+                             uint2 *list_bs, uint32_t *list_tri, uint64_t list_cap, const EmbBigQ &Q, cudaStream_t s,
+                             uint64_t expect = EMB_NO_EXPECT, uint32_t *d_total = nullptr);
+emb_status emb_enq_bin_scatter(const EmbLevel &lv, uint64_t *z, const uint2 *list_bs, const uint32_t *list_tri,
+                               uint64_t list_cap, const uint32_t *off, uint32_t *ent, uint64_t ent_cap,
+                               unsigned long long *d_req, bool check, cudaStream_t s);
 int64_t emb_vox_words(int64_t n);
 emb_status emb_enq_voxelize(const int4 *rec, int64_t T, const uint32_t *flist, int64_t nf, const uint32_t *d_nf,
                             const uint32_t *keep, LevelGeom g, const EmbLevel &lv, uint64_t *acc, uint64_t *mask_out,
@@ -301,14 +302,17 @@ struct LinkTable {
     int n;
     LinkMesh m[EMB_MAX_BATCH];
 };
-emb_status emb_enq_link_prep(const EmbLevel &lv, int lattice, uint64_t *cand, uint32_t *cnt, uint32_t *flag,
-                             uint32_t *work_n, uint32_t *work, uint32_t *blk_off, uint64_t *tmp, cudaStream_t s,
+int64_t emb_link_state_words(int64_t n);
+emb_status emb_enq_link_prep(const EmbLevel &lv, int lattice, uint64_t *cand, uint32_t *cnt, uint32_t *work_n,
+                             uint32_t *work, uint32_t *blk_off, uint64_t *state, cudaStream_t s,
                              uint64_t expect_work = EMB_NO_EXPECT, uint64_t expect_links = EMB_NO_EXPECT);
+// queue: two words, cleared here: the requests for extra entries, and the cursor of the
+// link kernel of one mesh (queue + 1)
 emb_status emb_enq_link_split(const EmbLevel &lv, const uint32_t *work, const uint32_t *work_n, const uint64_t *cand,
                               const uint32_t *blk_off, const uint32_t *bin_off, uint2 *witem, uint2 *extra,
-                              unsigned long long *extra_n, uint32_t extra_cap, cudaStream_t s);
+                              unsigned long long *queue, uint32_t extra_cap, int64_t *d_count, cudaStream_t s);
 int64_t emb_link_extra_capacity(int64_t n);
-emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, int ctas_per_sm, cudaStream_t s,
+emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, bool zeroed, int ctas_per_sm, cudaStream_t s,
                              int64_t items);
 emb_status emb_link_emit_init();
 size_t emb_link_emit_smem();
@@ -610,15 +614,13 @@ __device__ __forceinline__ unsigned long long emb_bigq_count(const EmbBigQ &Q)
     return n < Q.cap ? n : Q.cap;
 }
 
-// Host side (emb_common.cu): capacity for T triangles (0 when no triangle can have more than
-// EMB_BIG_ITEMS items, `items` being the most one can have: no queue and no chunk kernel),
-// allocation, per-launch reset.
-static inline long long emb_mesh_items(const emb_mesh_s *m, long long a, long long b, long long c)
+// Host side: entries for T triangles; whether a triangle may have more than EMB_BIG_ITEMS
+// items when none has more than a x b x c (no queue and no chunk kernel otherwise: 2 us and
+// a launch each).
+static inline bool emb_mesh_big(const emb_mesh_s *m, long long a, long long b, long long c)
 {
-    return m->ext_known ? a * b * c : EMB_BIG_ITEMS + 1;
+    return !m->ext_known || a * b * c > EMB_BIG_ITEMS;
 }
 int64_t emb_bigq_capacity(int64_t T);
-emb_status emb_bigq_alloc(EmbBigQ &Q, int64_t T, cudaStream_t s);  // stream-ordered
-void emb_bigq_free(EmbBigQ &Q, cudaStream_t s);
 #define EMB_BIG_GRID 1216   // CTAs of the chunk kernels (8 per SM on 152 SMs)
 #define EMB_BIG_BLOCK 128

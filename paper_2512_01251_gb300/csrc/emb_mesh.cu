@@ -2,7 +2,6 @@
 // triangle records, and the watertightness check on the GPU.
 #include <limits.h>
 #include <stdlib.h>
-#include <string.h>
 
 #include "emb_internal.cuh"
 
@@ -75,13 +74,15 @@ __device__ __forceinline__ bool edge_enter(const EdgeTable &E, uint32_t a, uint3
     return false;
 }
 
-// Records, the largest extents, and with E.done the edges (a thread per triangle).
+// Records, the largest extent, and with E.done the edges (a thread per triangle).
 __global__ void k_mesh_records(const float *__restrict__ verts, const int32_t *__restrict__ tris, int64_t V, int64_t T,
                                int32_t r_o, int4 *__restrict__ rec, EdgeTable E, int *ext, int *err)
 {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int bad = 0;
     uint32_t done = 0;
+    // few warps raise the extent: what it was on entry, read while the vertices are fetched
+    const int seen = *(volatile int *)ext;
     int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {0, 0, 0};
     if (t < T) {
         int32_t vid[3];
@@ -114,12 +115,11 @@ __global__ void k_mesh_records(const float *__restrict__ verts, const int32_t *_
         }
         if (bad) atomicOr(err, bad);
     }
+    int e = 0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const int e = __reduce_max_sync(0xffffffffu, hi[d] >= lo[d] ? hi[d] - lo[d] : 0);
-        // few warps raise it: a read first
-        if ((threadIdx.x & 31) == 0 && e > *(volatile int *)(ext + d)) atomicMax(ext + d, e);
-    }
+    for (int d = 0; d < 3; ++d) e = max(e, hi[d] - lo[d]);
+    e = __reduce_max_sync(0xffffffffu, t < T && !(bad & MESH_ERR_ID) ? e : 0);
+    if ((threadIdx.x & 31) == 0 && e > seen) atomicMax(ext, e);
     if (E.done) {
         done = __reduce_add_sync(0xffffffffu, done);
         if ((threadIdx.x & 31) == 0 && done) atomicAdd(E.done + blockIdx.x % EDGE_COUNTERS, done);
@@ -176,10 +176,10 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
     m->V = V;
     m->T = T;
     cudaGetDevice(&m->device);
-    // error word, completion counters and extents, then the edge table: cleared together
+    // error word, completion counters and extent, then the edge table: cleared together
     char *scratch = nullptr;
     emb_status rc = EMB_OK;
-    uint32_t head[1 + EDGE_COUNTERS + 3] = {0};
+    uint32_t head[1 + EDGE_COUNTERS + 1] = {0};
     const size_t a_head = 512;
     // room for every edge in a small mesh's overflow table (a triangle has 3/2); in a large
     // one for a third of them (a few percent overflow, more where a few vertices have many
@@ -224,7 +224,7 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
         for (int i = 0; i < EDGE_COUNTERS; ++i) closed += head[1 + i];
         if (2 * closed != 3 * T) head[0] |= MESH_ERR_OPEN_EDGE;
     }
-    memcpy(m->ext, head + 1 + EDGE_COUNTERS, sizeof(m->ext));
+    m->ext = (int32_t)head[1 + EDGE_COUNTERS];
     m->ext_known = true;
     if (head[0] & (MESH_ERR_ID | MESH_ERR_SNAP)) rc = EMB_ERR_BAD_INPUT;
     else if (head[0]) rc = EMB_ERR_NOT_WATERTIGHT;

@@ -377,9 +377,9 @@ extern "C" emb_status emb_refine_flags(emb_forest f, emb_bins b, int32_t level, 
     // EMB_BIG_ITEMS dilated blocks: [-dil, extent + dil] spans at most this many an axis
     const emb_mesh m = b->m;
     const LevelGeom g = level_geom(f, level);
-    auto span = [&](int d) { return ((m->ext[d] + 2 * dil) >> g.lW) + 2; };
+    const long long span = ((m->ext + 2 * dil) >> g.lW) + 2;
     EmbBigQ Q = {nullptr, nullptr, 0};
-    if (emb_mesh_items(m, span(0), span(1), span(2)) > EMB_BIG_ITEMS) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
+    if (emb_mesh_big(m, span, span, span)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
     const size_t a_bits = ((size_t)(nw + 1) * sizeof(unsigned long long) + 255) & ~(size_t)255;
     char *scratch = nullptr;

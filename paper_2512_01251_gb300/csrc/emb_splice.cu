@@ -280,7 +280,6 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
     if (f->cand) cudaFreeAsync(f->cand, s);
     if (f->blk_off) cudaFreeAsync(f->blk_off, s);
     if (f->work) cudaFreeAsync(f->work, s);
-    if (f->work_n) cudaFreeAsync(f->work_n, s);
     f->cand = nullptr;
     f->blk_off = nullptr;
     f->work = nullptr;

@@ -291,8 +291,7 @@ extern "C" emb_status emb_voxelize(emb_forest f, emb_bins b, int32_t level, uint
     // entries of the chunk queue
     const emb_mesh m = b->m;
     EmbBigQ Q = {nullptr, nullptr, 0};
-    if (emb_mesh_items(m, 1, (m->ext[1] >> g.lh) + 1, (m->ext[2] >> g.lh) + 1) > EMB_BIG_ITEMS)
-        Q.cap = (uint32_t)emb_bigq_capacity(m->T);
+    if (emb_mesh_big(m, 1, (m->ext >> g.lh) + 1, (m->ext >> g.lh) + 1)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const size_t a_acc = ((size_t)emb_vox_words(lv.n) * sizeof(uint64_t) + 255) & ~(size_t)255;
     char *scratch = nullptr;
     EMB_CUDA_TRY(emb_malloc_async(&scratch, a_acc + (size_t)Q.cap * sizeof(uint2), s));
