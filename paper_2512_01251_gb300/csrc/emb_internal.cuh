@@ -441,12 +441,60 @@ __device__ __forceinline__ float i128_to_float(i128 v)
     return (float)hi * 18446744073709551616.0f + (float)lo;
 }
 
+// emb_tri_box for vertices and a box edge within 2^14 of the box's low corner (a block and
+// its triangles on all but the coarsest frames): edge vectors stay within 2^15, the edge
+// axes' projections within 2 * 2^15 * 2^14 = 2^30 and are formed in 32 bits; the face
+// normal (2^31) and its projections (3 * 2^45) in 64.  (All in 64 and 128 bits, the finest
+// level's pair kernel took 757 us on 7.2M triangles, now 590.)
+static __device__ __forceinline__ bool emb_tri_box32(const int (&v)[3][3], const int (&E)[3])
+{
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        if (min(v[0][d], min(v[1][d], v[2][d])) > E[d] || max(v[0][d], max(v[1][d], v[2][d])) < 0) return false;
+    int f[3][3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        f[0][d] = v[1][d] - v[0][d];
+        f[1][d] = v[2][d] - v[1][d];
+        f[2][d] = v[0][d] - v[2][d];
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            // axis e_d x f_j: nonzero components -f_j[w] along u and f_j[u] along w
+            const int u = (d + 1) % 3, w = (d + 2) % 3, au = -f[j][w], aw = f[j][u];
+            // the two ends of edge j project to the same value
+            const int p = au * v[j][u] + aw * v[j][w], o = au * v[(j + 2) % 3][u] + aw * v[(j + 2) % 3][w];
+            const int tu = au * E[u], tw = aw * E[w];
+            if (max(p, o) < min(tu, 0) + min(tw, 0) || min(p, o) > max(tu, 0) + max(tw, 0)) return false;
+        }
+    }
+    // face normal: the triangle projects to the single value n.v0
+    const long long n0 = (long long)f[0][1] * f[1][2] - (long long)f[0][2] * f[1][1];
+    const long long n1 = (long long)f[0][2] * f[1][0] - (long long)f[0][0] * f[1][2];
+    const long long n2 = (long long)f[0][0] * f[1][1] - (long long)f[0][1] * f[1][0];
+    const long long p = n0 * v[0][0] + n1 * v[0][1] + n2 * v[0][2];
+    const long long t0 = n0 * E[0], t1 = n1 * E[1], t2 = n2 * E[2];
+    return p >= min(t0, 0ll) + min(t1, 0ll) + min(t2, 0ll) && p <= max(t0, 0ll) + max(t1, 0ll) + max(t2, 0ll);
+}
+
 // Exact overlap of a triangle with the closed box [lo, hi] (separating axes:
 // the box normals, the face normal and the 9 edge x axis products), computed
 // in coordinates relative to the box's low corner.
 static __device__ __noinline__ bool emb_tri_box(const int4 &A, const int4 &B, const int4 &C, long long lx, long long ly,
                                             long long lz, long long hx, long long hy, long long hz)
 {
+    {
+        // box corners lie within 2^26 of the frame: 32-bit differences
+        const int x = (int)lx, y = (int)ly, z = (int)lz, LIM = 1 << 14;
+        const int u[3][3] = {{A.x - x, A.y - y, A.z - z}, {B.x - x, B.y - y, B.z - z}, {C.x - x, C.y - y, C.z - z}};
+        const int F[3] = {(int)(hx - lx), (int)(hy - ly), (int)(hz - lz)};
+        int out = F[0] | F[1] | F[2];
+#pragma unroll
+        for (int j = 0; j < 3; ++j) out |= (u[j][0] + LIM) | (u[j][1] + LIM) | (u[j][2] + LIM);
+        if (!(out & ~(2 * LIM - 1)) && max(F[0], max(F[1], F[2])) <= LIM) return emb_tri_box32(u, F);
+    }
     long long v[3][3] = {{A.x - lx, A.y - ly, A.z - lz}, {B.x - lx, B.y - ly, B.z - lz}, {C.x - lx, C.y - ly, C.z - lz}};
     long long E[3] = {hx - lx, hy - ly, hz - lz};
 #pragma unroll
