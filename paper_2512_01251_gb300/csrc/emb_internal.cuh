@@ -573,14 +573,9 @@ __device__ __forceinline__ void line_range(long long mn, long long mx, int lh, l
 // ---------------------------------------------------------------------------
 // warp-cooperative visit of (triangle, block) overlaps
 // ---------------------------------------------------------------------------
-// A warp takes 32 consecutive triangles (neighbours in a mesh's storage order
-// are usually neighbours in space) and stages them in shared memory.  The refine
-// kernel may form the union of the block ranges their dilated boxes can touch and
-// let each lane test whole blocks of that union against all 32 triangles, which
-// trades 32 independent lookups per candidate block for one; when the union is
-// large (above EMB_WU_MAX blocks) or loose (more than an eighth of the warp's
-// summed per-triangle candidates), and always in the finest-level binning, the
-// warp's (triangle, candidate block) pairs are spread evenly over its lanes instead.
+// A warp takes 32 consecutive triangles (neighbours in a mesh's storage order are usually
+// neighbours in space).  In the finest-level binning it stages them in shared memory and
+// spreads their (triangle, candidate block) pairs evenly over its lanes.
 #define EMB_WU_WARPS 4
 // Division by a per-triangle divisor d >= 1 in the pair-spreading loops, through its
 // reciprocal m = ceil(2^32 / d) (emb_recip, once per triangle): q = floor(r m / 2^32)
@@ -593,23 +588,10 @@ __device__ __forceinline__ uint32_t emb_div_recip(uint32_t r, uint32_t d, uint32
     q -= (uint32_t)(q * d > r);
     return d > 1u ? q : r;
 }
-#define EMB_WU_MAX 2048
 
 struct WuTri {
     int4 A[32], B[32], C[32];
-    int lo[3][32], hi[3][32];
 };
-
-// Overlap of triangle j of the tile with the closed box [l, u] (exact).
-__device__ __forceinline__ bool wu_overlap(const WuTri &S, int j, long long lx, long long ly, long long lz, long long ux,
-                                           long long uy, long long uz)
-{
-    if (S.lo[0][j] > ux || S.hi[0][j] < lx || S.lo[1][j] > uy || S.hi[1][j] < ly || S.lo[2][j] > uz || S.hi[2][j] < lz)
-        return false;
-    const int4 A = S.A[j], B = S.B[j], C = S.C[j];
-    return emb_point_in_box(A, lx, ly, lz, ux, uy, uz) || emb_point_in_box(B, lx, ly, lz, ux, uy, uz) ||
-           emb_point_in_box(C, lx, ly, lz, ux, uy, uz) || emb_tri_box(A, B, C, lx, ly, lz, ux, uy, uz);
-}
 
 // ---------------------------------------------------------------------------
 // work split of large triangles

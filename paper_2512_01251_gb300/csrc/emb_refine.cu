@@ -9,19 +9,20 @@
 // rho_L = max(band, rho_{L+1}/2 + 5/2), which keeps all 26 neighbours of every
 // refined block present (2:1 balance) and leaves unrefined blocks surface-free.
 //
-// Warp-cooperative over 32 consecutive triangles (see emb_internal.cuh): when the
-// union of their candidate blocks is at most an eighth of their summed candidates,
-// each block of the union is looked up once and tested against the 32 triangles;
-// otherwise the warp's (triangle, candidate block) pairs are spread evenly over its
-// lanes, and a triangle with very many candidates goes in queued chunks to whole
-// warps.  Flags are idempotent byte stores.
+// Warps over tiles of 32 consecutive triangles (details at k_refine); a triangle with very
+// many candidates goes in queued chunks to whole warps.  Flags are idempotent byte stores.
 #include <math.h>
+
+#include <atomic>
 
 #include "emb_internal.cuh"
 
+#define REFINE_WARPS 8
 #ifndef REFINE_MINB
 #define REFINE_MINB 4
 #endif
+// Largest bitmap (words) that a CTA of k_refine keeps a copy of: up to 64 blocks an axis.
+#define REFINE_SM_WORDS 4096
 
 __device__ __forceinline__ void refine_setup(const int4 *__restrict__ rec, int64_t t, const LevelGeom &g, long long dil,
                                              int4 &A, int4 &B, int4 &C, long long b0[3], long long b1[3])
@@ -41,66 +42,83 @@ __device__ __forceinline__ unsigned long long refine_items(const long long b0[3]
            (unsigned long long)(b1[2] - b0[2] + 1);
 }
 
-// Flagged blocks of the level as one bit per dense position (bx + nb (by + nb bz)),
-// when the level is small enough to have one: the common "already flagged" case
-// then costs one cached load instead of a block lookup and a flag load.
-struct FlagBits {
-    unsigned long long *w;  // null: no dense bits, test the flag bytes
+// Blocks of the level that are not flagged yet as one bit per dense position (bx + nb (by +
+// nb bz)), when the level has a rank bitmap: a copy of it, from which flagging clears bits.
+// One load tells a candidate that is missing or flagged from one that is left, and flagging
+// is one atomic that nothing waits for; k_refine_flags turns the bits into the flag bytes
+// afterwards.  w is in global memory, or for a small level in shared memory: a copy that the
+// CTA keeps and merges at its end, since every warp of the grid reads and clears the few
+// words of a coarse level (111K triangles on 16^3 blocks: 139 us through the L2).  A word
+// read before another warp cleared a bit only sends the candidate through the full test,
+// which decides exactly and flags once more.
+// Words of 32 bits: those have native atomics in shared memory, 64-bit ones a
+// compare-and-swap loop.
+struct TodoBits {
+    uint32_t *w;  // null: no dense bits, look the block up and test the flag bytes
     long long nb;
-    // A plain (L1-cached) load: a word cached before another SM set a bit only sends
-    // the candidate through the full test, which decides exactly.
-    __device__ __forceinline__ bool test(long long bx, long long by, long long bz, unsigned long long &pos) const
+    __device__ __forceinline__ unsigned long long pos(long long bx, long long by, long long bz) const
     {
-        pos = (unsigned long long)((bz * nb + by) * nb + bx);
-        return (w[pos >> 6] >> (pos & 63)) & 1ull;
+        return (unsigned long long)((bz * nb + by) * nb + bx);
     }
-    __device__ __forceinline__ void set(unsigned long long pos) const { atomicOr(w + (pos >> 6), 1ull << (pos & 63)); }
+    __device__ __forceinline__ bool test(long long bx, long long by, long long bz) const
+    {
+        const unsigned long long p = pos(bx, by, bz);
+        return (w[p >> 5] >> (p & 31)) & 1u;
+    }
+    __device__ __forceinline__ void clear(long long bx, long long by, long long bz) const
+    {
+        const unsigned long long p = pos(bx, by, bz);
+        atomicAnd(w + (p >> 5), ~(1u << (p & 31)));
+    }
+    // bits [0, nx) of the row segment from (bx, by, bz), nx <= 32
+    __device__ __forceinline__ uint32_t row(int bx, int by, int bz, int nx) const
+    {
+        const unsigned long long p = pos(bx, by, bz);
+        const int sh = (int)(p & 31);
+        const uint32_t lo = w[p >> 5], hi = sh + nx > 32 ? w[(p >> 5) + 1] : 0u;
+        return __funnelshift_r(lo, hi, sh) & (0xffffffffu >> (32 - nx));
+    }
 };
 
-// Id of block (bx, by, bz) if it exists and is not flagged yet, else -1; pos receives
-// its dense position.  With both dense bitmaps (flagged bits and the level's rank
-// bitmap) the flagged word, the existence word and its rank prefix are independent
-// loads issued together, and the flag byte is not read: a flagged word read before
-// another SM set the bit only sends the block through the exact test once more, whose
-// flag store is idempotent.  Otherwise: the flagged bit, the lookup, the flag byte.
-__device__ __forceinline__ int32_t refine_candidate(const EmbLookup &lk, const FlagBits &fb,
-                                                    const uint8_t *__restrict__ flags, long long bx, long long by,
-                                                    long long bz, unsigned long long &pos)
+// Block (bx, by, bz) is left to flag.
+__device__ __forceinline__ bool refine_left(const EmbLookup &lk, const TodoBits &td, const uint8_t *__restrict__ flags,
+                                            long long bx, long long by, long long bz)
 {
-    if (fb.w && lk.bits) {
-        pos = (unsigned long long)((bz * fb.nb + by) * fb.nb + bx);
-        if (!emb_ck(pos, (uint64_t)lk.nb * lk.nb * lk.nb, lk.st)) return -1;
-        const unsigned long long fw = fb.w[pos >> 6];
-        const uint64_t ew = __ldg(lk.bits + (pos >> 6));
-        const uint32_t pre = __ldg(lk.wpre + (pos >> 6));
-        const int sh = (int)(pos & 63);
-        if (((fw >> sh) & 1ull) || !((ew >> sh) & 1ull)) return -1;
-        const int32_t id = (int32_t)(pre + (uint32_t)__popcll(ew & ((1ull << sh) - 1ull)));
-        return emb_ck((uint64_t)id, (uint64_t)lk.n, lk.st) ? id : -1;
-    }
-    if (fb.w && fb.test(bx, by, bz, pos)) return -1;
+    if (td.w) return td.test(bx, by, bz);
     const int32_t id = emb_lookup(lk, bx, by, bz);
-    if (id < 0 || *((volatile const uint8_t *)flags + id)) return -1;
-    return id;
+    return id >= 0 && !*((volatile const uint8_t *)flags + id);
 }
 
-// Flag block (bx, by, bz) if it exists, is not flagged yet and the triangle meets its dilated box.
-__device__ __forceinline__ void refine_block(const int4 &A, const int4 &B, const int4 &C, long long bx, long long by,
-                                             long long bz, const LevelGeom &g, long long dil, const EmbLookup &lk,
-                                             uint8_t *__restrict__ flags, const FlagBits &fb)
+__device__ __forceinline__ void refine_flag(const EmbLookup &lk, const TodoBits &td, uint8_t *__restrict__ flags,
+                                            long long bx, long long by, long long bz)
 {
-    unsigned long long pos = 0;
-    const int32_t id = refine_candidate(lk, fb, flags, bx, by, bz, pos);
-    if (id < 0) return;
-    const long long lx = bx * g.W - dil, ly = by * g.W - dil, lz = bz * g.W - dil;
-    const long long hx = lx + g.W + 2 * dil, hy = ly + g.W + 2 * dil, hz = lz + g.W + 2 * dil;
-    if (emb_point_in_box(A, lx, ly, lz, hx, hy, hz) || emb_point_in_box(B, lx, ly, lz, hx, hy, hz) ||
-        emb_point_in_box(C, lx, ly, lz, hx, hy, hz) || emb_tri_box(A, B, C, lx, ly, lz, hx, hy, hz)) {
-        flags[id] = 1;
-        if (fb.w) fb.set(pos);
+    if (td.w) {
+        td.clear(bx, by, bz);
+        return;
     }
+    const int32_t id = emb_lookup(lk, bx, by, bz);
+    if (id >= 0) flags[id] = 1;
 }
 
+// The flag bytes of a level with the bitmap: the blocks whose bit was cleared (none of the
+// entries past a replay's count).
+__global__ void k_refine_flags(const uint64_t *__restrict__ key, int64_t n, const uint32_t *d_n,
+                               const uint32_t *__restrict__ todo, int64_t nb, uint8_t *__restrict__ flags)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    uint8_t f = 0;
+    if (i < emb_count(n, d_n)) {
+        const uint64_t k = key[i];
+        const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
+                      bz = (int64_t)(k >> (2 * EMB_KEY_BITS));
+        if (bx < nb && by < nb && bz < nb) {
+            const int64_t pos = (bz * nb + by) * nb + bx;
+            f = (uint8_t)(((todo[pos >> 5] >> (pos & 31)) & 1u) ^ 1u);
+        }
+    }
+    flags[i] = f;
+}
 
 // 32-bit forms of the per-block arithmetic: coordinates, block origins, widths and
 // dilations all lie below 2^25 in magnitude, block indices below 2^21.
@@ -115,43 +133,62 @@ __device__ __forceinline__ bool ref_pt(const int4 &P, int lx, int ly, int lz, in
 {
     return P.x >= lx && P.x <= hx && P.y >= ly && P.y <= hy && P.z >= lz && P.z <= hz;
 }
-__device__ __forceinline__ bool ref_overlap(const WuTri &S, int j, int lx, int ly, int lz, int ux, int uy, int uz)
+// (triangle lane, bx, by, bz) of candidates none of whose vertices lies in the dilated block,
+// waiting for the separating-axis test.
+struct RefWarp {
+    int4 A[32], B[32], C[32];
+    int4 q[64];
+};
+
+// The separating-axis test of the last n queued candidates, one a lane; a block flagged in
+// the meantime is passed over.
+__device__ __forceinline__ void ref_drain(RefWarp &S, int &qn, int n, int lane, int W, int dil, const EmbLookup &lk,
+                                          const TodoBits &td, uint8_t *__restrict__ flags)
 {
-    if (S.lo[0][j] > ux || S.hi[0][j] < lx || S.lo[1][j] > uy || S.hi[1][j] < ly || S.lo[2][j] > uz || S.hi[2][j] < lz)
-        return false;
-    const int4 A = S.A[j], B = S.B[j], C = S.C[j];
-    return ref_pt(A, lx, ly, lz, ux, uy, uz) || ref_pt(B, lx, ly, lz, ux, uy, uz) || ref_pt(C, lx, ly, lz, ux, uy, uz) ||
-           emb_tri_box(A, B, C, lx, ly, lz, ux, uy, uz);
-}
-__device__ __forceinline__ void ref_block(const int4 &A, const int4 &B, const int4 &C, int bx, int by, int bz, int W,
-                                          int dil, const EmbLookup &lk, uint8_t *__restrict__ flags, const FlagBits &fb)
-{
-    unsigned long long pos = 0;
-    const int32_t id = refine_candidate(lk, fb, flags, bx, by, bz, pos);
-    if (id < 0) return;
-    const int lx = bx * W - dil, ly = by * W - dil, lz = bz * W - dil;
-    const int hx = lx + W + 2 * dil, hy = ly + W + 2 * dil, hz = lz + W + 2 * dil;
-    if (ref_pt(A, lx, ly, lz, hx, hy, hz) || ref_pt(B, lx, ly, lz, hx, hy, hz) || ref_pt(C, lx, ly, lz, hx, hy, hz) ||
-        emb_tri_box(A, B, C, lx, ly, lz, hx, hy, hz)) {
-        flags[id] = 1;
-        if (fb.w) fb.set(pos);
+    __syncwarp();
+    if (lane < n) {
+        const int4 e = S.q[qn - n + lane];
+        if (refine_left(lk, td, flags, e.y, e.z, e.w)) {
+            const int lx = e.y * W - dil, ly = e.z * W - dil, lz = e.w * W - dil, w = W + 2 * dil;
+            if (emb_tri_box(S.A[e.x], S.B[e.x], S.C[e.x], lx, ly, lz, lx + w, ly + w, lz + w))
+                refine_flag(lk, td, flags, e.y, e.z, e.w);
+        }
     }
+    qn -= n;
+    __syncwarp();
 }
 
-// Persistent warps over tiles of 32 consecutive triangles; each warp loads the
-// records of its next tile before it works on the current one, so that the loads
-// are in flight during the work (a warp otherwise spends most of its life after its
-// loads, in dependent lookups, and the record stream runs far below HBM speed).
-__global__ void __launch_bounds__(EMB_WU_WARPS * 32, REFINE_MINB) k_refine(const int4 *__restrict__ rec, int64_t T, LevelGeom g,
+// Persistent CTAs, each over consecutive tiles of 32 consecutive triangles (so that the
+// blocks it meets are few and soon flagged); each warp loads the records of its next tile
+// before it works on the current one.  A tile is screened first: the rows of the union of its
+// candidate blocks, one a lane, show in one load each which of them are left to flag; in a
+// large mesh there is none for most tiles, or only where no lane's own candidates reach (the
+// union is a box).  Otherwise every lane goes through the blocks left
+// among its own triangle's candidates: a vertex in the dilated block flags it, else the
+// pair waits for the separating-axis test, which the warp runs 32 at a time.
+// Latency-bound; four CTAs an SM (64 registers) over three: 5 % on 7.2M triangles.  Time over
+// the levels, before (the union's or the spread pairs' blocks looked up and tested at once,
+// global flag bits) and now: 7.2M triangles 1311 -> 899 us, 1.0M 311 -> 229, 111K 118 -> 91.
+// Taking the union's blocks left one at a time for the whole warp is slower on most levels
+// (986 us, 111K: 154).
+template <bool SM>
+__global__ void __launch_bounds__(REFINE_WARPS * 32, REFINE_MINB) k_refine(const int4 *__restrict__ rec, int64_t T, LevelGeom g,
                                                               long long dil, EmbLookup lk, uint8_t *__restrict__ flags,
-                                                              FlagBits fb, EmbBigQ Q)
+                                                              uint32_t *todo, int nw, int64_t chunk, EmbBigQ Q)
 {
-    __shared__ WuTri tiles[EMB_WU_WARPS];
+    extern __shared__ __align__(16) unsigned char ref_smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WuTri &S = tiles[w];
-    const int64_t ntiles = (T + 31) / 32;
-    const int64_t stride = (int64_t)gridDim.x * EMB_WU_WARPS;
-    int64_t tile = (int64_t)blockIdx.x * EMB_WU_WARPS + w;
+    RefWarp &S = reinterpret_cast<RefWarp *>(ref_smem)[w];
+    uint32_t *const s_todo = (uint32_t *)(ref_smem + REFINE_WARPS * sizeof(RefWarp));
+    if (SM) {
+        for (int i = threadIdx.x; i < nw; i += REFINE_WARPS * 32) s_todo[i] = __ldcg(todo + i);
+        __syncthreads();
+    }
+    const TodoBits td = {SM ? s_todo : todo, g.nb};
+    const int64_t first = (int64_t)blockIdx.x * chunk, all = (T + 31) / 32;
+    const int64_t ntiles = first + chunk < all ? first + chunk : all, stride = REFINE_WARPS;
+    int64_t tile = first + w;
+    const int dil32 = (int)dil, W32 = (int)g.W, nb32 = (int)g.nb;
     int4 nA = make_int4(0, 0, 0, 0), nB = nA, nC = nA;
     if (tile < ntiles && tile * 32 + lane < T) {
         const int64_t t = tile * 32 + lane;
@@ -161,7 +198,6 @@ __global__ void __launch_bounds__(EMB_WU_WARPS * 32, REFINE_MINB) k_refine(const
     }
     for (; tile < ntiles; tile += stride) {
         const int64_t t = tile * 32 + lane;
-        const bool valid = t < T;
         const int4 A = nA, B = nB, C = nC;
         {
             const int64_t tn = (tile + stride) * 32 + lane;
@@ -171,117 +207,130 @@ __global__ void __launch_bounds__(EMB_WU_WARPS * 32, REFINE_MINB) k_refine(const
                 nC = rec[3 * tn + 2];
             }
         }
-        const int dil32 = (int)dil, W32 = (int)g.W, nb32 = (int)g.nb;
         int b0[3] = {0x7fffffff, 0x7fffffff, 0x7fffffff}, b1[3] = {-1, -1, -1};
-        if (valid) {
+        if (t < T) {
             ref_range(min(A.x, min(B.x, C.x)), max(A.x, max(B.x, C.x)), g.lW, dil32, nb32, b0[0], b1[0]);
             ref_range(min(A.y, min(B.y, C.y)), max(A.y, max(B.y, C.y)), g.lW, dil32, nb32, b0[1], b1[1]);
             ref_range(min(A.z, min(B.z, C.z)), max(A.z, max(B.z, C.z)), g.lW, dil32, nb32, b0[2], b1[2]);
         }
-        __syncwarp();  // the previous tile's lanes are done with S
-        S.A[lane] = A;
-        S.B[lane] = B;
-        S.C[lane] = C;
-        S.lo[0][lane] = valid ? min(A.x, min(B.x, C.x)) : 0x7fffffff;
-        S.hi[0][lane] = valid ? max(A.x, max(B.x, C.x)) : -0x7fffffff;
-        S.lo[1][lane] = min(A.y, min(B.y, C.y));
-        S.hi[1][lane] = max(A.y, max(B.y, C.y));
-        S.lo[2][lane] = min(A.z, min(B.z, C.z));
-        S.hi[2][lane] = max(A.z, max(B.z, C.z));
-        __syncwarp();
-        int u0[3], u1[3];
+        int u0[3], un[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             u0[d] = __reduce_min_sync(0xffffffffu, b0[d]);
-            u1[d] = __reduce_max_sync(0xffffffffu, b1[d]);
+            un[d] = __reduce_max_sync(0xffffffffu, b1[d]) - u0[d] + 1;
         }
-        const long long nx = u1[0] - u0[0] + 1, ny = u1[1] - u0[1] + 1, nz = u1[2] - u0[2] + 1;
-        if (nx <= 0 || ny <= 0 || nz <= 0) continue;
-        const long long total = nx * ny * nz;
-        // per-triangle candidates summed over the warp: the union pays off only when it is
-        // much smaller (eight times: measured against two and four, and against sixteen)
-        const unsigned long long own =
-            valid && b1[0] >= b0[0] && b1[1] >= b0[1] && b1[2] >= b0[2]
-                ? (unsigned long long)(b1[0] - b0[0] + 1) * (unsigned long long)(b1[1] - b0[1] + 1) *
-                      (unsigned long long)(b1[2] - b0[2] + 1)
-                : 0ull;
-        const unsigned own_sum = __reduce_add_sync(0xffffffffu, (unsigned)min(own, 1ull << 20));
-        if (total <= EMB_WU_MAX && 8 * total <= (long long)own_sum) {
-            // total <= EMB_WU_MAX: decode the union index in 32-bit arithmetic.  Each lane
-            // takes a union block; the blocks that exist and are not flagged yet are then
-            // tested one at a time by the whole warp, each lane against its own triangle.
-            const unsigned ux = (unsigned)nx, uxy = (unsigned)(nx * ny);
-            const unsigned mx = emb_recip(ux), mxy = emb_recip(uxy);
-            for (unsigned c0 = 0; c0 < (unsigned)total; c0 += 32) {
-                const unsigned c = c0 + lane;
-                int bx = 0, by = 0, bz = 0;
-                unsigned long long pos = 0;
-                int32_t id = -1;
-                if (c < (unsigned)total) {
-                    const unsigned cz = emb_div_recip(c, uxy, mxy), cr = c - cz * uxy, cy = emb_div_recip(cr, ux, mx);
-                    bx = u0[0] + (int)(cr - cy * ux);
-                    by = u0[1] + (int)cy;
-                    bz = u0[2] + (int)cz;
-                    id = refine_candidate(lk, fb, flags, bx, by, bz, pos);
+        if (un[0] <= 0 || un[1] <= 0 || un[2] <= 0) continue;
+        bool may = true;  // a block left may be among the lane's candidates
+        if (td.w && un[0] <= 32 && un[1] <= 32 && un[2] <= 32) {
+            const unsigned ny = (unsigned)un[1], rows = ny * (unsigned)un[2], my = emb_recip(ny);
+            uint32_t xs = 0, ys = 0, zs = 0;  // where on the axes of the union there are any
+            for (unsigned r = lane; r < rows; r += 32) {
+                const unsigned rz = emb_div_recip(r, ny, my), ry = r - rz * ny;
+                const uint32_t m = td.row(u0[0], u0[1] + (int)ry, u0[2] + (int)rz, un[0]);
+                if (m) {
+                    xs |= m;
+                    ys |= 1u << ry;
+                    zs |= 1u << rz;
                 }
-                unsigned m = __ballot_sync(0xffffffffu, id >= 0);
-                while (m) {
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1;
-                    const int lx = __shfl_sync(0xffffffffu, bx, src) * W32 - dil32,
-                              ly = __shfl_sync(0xffffffffu, by, src) * W32 - dil32,
-                              lz = __shfl_sync(0xffffffffu, bz, src) * W32 - dil32;
-                    const bool hit = ref_overlap(S, lane, lx, ly, lz, lx + W32 + 2 * dil32, ly + W32 + 2 * dil32,
-                                                 lz + W32 + 2 * dil32);
-                    if (__any_sync(0xffffffffu, hit) && lane == src) {
-                        flags[id] = 1;
-                        if (fb.w) fb.set(pos);
+            }
+            xs = __reduce_or_sync(0xffffffffu, xs);
+            if (xs == 0u) continue;
+            ys = __reduce_or_sync(0xffffffffu, ys);
+            zs = __reduce_or_sync(0xffffffffu, zs);
+            auto in = [&](int d) {  // b0 <= b1 within the union: shifts of 0 .. 31
+                return b0[d] <= b1[d] ? (0xffffffffu >> (31 - (b1[d] - u0[d]))) & (0xffffffffu << (b0[d] - u0[d])) : 0u;
+            };
+            may = (xs & in(0)) && (ys & in(1)) && (zs & in(2));
+            if (!__any_sync(0xffffffffu, may)) continue;
+        }
+        const int onx = b1[0] - b0[0] + 1, ony = b1[1] - b0[1] + 1, onz = b1[2] - b0[2] + 1;
+        const unsigned long long own = t < T && onx > 0 && ony > 0 && onz > 0
+                                           ? (unsigned long long)onx * (unsigned long long)ony * (unsigned long long)onz
+                                           : 0ull;
+        const bool mine = may && own > 0 && !(own > EMB_BIG_ITEMS && emb_bigq_push(Q, (uint32_t)t, own));
+        S.A[lane] = A;  // the previous tile's queue was drained behind a warp barrier
+        S.B[lane] = B;
+        S.C[lane] = C;
+        int qn = 0;
+        // the lane's place in its candidates: a row (y, z) and, in it, the blocks from x on
+        int x = 0x7fffffff, y = b0[1] - 1, z = b0[2];
+        uint32_t m = 0;  // blocks left in the row segment from x (with the bitmap)
+        bool more = mine;
+        while (__any_sync(0xffffffffu, more)) {
+            bool need = false;
+            int bx = 0, by = 0, bz = 0;
+            while (more && !need) {
+                // the next candidate that is left to flag
+                bool have = false;
+                if (td.w) {
+                    if (m == 0) {
+                        // the next 32 blocks of the row, or the next row
+                        if (y >= b0[1] && x + 32 <= b1[0]) {
+                            x += 32;
+                        } else {
+                            x = b0[0];
+                            if (++y > b1[1]) {
+                                y = b0[1];
+                                ++z;
+                            }
+                        }
+                        if (z > b1[2]) {
+                            more = false;
+                            break;
+                        }
+                        m = td.row(x, y, z, min(32, b1[0] - x + 1));
                     }
+                    if (m) {
+                        const int i = __ffs(m) - 1;
+                        m &= m - 1;
+                        bx = x + i;
+                        have = true;
+                    }
+                } else {
+                    if (y < b0[1] || ++x > b1[0]) {
+                        x = b0[0];
+                        if (++y > b1[1]) {
+                            y = b0[1];
+                            ++z;
+                        }
+                    }
+                    if (z > b1[2]) {
+                        more = false;
+                        break;
+                    }
+                    bx = x;
+                    have = refine_left(lk, td, flags, x, y, z);
                 }
+                if (!have) continue;
+                by = y;
+                bz = z;
+                const int lx = bx * W32 - dil32, ly = by * W32 - dil32, lz = bz * W32 - dil32, wd = W32 + 2 * dil32;
+                if (ref_pt(A, lx, ly, lz, lx + wd, ly + wd, lz + wd) || ref_pt(B, lx, ly, lz, lx + wd, ly + wd, lz + wd) ||
+                    ref_pt(C, lx, ly, lz, lx + wd, ly + wd, lz + wd))
+                    refine_flag(lk, td, flags, bx, by, bz);
+                else
+                    need = true;
             }
-            continue;
+            const unsigned nm = __ballot_sync(0xffffffffu, need);
+            if (need) S.q[qn + __popc(nm & ((1u << lane) - 1u))] = make_int4(lane, bx, by, bz);
+            qn += __popc(nm);
+            if (qn >= 32) ref_drain(S, qn, 32, lane, W32, dil32, lk, td, flags);
         }
-        // large or loose union: the warp's (triangle, candidate block) pairs spread evenly over
-        // the lanes (a triangle with very many candidates goes to the chunk queue instead)
-        const bool mine = valid && own > 0 && !(own > EMB_BIG_ITEMS && emb_bigq_push(Q, (uint32_t)t, own));
-        const uint32_t k = mine ? (uint32_t)own : 0u;
-        uint32_t incl = k;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const uint32_t wtot = __shfl_sync(0xffffffffu, incl, 31);
-        const int ox = (int)b0[0], oy = (int)b0[1], oz = (int)b0[2];
-        const int onx = mine ? (int)(b1[0] - b0[0] + 1) : 1, ony = mine ? (int)(b1[1] - b0[1] + 1) : 1;
-        const uint32_t omx = emb_recip((uint32_t)onx), omy = emb_recip((uint32_t)ony);
-        for (uint32_t s0 = 0; s0 < wtot; s0 += 32) {
-            const uint32_t gi = s0 + lane;
-            int lo = 0;
-#pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const uint32_t v = __shfl_sync(0xffffffffu, incl, lo + step - 1);
-                if (v <= gi) lo += step;
-            }
-            const int ti = lo > 31 ? 31 : lo;
-            const uint32_t first = __shfl_sync(0xffffffffu, incl, ti) - __shfl_sync(0xffffffffu, k, ti);
-            const int bx0 = __shfl_sync(0xffffffffu, ox, ti), by0 = __shfl_sync(0xffffffffu, oy, ti),
-                      bz0 = __shfl_sync(0xffffffffu, oz, ti), nbx = __shfl_sync(0xffffffffu, onx, ti),
-                      nby = __shfl_sync(0xffffffffu, ony, ti);
-            const uint32_t mbx = __shfl_sync(0xffffffffu, omx, ti), mby = __shfl_sync(0xffffffffu, omy, ti);
-            if (gi < wtot) {
-                const uint32_t r = gi - first, rr = emb_div_recip(r, (uint32_t)nbx, mbx), cx = r - rr * (uint32_t)nbx,
-                               cz = emb_div_recip(rr, (uint32_t)nby, mby), cy = rr - cz * (uint32_t)nby;
-                ref_block(S.A[ti], S.B[ti], S.C[ti], bx0 + (int)cx, by0 + (int)cy, bz0 + (int)cz, W32, dil32, lk, flags,
-                          fb);
-            }
+        if (qn > 0) ref_drain(S, qn, qn, lane, W32, dil32, lk, td, flags);
+        __syncwarp();
+    }
+    if (SM) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < nw; i += REFINE_WARPS * 32) {
+            const uint32_t v = s_todo[i];
+            if (__ldcg(todo + i) & ~v) atomicAnd(todo + i, v);
         }
     }
 }
 
 // The queued chunks of large triangles, one warp per chunk (candidates x fastest).
 __global__ void __launch_bounds__(EMB_BIG_BLOCK) k_refine_big(const int4 *__restrict__ rec, LevelGeom g, long long dil,
-                                                              EmbLookup lk, uint8_t *__restrict__ flags, FlagBits fb,
+                                                              EmbLookup lk, uint8_t *__restrict__ flags, TodoBits td,
                                                               EmbBigQ Q)
 {
     const int lane = threadIdx.x & 31;
@@ -303,7 +352,15 @@ __global__ void __launch_bounds__(EMB_BIG_BLOCK) k_refine_big(const int4 *__rest
         long long z = (long long)((first / (unsigned long long)nx) / (unsigned long long)ny);
         const long long dx = 32 % nx, dy = (32 / nx) % ny, dz = (32 / nx) / ny;
         for (unsigned long long it = first; it < i1; it += 32) {
-            refine_block(A, B, C, b0[0] + x, b0[1] + y, b0[2] + z, g, dil, lk, flags, fb);
+            const long long bx = b0[0] + x, by = b0[1] + y, bz = b0[2] + z;
+            if (refine_left(lk, td, flags, bx, by, bz)) {
+                const long long lx = bx * g.W - dil, ly = by * g.W - dil, lz = bz * g.W - dil, wd = g.W + 2 * dil;
+                if (emb_point_in_box(A, lx, ly, lz, lx + wd, ly + wd, lz + wd) ||
+                    emb_point_in_box(B, lx, ly, lz, lx + wd, ly + wd, lz + wd) ||
+                    emb_point_in_box(C, lx, ly, lz, lx + wd, ly + wd, lz + wd) ||
+                    emb_tri_box(A, B, C, lx, ly, lz, lx + wd, ly + wd, lz + wd))
+                    refine_flag(lk, td, flags, bx, by, bz);
+            }
             x += dx;
             y += dy;
             z += dz;
@@ -334,29 +391,55 @@ long long emb_refine_dilation(const emb_forest_s *f, int L, int band)
     return num >> sh;
 }
 
-// Enqueue only: flags (lv.n bytes) are cleared and set; fbits (NULL for a level without a
-// bitmap) is scratch of a word more than the level's bitmap has, the last one the count of
-// the chunk queue.
+// The shared memory of the largest copied bitmap is above the default limit; set once a
+// device, before any capture (a batch plans, and so launches, outside of one).
+static emb_status refine_init()
+{
+    static std::atomic<bool> done[64];
+    int dev = 0;
+    EMB_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return EMB_ERR_CUDA;
+    if (done[dev].load(std::memory_order_acquire)) return EMB_OK;
+    EMB_CUDA_TRY(cudaFuncSetAttribute(k_refine<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(REFINE_WARPS * sizeof(RefWarp) + REFINE_SM_WORDS * sizeof(uint64_t))));
+    done[dev].store(true, std::memory_order_release);
+    return EMB_OK;
+}
+
+// Enqueue only: flags (lv.n bytes) are written; fbits (NULL for a level without a
+// bitmap) is scratch of the size of the level's bitmap.
 emb_status emb_enq_refine(const int4 *rec, int64_t T, LevelGeom g, long long dil, const EmbLevel &lv, uint8_t *flags,
                           unsigned long long *fbits, const EmbBigQ &Q, cudaStream_t s)
 {
     if (lv.n == 0) return EMB_OK;
-    EMB_CUDA_TRY(cudaMemsetAsync(flags, 0, lv.n, s));
+    const emb_status ri = refine_init();
+    if (ri != EMB_OK) return ri;
     const EmbLookup lk = emb_lookup_of(lv);
-    FlagBits fb = {nullptr, g.nb};
-    EmbBigQ q = Q;
+    TodoBits td = {nullptr, g.nb};
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
-    if (fbits && nw > 0) {
-        EMB_CUDA_TRY(cudaMemsetAsync(fbits, 0, (nw + 1) * sizeof(unsigned long long), s));
-        fb.w = fbits;
-        q.n = fbits + nw;
-    } else if (Q.cap) EMB_CUDA_TRY(cudaMemsetAsync(Q.n, 0, sizeof(unsigned long long), s));
-    int64_t grid = (T + 32 * EMB_WU_WARPS - 1) / (32 * EMB_WU_WARPS);
-    const int64_t resident = (int64_t)emb_sm_count() * REFINE_MINB;
-    if (grid > resident) grid = resident;
-    if (grid < 1) grid = 1;
-    EMB_LAUNCH((k_refine), (int)grid, 32 * EMB_WU_WARPS, 0, s)(rec, T, g, dil, lk, flags, fb, q);
-    if (q.cap) EMB_LAUNCH((k_refine_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, dil, lk, flags, fb, q);
+    if (fbits && lv.bits && nw > 0) {
+        EMB_CUDA_TRY(cudaMemcpyAsync(fbits, lv.bits, nw * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+        td.w = (uint32_t *)fbits;
+    } else {
+        EMB_CUDA_TRY(cudaMemsetAsync(flags, 0, lv.n, s));
+    }
+    if (Q.cap) EMB_CUDA_TRY(cudaMemsetAsync(Q.n, 0, sizeof(unsigned long long), s));
+    // consecutive tiles for each CTA, a whole number of its warps
+    const int64_t tiles = (T + 31) / 32, resident = (int64_t)emb_sm_count() * REFINE_MINB;
+    int64_t chunk = (tiles + resident - 1) / resident;
+    chunk = (chunk + REFINE_WARPS - 1) / REFINE_WARPS * REFINE_WARPS;
+    const int grid = emb_grid(tiles, (int)(chunk > 0 ? chunk : REFINE_WARPS));
+    if (chunk < REFINE_WARPS) chunk = REFINE_WARPS;
+    const size_t smem = REFINE_WARPS * sizeof(RefWarp);
+    if (td.w && nw <= REFINE_SM_WORDS) {
+        EMB_LAUNCH((k_refine<true>), grid, 32 * REFINE_WARPS, smem + (size_t)nw * sizeof(uint64_t), s)
+        (rec, T, g, dil, lk, flags, td.w, (int)(2 * nw), chunk, Q);
+    } else {
+        EMB_LAUNCH((k_refine<false>), grid, 32 * REFINE_WARPS, smem, s)(rec, T, g, dil, lk, flags, td.w, 0, chunk, Q);
+    }
+    if (Q.cap) EMB_LAUNCH((k_refine_big), EMB_BIG_GRID, EMB_BIG_BLOCK, 0, s)(rec, g, dil, lk, flags, td, Q);
+    if (td.w)
+        EMB_LAUNCH((k_refine_flags), emb_grid(lv.n, 256), 256, 0, s)(lv.key, lv.n, lv.d_n, td.w, g.nb, flags);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
