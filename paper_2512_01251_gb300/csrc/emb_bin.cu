@@ -697,9 +697,10 @@ extern "C" emb_status emb_bin_ex(emb_mesh m, emb_forest f, int32_t level, int32_
         const uint64_t cap = (uint64_t)4 * m->T + (1 << 20);
         rc = bin_finest(b, cap, cap, s);
     }
-    // the counts travel to a pinned slot behind the bins, so that emb_bins_sync only
-    // waits for them instead of synchronising the stream
-    if (rc == EMB_OK) {
+    // the finest bins' counts travel to a pinned slot behind them, so that emb_bins_sync
+    // only waits for them instead of synchronising the stream (below the finest level the
+    // only reader is a caller that asks for them)
+    if (rc == EMB_OK && level == f->max_level) {
         b->rb_slot = emb_readback_acquire(&b->rb_h, &b->rb_ev);
         if (b->rb_slot >= 0 && (cudaMemcpyAsync(b->rb_h, b->dcount, 16, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                                 cudaEventRecord(b->rb_ev, s) != cudaSuccess))

@@ -106,10 +106,25 @@ extern "C" emb_status emb_status_get(void *stream, emb_status *out)
     if (!out) return EMB_ERR_BAD_INPUT;
     int *st = emb_status_word();
     if (!st) return EMB_ERR_CUDA;
-    EMB_CUDA_TRY(cudaStreamSynchronize(emb_stream(stream)));
+    cudaStream_t s = emb_stream(stream);
     int v = 0;
-    EMB_CUDA_TRY(cudaMemcpy(&v, st, sizeof(int), cudaMemcpyDeviceToHost));
-    EMB_CUDA_TRY(cudaMemset(st, 0, sizeof(int)));
+    uint64_t *h = nullptr;
+    cudaEvent_t ev;
+    const int slot = emb_readback_acquire(&h, &ev);
+    if (slot >= 0) {
+        // through page-locked memory, behind the stream's work: one wait
+        cudaError_t e = cudaMemcpyAsync(h, st, sizeof(int), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(st, 0, sizeof(int), s);
+        if (e == cudaSuccess) e = cudaEventRecord(ev, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess) v = *(volatile int *)h;
+        emb_readback_release(slot);
+        EMB_CUDA_TRY(e);
+    } else {
+        EMB_CUDA_TRY(cudaStreamSynchronize(s));
+        EMB_CUDA_TRY(cudaMemcpy(&v, st, sizeof(int), cudaMemcpyDeviceToHost));
+        EMB_CUDA_TRY(cudaMemset(st, 0, sizeof(int)));
+    }
     *out = v;
     return EMB_OK;
 }
@@ -388,7 +403,7 @@ int emb_readback_acquire(uint64_t **h, cudaEvent_t *ev)
     if (cudaGetDevice(&dev) != cudaSuccess) return -1;
     std::lock_guard<std::mutex> lk(g_rb_mu);
     if (!g_rb_host) {
-        if (cudaHostAlloc((void **)&g_rb_host, EMB_RB_SLOTS * 64, cudaHostAllocPortable) != cudaSuccess) {
+        if (cudaHostAlloc((void **)&g_rb_host, EMB_RB_SLOTS * EMB_RB_WORDS * sizeof(uint64_t), cudaHostAllocPortable) != cudaSuccess) {
             g_rb_host = nullptr;
             return -1;
         }
@@ -417,7 +432,7 @@ int emb_readback_acquire(uint64_t **h, cudaEvent_t *ev)
             g_rb_dev[i] = dev;
         }
         g_rb_used[i] = true;
-        *h = g_rb_host + 8 * i;
+        *h = g_rb_host + EMB_RB_WORDS * i;
         *ev = g_rb_ev[i];
         return i;
     }

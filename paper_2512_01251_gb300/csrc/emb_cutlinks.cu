@@ -1148,17 +1148,25 @@ emb_status emb_enq_link_emit(const LinkTable &tab, unsigned int *next, bool zero
 // (blk_off[n]); >= 0 the count, read back.  With read_count the count is read back
 // (synchronising s); without it nothing is read back.
 #define EMB_LINKS_ON_DEVICE (-2)
+static emb_status read_links(emb_forest f, cudaStream_t s)
+{
+    uint32_t here = 0;
+    // the forest's page-locked slot is free once its block counts have settled
+    uint32_t *h = f->rb_slot >= 0 ? (uint32_t *)f->rb_h : &here;
+    EMB_CUDA_TRY(cudaMemcpyAsync(h, f->blk_off + f->lv[f->max_level].n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+    if (f->rb_slot >= 0) EMB_CUDA_TRY(cudaEventRecord(f->rb_ev, s));
+    EMB_CUDA_TRY(cudaStreamSynchronize(s));
+    f->n_links = (int64_t) * (volatile uint32_t *)h;
+    return EMB_OK;
+}
+
 static emb_status build_candidates(emb_forest f, int lattice, cudaStream_t s, bool read_count)
 {
     int L = f->max_level;
     if (f->top != L || !f->lv[L].mask_valid) return EMB_ERR_STATE;
     if ((f->n_links >= 0 || f->n_links == EMB_LINKS_ON_DEVICE) && f->cand_lattice == lattice && f->cand) {
         if (f->n_links >= 0 || !read_count) return EMB_OK;
-        uint32_t total = 0;
-        EMB_CUDA_TRY(cudaMemcpyAsync(&total, f->blk_off + f->lv[L].n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        EMB_CUDA_TRY(cudaStreamSynchronize(s));
-        f->n_links = (int64_t)total;
-        return EMB_OK;
+        return read_links(f, s);
     }
     EmbLevel &lv = f->lv[L];
     emb_status rc = emb_build_neighbors(lv, s);
@@ -1178,11 +1186,7 @@ static emb_status build_candidates(emb_forest f, int lattice, cudaStream_t s, bo
     f->cand_lattice = lattice;
     f->n_links = EMB_LINKS_ON_DEVICE;
     if (!read_count) return EMB_OK;
-    uint32_t total = 0;
-    EMB_CUDA_TRY(cudaMemcpyAsync(&total, f->blk_off + lv.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    EMB_CUDA_TRY(cudaStreamSynchronize(s));
-    f->n_links = (int64_t)total;
-    return EMB_OK;
+    return read_links(f, s);
 }
 
 extern "C" emb_status emb_cutlinks_count(emb_forest f, int32_t lattice, int64_t *h_count, void *stream)

@@ -236,7 +236,8 @@ emb_status emb_build_hash(EmbLevel &lv, cudaStream_t s);
 // through its mapping); EMB_ERR_BAD_INPUT for pageable memory.  NULL stays NULL.  *device:
 // plain device memory.
 emb_status emb_device_view(void *p, void **dp, bool *device = nullptr);
-// A pinned host slot (8 words) and its event for a count read-back; -1 when none is free.
+#define EMB_RB_WORDS 64
+// A pinned host slot (EMB_RB_WORDS words) and its event for a count read-back; -1 when none is free.
 int emb_readback_acquire(uint64_t **h, cudaEvent_t *ev);
 void emb_readback_release(int slot);
 emb_status emb_enq_neighbors(EmbLevel &lv, cudaStream_t s);

@@ -179,7 +179,13 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
     // error word, completion counters and extent, then the edge table: cleared together
     char *scratch = nullptr;
     emb_status rc = EMB_OK;
-    uint32_t head[1 + EDGE_COUNTERS + 1] = {0};
+    // its copy on the host, in page-locked memory where a slot is free
+    uint32_t here[1 + EDGE_COUNTERS + 1] = {0}, *head = here;
+    static_assert(sizeof(here) <= EMB_RB_WORDS * sizeof(uint64_t), "a read-back slot holds the head");
+    uint64_t *rb = nullptr;
+    cudaEvent_t rb_ev;
+    const int slot = emb_readback_acquire(&rb, &rb_ev);
+    if (slot >= 0) head = (uint32_t *)rb;
     const size_t a_head = 512;
     // room for every edge in a small mesh's overflow table (a triangle has 3/2); in a large
     // one for a third of them (a few percent overflow, more where a few vertices have many
@@ -209,7 +215,8 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
         EMB_LAUNCH((k_mesh_records), emb_grid(T, 256), 256, 0, s)(d_verts, d_tris, V, T, r_o, m->rec, E,
                                                                       (int *)scratch + 1 + EDGE_COUNTERS, (int *)scratch);
         if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(head, scratch, sizeof(head), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaMemcpyAsync(head, scratch, sizeof(here), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            (slot >= 0 && cudaEventRecord(rb_ev, s) != cudaSuccess) ||
             cudaStreamSynchronize(s) != cudaSuccess) {
             rc = EMB_ERR_CUDA;
             goto done;
@@ -229,6 +236,7 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
     if (head[0] & (MESH_ERR_ID | MESH_ERR_SNAP)) rc = EMB_ERR_BAD_INPUT;
     else if (head[0]) rc = EMB_ERR_NOT_WATERTIGHT;
 done:
+    emb_readback_release(slot);
     if (scratch) cudaFreeAsync(scratch, s);
     if (rc != EMB_OK) {
         emb_mesh_destroy(m);
