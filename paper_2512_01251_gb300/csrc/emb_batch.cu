@@ -60,7 +60,7 @@ struct BMesh {
     uint2 *witem = nullptr;                         // link work items
     uint2 *extra = nullptr;                         // extra parts of split blocks
     unsigned long long *queue = nullptr;            // extra parts asked for, cursor of a per-mesh link launch
-    EmbBigQ bq = {nullptr, nullptr, 0};             // chunk queue of large triangles
+    EmbBigQ bq = emb_bigq(0);                       // chunk queue of large triangles
     unsigned long long *fbits = nullptr;            // dense flagged bits (largest refined level)
     int32_t *o_cell = nullptr, *o_tri = nullptr;
     uint8_t *o_dir = nullptr;
@@ -231,6 +231,7 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     BTRY(balloc(B, &B.witem, fin.n + 1));
     BTRY(balloc(B, &B.extra, (size_t)emb_link_extra_capacity(fin.n)));
     BTRY(balloc(B, &B.queue, 2));
+    B.bq = emb_bigq(T);
     BTRY(balloc(B, &B.bq.n, 1));
     BTRY(balloc(B, &B.bq.q, (size_t)emb_bigq_capacity(T)));
     B.bq.cap = (uint32_t)emb_bigq_capacity(T);

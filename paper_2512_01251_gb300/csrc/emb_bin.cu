@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(EMB_WU_WARPS * 32, 8) k_bin_pairs(const int4 *
             ? (unsigned long long)(b1[0] - b0[0] + 1) * (unsigned long long)(b1[1] - b0[1] + 1) *
                   (unsigned long long)(b1[2] - b0[2] + 1)
             : 0ull;
-    const bool mine = valid && own > 0 && !(own > EMB_BIG_ITEMS && emb_bigq_push(Q, (uint32_t)t, own));
+    const bool mine = valid && own > 0 && !(own > Q.items && emb_bigq_push(Q, (uint32_t)t, own));
     const uint32_t k = mine ? (uint32_t)own : 0u;
     uint32_t incl = k;
 #pragma unroll
@@ -592,7 +592,7 @@ static emb_status bin_finest(emb_bins b, uint64_t list_cap, uint64_t ent_cap, cu
     // one scratch: the cleared words, the pair list, and the chunk queue where a triangle may
     // meet more than EMB_BIG_ITEMS blocks dilated by half a cell
     const long long span = ((m->ext + g.h) >> g.lW) + 2;
-    EmbBigQ Q = {nullptr, nullptr, 0};
+    EmbBigQ Q = emb_bigq(m->T);
     if (emb_mesh_big(m, span, span, span)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t a_z = up((size_t)emb_bin_words(lv.n) * sizeof(uint64_t)), a_bs = up((size_t)list_cap * sizeof(uint2)),

@@ -566,7 +566,8 @@ emb_status emb_build_neighbors(EmbLevel &lv, cudaStream_t s)
 // ---------------------------------------------------------------------------
 int64_t emb_bigq_capacity(int64_t T)
 {
-    const int64_t c = 16 * T + 1024;
+    // a small mesh's triangles take up to EMB_BIG_CHUNKS_SMALL entries more
+    const int64_t c = (T < EMB_BIG_SMALL_T ? 16 + EMB_BIG_CHUNKS_SMALL : 16) * T + 1024;
     return c < (1 << 20) ? c : (1 << 20);
 }
 

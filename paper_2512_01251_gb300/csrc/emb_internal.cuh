@@ -604,20 +604,37 @@ struct WuTri {
 // entries to a queue, and a second kernel walks every chunk with one warp.  A
 // thread that finds the queue full walks its items itself: the queue's size
 // affects the speed only, never the result.
+// A small mesh has few warps, which leave the chip idle while each lane walks its own
+// triangle: its line lies at 8 items, and a triangle gets up to 16 chunks of 64 before
+// their size grows to EMB_BIG_CHUNK (1,103 triangles on 384 cells an axis, 35 warps: refine,
+// voxelize and bin kernels 700 -> 140 us, embed_1k_fine 1346 -> 771 us).
 #define EMB_BIG_ITEMS 64
 #define EMB_BIG_CHUNK 512
+#define EMB_BIG_SMALL_T 16384
+#define EMB_BIG_ITEMS_SMALL 8
+#define EMB_BIG_CHUNK_SMALL 64
+#define EMB_BIG_CHUNKS_SMALL 16
 #define EMB_BIG_NONE 0xFFFFFFFFu
 struct EmbBigQ {
     uint2 *q;               // entries (triangle, chunk | chunk count << 16); EMB_BIG_NONE = unused
     unsigned long long *n;  // entries requested (may exceed cap)
     uint32_t cap;           // 0: no queue, every thread walks its own items
+    uint32_t items;         // a triangle with more items than this is cut into chunks
 };
+static inline EmbBigQ emb_bigq(int64_t T)
+{
+    return {nullptr, nullptr, 0, T < EMB_BIG_SMALL_T ? (uint32_t)EMB_BIG_ITEMS_SMALL : (uint32_t)EMB_BIG_ITEMS};
+}
 
 // Reserves the chunks of triangle t; false when they do not fit.
 __device__ __forceinline__ bool emb_bigq_push(const EmbBigQ &Q, uint32_t t, unsigned long long items)
 {
     if (Q.cap == 0) return false;
     unsigned long long nch = (items + EMB_BIG_CHUNK - 1) / EMB_BIG_CHUNK;
+    if (Q.items < EMB_BIG_ITEMS) {
+        const unsigned long long small = (items + EMB_BIG_CHUNK_SMALL - 1) / EMB_BIG_CHUNK_SMALL;
+        nch = max(nch, min(small, (unsigned long long)EMB_BIG_CHUNKS_SMALL));
+    }
     if (nch > 0xFFFFull) nch = 0xFFFFull;
     const unsigned long long base = atomicAdd(Q.n, nch);
     if (base + nch > Q.cap) {

@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32, REFINE_MINB) k_refine(const
         const unsigned long long own = t < T && onx > 0 && ony > 0 && onz > 0
                                            ? (unsigned long long)onx * (unsigned long long)ony * (unsigned long long)onz
                                            : 0ull;
-        const bool mine = may && own > 0 && !(own > EMB_BIG_ITEMS && emb_bigq_push(Q, (uint32_t)t, own));
+        const bool mine = may && own > 0 && !(own > Q.items && emb_bigq_push(Q, (uint32_t)t, own));
         S.A[lane] = A;  // the previous tile's queue was drained behind a warp barrier
         S.B[lane] = B;
         S.C[lane] = C;
@@ -461,7 +461,7 @@ extern "C" emb_status emb_refine_flags(emb_forest f, emb_bins b, int32_t level, 
     const emb_mesh m = b->m;
     const LevelGeom g = level_geom(f, level);
     const long long span = ((m->ext + 2 * dil) >> g.lW) + 2;
-    EmbBigQ Q = {nullptr, nullptr, 0};
+    EmbBigQ Q = emb_bigq(m->T);
     if (emb_mesh_big(m, span, span, span)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
     const size_t a_bits = ((size_t)(nw + 1) * sizeof(unsigned long long) + 255) & ~(size_t)255;

@@ -138,7 +138,7 @@ __global__ void k_vox(const int4 *__restrict__ rec, int64_t T, const uint32_t *_
         VoxTri V;
         if (!vox_setup(rec, t, g, V)) continue;
         const unsigned long long items = vox_items(V);
-        if (items > EMB_BIG_ITEMS && emb_bigq_push(Q, t, items)) continue;
+        if (items > Q.items && emb_bigq_push(Q, t, items)) continue;
         for (long long k = V.k0; k <= V.k1; ++k)
             for (long long j = V.j0; j <= V.j1; ++j) vox_line(V, g, lk, j, k, acc, st);
     }
@@ -290,7 +290,7 @@ extern "C" emb_status emb_voxelize(emb_forest f, emb_bins b, int32_t level, uint
     // the accumulators and, where a triangle may cross more than EMB_BIG_ITEMS lines, the
     // entries of the chunk queue
     const emb_mesh m = b->m;
-    EmbBigQ Q = {nullptr, nullptr, 0};
+    EmbBigQ Q = emb_bigq(m->T);
     if (emb_mesh_big(m, 1, (m->ext >> g.lh) + 1, (m->ext >> g.lh) + 1)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const size_t a_acc = ((size_t)emb_vox_words(lv.n) * sizeof(uint64_t) + 255) & ~(size_t)255;
     char *scratch = nullptr;
