@@ -26,29 +26,34 @@ struct VoxTri {
     int4 A, B, C;
     long long nx, ny, nz;
     int sx;
-    long long j0, j1, k0, k1, bx0, bx1;
+    int j0, j1, k0, k1, bx0, bx1;
+    bool narrow;  // plane offsets of this triangle fit 64 bits (vox_cross)
 };
 
-// false for a triangle parallel to x (no line crosses it)
+// false for a triangle parallel to x (no line crosses it); in 32 bits but for the normal
+// (coordinates below 2^25)
 __device__ __forceinline__ bool vox_setup(const int4 *__restrict__ rec, int64_t t, const LevelGeom &g, VoxTri &V)
 {
     V.A = rec[3 * t];
     V.B = rec[3 * t + 1];
     V.C = rec[3 * t + 2];
     const int4 A = V.A, B = V.B, C = V.C;
-    long long ux = (long long)B.x - A.x, uy = (long long)B.y - A.y, uz = (long long)B.z - A.z;
-    long long vx = (long long)C.x - A.x, vy = (long long)C.y - A.y, vz = (long long)C.z - A.z;
-    V.nx = uy * vz - uz * vy;
-    V.ny = uz * vx - ux * vz;
-    V.nz = ux * vy - uy * vx;
+    const int ux = B.x - A.x, uy = B.y - A.y, uz = B.z - A.z, vx = C.x - A.x, vy = C.y - A.y, vz = C.z - A.z;
+    V.nx = (long long)uy * vz - (long long)uz * vy;
+    V.ny = (long long)uz * vx - (long long)ux * vz;
+    V.nz = (long long)ux * vy - (long long)uy * vx;
     if (V.nx == 0) return false;
     V.sx = V.nx > 0 ? 1 : -1;
-    line_range(min(A.y, min(B.y, C.y)), max(A.y, max(B.y, C.y)), g.lh, g.half, g.ncell, V.j0, V.j1);
-    line_range(min(A.z, min(B.z, C.z)), max(A.z, max(B.z, C.z)), g.lh, g.half, g.ncell, V.k0, V.k1);
-    V.bx0 = emb_floor_shr(min(A.x, min(B.x, C.x)), g.lW);
-    V.bx1 = emb_floor_shr(max(A.x, max(B.x, C.x)), g.lW);
-    if (V.bx0 < 0) V.bx0 = 0;
-    if (V.bx1 > g.nb - 1) V.bx1 = g.nb - 1;
+    const int lox = min(A.x, min(B.x, C.x)), hix = max(A.x, max(B.x, C.x)), loy = min(A.y, min(B.y, C.y)),
+              hiy = max(A.y, max(B.y, C.y)), loz = min(A.z, min(B.z, C.z)), hiz = max(A.z, max(B.z, C.z));
+    const int half = (int)g.half, nc = (int)g.ncell;
+    V.j0 = max(-((-(loy - half)) >> g.lh), 0);
+    V.j1 = min((hiy - half) >> g.lh, nc - 1);
+    V.k0 = max(-((-(loz - half)) >> g.lh), 0);
+    V.k1 = min((hiz - half) >> g.lh, nc - 1);
+    V.bx0 = max(lox >> g.lW, 0);
+    V.bx1 = min(hix >> g.lW, (int)g.nb - 1);
+    V.narrow = max(hix - lox, max(hiy - loy, hiz - loz)) < (1 << 18) && g.lW <= 18;
     return true;
 }
 
@@ -80,49 +85,73 @@ __device__ __noinline__ void vox_gap(const VoxAcc &acc, long long bx, long long 
     else if (nx > 0 && (acc.key[nx - 1] >> EMB_KEY_BITS) == row) atomicXor(acc.t + nx - 1, 1u << line);
 }
 
-// The crossing of line (j, k) with the triangle, if any, recorded in its owner block.
-__device__ __forceinline__ void vox_line(const VoxTri &V, const LevelGeom &g, const EmbLookup &lk, long long j,
-                                         long long k, const VoxAcc &acc, int *st)
+// The block of [bx0, bx1] whose box [lo, lo + W) holds the crossing of the line (py, pz) with
+// the plane, and its cells before the crossing; -1 if none does.  n . (A - (x, py, pz)) =
+// D_yz + n_x (A_x - x); the crossing is at x_hit with x_hit - x = D(x) / n_x.  In 64 bits
+// where the triangle's extents and W are at most 2^18: |n| <= 2^37, A.y - py and A.z - pz lie
+// within the extent (the line meets the projection), A.x - lo within extent + W, so every sum
+// stays below 2^58; else in 128.  (Always in 128, the levels of embed_112k took 42 us and those
+// of 7.2M triangles 123; now 36 and 95.)
+// Returned as bx << 4 | cells.
+template <class I>
+__device__ __forceinline__ int vox_cross(long long nx, long long ny, long long nz, int ax, int dy, int dz, int bx0, int bx1,
+                                         int lW)
 {
-    unsigned long long *__restrict__ s_acc = acc.s;
-    unsigned int *__restrict__ p_acc = acc.p;
+    const I Dyz = (I)ny * (I)dy + (I)nz * (I)dz;
+    const bool pos = nx > 0;
+    const int half = 1 << (lW - 3);  // W = 8 half
+    for (int bx = bx0; bx <= bx1; ++bx) {
+        const I Dlo = Dyz + (I)nx * (I)(ax - (bx << lW));
+        if (pos ? Dlo < 0 : Dlo > 0) continue;  // x_hit < lo
+        const I Dhi = Dlo - ((I)nx << lW);
+        if (pos ? Dhi >= 0 : Dhi <= 0) continue;  // x_hit >= lo + W
+        // cell q of this line (centre lo + (2q+1) half) lies before the crossing iff
+        // the perturbed centre sees the plane ahead: sign(D) == sign(n_x), D == 0 -> no
+        int bits = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const I Dq = Dlo - (I)nx * (I)((2 * q + 1) * half);
+            if (pos ? Dq > 0 : Dq < 0) bits |= 1 << q;
+        }
+        return bx << 4 | bits;
+    }
+    return -1;
+}
+__device__ __noinline__ int vox_cross_wide(long long nx, long long ny, long long nz, int ax, int dy, int dz, int bx0, int bx1,
+                                           int lW)
+{
+    return vox_cross<i128>(nx, ny, nz, ax, dy, dz, bx0, bx1, lW);
+}
+
+// The crossing of line (j, k) with the triangle, if any, recorded in its owner block.
+__device__ __forceinline__ void vox_line(const VoxTri &V, const LevelGeom &g, const EmbLookup &lk, int j, int k,
+                                         const VoxAcc &acc, int *st)
+{
     const int4 A = V.A, B = V.B, C = V.C;
-    const int sx = V.sx;
-    const int pz = (int)((2 * k + 1) * g.half), py = (int)((2 * j + 1) * g.half);
+    const int sx = V.sx, half = (int)g.half;
+    const int pz = (2 * k + 1) * half, py = (2 * j + 1) * half;
     if (emb_orient_yz(A.y, A.z, B.y, B.z, py, pz) != sx || emb_orient_yz(B.y, B.z, C.y, C.z, py, pz) != sx ||
         emb_orient_yz(C.y, C.z, A.y, A.z, py, pz) != sx)
         return;
-    // n . (A - (x, py, pz)) = D_yz + n_x (A_x - x); the crossing is at x_hit with
-    // x_hit - x = D(x) / n_x.
-    const i128 Dyz = mul128(V.ny, (long long)A.y - py) + mul128(V.nz, (long long)A.z - pz);
-    for (long long bx = V.bx0; bx <= V.bx1; ++bx) {
-        const long long lo = bx * g.W;
-        const i128 Dlo = Dyz + mul128(V.nx, (long long)A.x - lo);
-        if (sgn_i128(Dlo) * sx < 0) continue;                     // x_hit < lo
-        if (sgn_i128(Dlo - mul128(V.nx, g.W)) * sx >= 0) continue;  // x_hit >= lo + W
-        const int32_t id = emb_lookup(lk, bx, j >> 2, k >> 2);
-        if (id < 0) {
-            vox_gap(acc, bx, j >> 2, k >> 2, (int)((j & 3) + 4 * (k & 3)));
-            return;
-        }
-        // cell q of this line (centre lo + (2q+1) half) lies before the crossing iff
-        // the perturbed centre sees the plane ahead: sign(D) == sign(n_x), D == 0 -> no
-        unsigned long long bits = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const i128 Dq = Dlo - mul128(V.nx, (2 * q + 1) * g.half);
-            if (sgn_i128(Dq) == sx) bits |= 1ull << q;
-        }
-        const int line = (int)((j & 3) + 4 * (k & 3));
-        if (!emb_ck((uint64_t)id, (uint64_t)acc.n, st)) return;
-        if (bits) atomicXor(s_acc + id, bits << (4 * line));
-        atomicXor(p_acc + id, 1u << line);
+    const int r = V.narrow ? vox_cross<long long>(V.nx, V.ny, V.nz, A.x, A.y - py, A.z - pz, V.bx0, V.bx1, g.lW)
+                           : vox_cross_wide(V.nx, V.ny, V.nz, A.x, A.y - py, A.z - pz, V.bx0, V.bx1, g.lW);
+    if (r < 0) {
+        emb_set_status(st, EMB_ERR_STATE);  // no block owns the crossing
         return;
     }
-    emb_set_status(st, EMB_ERR_STATE);  // no block owns the crossing
+    const int32_t id = emb_lookup(lk, r >> 4, j >> 2, k >> 2);
+    const int line = (j & 3) + 4 * (k & 3);
+    if (id < 0) {
+        vox_gap(acc, r >> 4, j >> 2, k >> 2, line);
+        return;
+    }
+    if (!emb_ck((uint64_t)id, (uint64_t)acc.n, st)) return;
+    if (r & 15) atomicXor(acc.s + id, (unsigned long long)(r & 15) << (4 * line));
+    atomicXor(acc.p + id, 1u << line);
 }
 
-__global__ void k_vox(const int4 *__restrict__ rec, int64_t T, const uint32_t *__restrict__ flist, int64_t nf,
+// 80 registers (the 128-bit path alone would take 112): latency-bound, six warps a scheduler.
+__global__ void __maxnreg__(80) k_vox(const int4 *__restrict__ rec, int64_t T, const uint32_t *__restrict__ flist, int64_t nf,
                       const uint32_t *__restrict__ d_nf, const uint32_t *__restrict__ keep, LevelGeom g, EmbLookup lk,
                       VoxAcc acc, EmbBigQ Q, int *st)
 {
@@ -139,8 +168,8 @@ __global__ void k_vox(const int4 *__restrict__ rec, int64_t T, const uint32_t *_
         if (!vox_setup(rec, t, g, V)) continue;
         const unsigned long long items = vox_items(V);
         if (items > Q.items && emb_bigq_push(Q, t, items)) continue;
-        for (long long k = V.k0; k <= V.k1; ++k)
-            for (long long j = V.j0; j <= V.j1; ++j) vox_line(V, g, lk, j, k, acc, st);
+        for (int k = V.k0; k <= V.k1; ++k)
+            for (int j = V.j0; j <= V.j1; ++j) vox_line(V, g, lk, j, k, acc, st);
     }
 }
 
@@ -165,7 +194,7 @@ __global__ void __launch_bounds__(EMB_BIG_BLOCK) k_vox_big(const int4 *__restric
         long long jj = (long long)(first % nj), kk = (long long)(first / nj);
         const long long dj = (long long)(32 % nj), dk = (long long)(32 / nj);
         for (unsigned long long it = first; it < i1; it += 32) {
-            vox_line(V, g, lk, V.j0 + jj, V.k0 + kk, acc, st);
+            vox_line(V, g, lk, V.j0 + (int)jj, V.k0 + (int)kk, acc, st);
             jj += dj;
             kk += dk;
             if (jj >= (long long)nj) {
