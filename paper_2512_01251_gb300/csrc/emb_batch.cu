@@ -23,6 +23,7 @@
 // this batch and keeps the fastest; emb_batch_configure sets one directly.
 #include <stdio.h>
 #include <stdlib.h>
+#include <string.h>
 
 #include <mutex>
 #include <vector>
@@ -66,7 +67,9 @@ struct BMesh {
     uint8_t *o_dir = nullptr;
     float *o_q = nullptr;
     int64_t pairs = 0, nwork = 0, links = 0;
-    uint32_t *d_n = nullptr;                        // with headroom: blocks of each level in this replay
+    // with headroom: blocks of each level in this replay, then its links (8 bytes at
+    // EMB_MAX_LEVELS), so that one copy reads them all back
+    uint32_t *d_n = nullptr;
     std::vector<void *> owned;
 };
 
@@ -182,7 +185,7 @@ static emb_status alloc_mesh(BMesh &B, int headroom)
     const int64_t T = B.m->T;
     if (headroom > 0) {
         headroom_caps(B, headroom);
-        BTRY(balloc(B, &B.d_n, EMB_MAX_LEVELS));
+        BTRY(balloc(B, &B.d_n, EMB_MAX_LEVELS + 2));
         for (int L = 1; L <= B.Lf; ++L) B.L[L].lv.d_n = B.d_n + L;
     }
     int64_t nmax = 1, wmax = 1;
@@ -275,7 +278,8 @@ static emb_status enqueue_mesh(BMesh &B, int tri_block, cudaStream_t s)
             BTRY(emb_enq_link_prep(lv, B.lattice, B.cand, B.rank, B.work_n, B.work, B.blk_off, B.tmp, s,
                                    hr ? EMB_NO_EXPECT : (uint64_t)B.nwork, hr ? EMB_NO_EXPECT : (uint64_t)B.links));
             BTRY(emb_enq_link_split(lv, B.work, B.work_n, B.cand, B.blk_off, B.bin_off, B.witem, B.extra, B.queue,
-                                    (uint32_t)emb_link_extra_capacity(lv.n), nullptr, s));
+                                    (uint32_t)emb_link_extra_capacity(lv.n),
+                                    hr ? (int64_t *)(B.d_n + EMB_MAX_LEVELS) : nullptr, s));
         }
     }
     return EMB_OK;
@@ -730,13 +734,21 @@ static emb_status replay_counts(const BMesh &B, cudaStream_t s, int64_t *blocks,
     for (int L = 0; L <= B.Lf; ++L) blocks[L] = B.L[L].lv.n;
     *links = B.links;
     if (!B.d_n) return EMB_OK;
-    uint32_t h[EMB_MAX_LEVELS + 1];
-    const EmbLevel &fin = B.L[B.Lf].lv;
-    if (B.Lf > 0) EMB_CUDA_TRY(cudaMemcpyAsync(h + 1, B.d_n + 1, B.Lf * sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    EMB_CUDA_TRY(cudaMemcpyAsync(h + EMB_MAX_LEVELS, B.blk_off + fin.n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    EMB_CUDA_TRY(cudaStreamSynchronize(s));
+    const size_t bytes = (EMB_MAX_LEVELS + 2) * sizeof(uint32_t);
+    uint32_t here[EMB_MAX_LEVELS + 2], *h = here;
+    uint64_t *rb = nullptr;
+    cudaEvent_t ev;
+    const int slot = emb_readback_acquire(&rb, &ev);
+    cudaError_t e = cudaMemcpyAsync(slot >= 0 ? (void *)rb : (void *)here, B.d_n, bytes, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && slot >= 0) e = cudaEventRecord(ev, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && slot >= 0) memcpy(here, rb, bytes);
+    emb_readback_release(slot);
+    EMB_CUDA_TRY(e);
+    int64_t nl = 0;
+    memcpy(&nl, h + EMB_MAX_LEVELS, sizeof(nl));
     for (int L = 1; L <= B.Lf; ++L) blocks[L] = h[L] < (uint64_t)B.L[L].lv.n ? h[L] : B.L[L].lv.n;
-    *links = h[EMB_MAX_LEVELS] < (uint64_t)B.links ? h[EMB_MAX_LEVELS] : B.links;
+    *links = nl < B.links ? nl : B.links;
     return EMB_OK;
 }
 
@@ -752,6 +764,51 @@ extern "C" emb_status emb_batch_counts(emb_batch b, int32_t j, void *stream, int
     return EMB_OK;
 }
 
+// A level's masks and block coordinates in one pass (either may be NULL).
+__global__ void k_copy_level(const uint64_t *__restrict__ key, const uint64_t *__restrict__ mask, int64_t n,
+                             uint64_t *__restrict__ o_mask, int32_t *__restrict__ o_blocks)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    if (o_mask) o_mask[i] = mask[i];
+    if (o_blocks) {
+        const uint64_t k = key[i];
+        o_blocks[3 * i + 0] = (int32_t)(k & EMB_KEY_MASK);
+        o_blocks[3 * i + 1] = (int32_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK);
+        o_blocks[3 * i + 2] = (int32_t)(k >> (2 * EMB_KEY_BITS));
+    }
+}
+
+// The columns of a link table in one pass (an output may be NULL), four links a thread
+// where the outputs are aligned for it.
+struct LinkColumns {
+    const int32_t *cell, *tri;
+    const uint8_t *dir;
+    const float *q;
+    int32_t *o_cell, *o_tri;
+    uint8_t *o_dir;
+    float *o_q;
+    bool wide;
+};
+__global__ void k_copy_links(LinkColumns c, int64_t n)
+{
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i >= n) return;
+    if (c.wide && i + 4 <= n) {
+        if (c.o_cell) *(int4 *)(c.o_cell + i) = *(const int4 *)(c.cell + i);
+        if (c.o_tri) *(int4 *)(c.o_tri + i) = *(const int4 *)(c.tri + i);
+        if (c.o_q) *(float4 *)(c.o_q + i) = *(const float4 *)(c.q + i);
+        if (c.o_dir) *(uchar4 *)(c.o_dir + i) = *(const uchar4 *)(c.dir + i);
+        return;
+    }
+    for (int64_t k = i; k < n && k < i + 4; ++k) {
+        if (c.o_cell) c.o_cell[k] = c.cell[k];
+        if (c.o_tri) c.o_tri[k] = c.tri[k];
+        if (c.o_q) c.o_q[k] = c.q[k];
+        if (c.o_dir) c.o_dir[k] = c.dir[k];
+    }
+}
+
 extern "C" emb_status emb_batch_results(emb_batch b, int32_t j, int32_t level, uint64_t *d_mask, int32_t *d_blocks,
                                         int32_t *d_cell, uint8_t *d_dir, float *d_q, int32_t *d_tri, void *stream)
 {
@@ -763,21 +820,33 @@ extern "C" emb_status emb_batch_results(emb_batch b, int32_t j, int32_t level, u
     BTRY(replay_counts(B, s, cnt_blocks, &cnt_links));
     EmbLevel lv = B.L[level].lv;  // a view: n becomes this replay's count
     lv.n = cnt_blocks[level];
-    if (d_mask && lv.n)
-        EMB_CUDA_TRY(cudaMemcpyAsync(d_mask, lv.mask, lv.n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
-    if (d_blocks && lv.n) {
-        emb_forest_s tmp;
-        tmp.R = B.R;
-        tmp.top = level;
-        tmp.lv[level] = lv;
-        emb_status rc = emb_forest_blocks(&tmp, level, d_blocks, stream);
-        tmp.lv[level] = EmbLevel();  // not owned
-        BTRY(rc);
+    // device memory: one pass a level and one a table (a copy for every array was 124 small
+    // copies for ten meshes; batch_10 3932 -> 3507 us, moving_112k 860 -> 772); anything else
+    // goes through copies
+    auto device = [](void *p) {
+        void *v;
+        bool d = false;
+        return !p || (emb_device_view(p, &v, &d) == EMB_OK && d);
+    };
+    if (lv.n && (d_mask || d_blocks)) {
+        const bool dm = device(d_mask);
+        if (d_blocks || dm)
+            EMB_LAUNCH((k_copy_level), emb_grid(lv.n, 256), 256, 0, s)(lv.key, lv.mask, lv.n, dm ? d_mask : nullptr, d_blocks);
+        if (!dm) EMB_CUDA_TRY(cudaMemcpyAsync(d_mask, lv.mask, lv.n * sizeof(uint64_t), cudaMemcpyDeviceToDevice, s));
     }
     const size_t n = (size_t)cnt_links;
-    if (d_cell && n) EMB_CUDA_TRY(cudaMemcpyAsync(d_cell, B.o_cell, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    if (d_dir && n) EMB_CUDA_TRY(cudaMemcpyAsync(d_dir, B.o_dir, n, cudaMemcpyDeviceToDevice, s));
-    if (d_q && n) EMB_CUDA_TRY(cudaMemcpyAsync(d_q, B.o_q, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    if (d_tri && n) EMB_CUDA_TRY(cudaMemcpyAsync(d_tri, B.o_tri, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+    if (n && (d_cell || d_dir || d_q || d_tri)) {
+        if (device(d_cell) && device(d_dir) && device(d_q) && device(d_tri)) {
+            const bool wide = (((uintptr_t)d_cell | (uintptr_t)d_q | (uintptr_t)d_tri) & 15) == 0 && ((uintptr_t)d_dir & 3) == 0;
+            const LinkColumns c = {B.o_cell, B.o_tri, B.o_dir, B.o_q, d_cell, d_tri, d_dir, d_q, wide};
+            EMB_LAUNCH((k_copy_links), emb_grid(cnt_links, 1024), 256, 0, s)(c, cnt_links);
+        } else {
+            if (d_cell) EMB_CUDA_TRY(cudaMemcpyAsync(d_cell, B.o_cell, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+            if (d_dir) EMB_CUDA_TRY(cudaMemcpyAsync(d_dir, B.o_dir, n, cudaMemcpyDeviceToDevice, s));
+            if (d_q) EMB_CUDA_TRY(cudaMemcpyAsync(d_q, B.o_q, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
+            if (d_tri) EMB_CUDA_TRY(cudaMemcpyAsync(d_tri, B.o_tri, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+        }
+    }
+    EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;
 }
