@@ -73,14 +73,14 @@ __global__ void k_lbm_bouzidi(const int32_t *__restrict__ cell, const uint8_t *_
     const int o = (d & 1) ? d + 1 : d - 1;
     int cx, cy, cz;
     emb_dir(d, cx, cy, cz);
-    const float f_d = pop[(int64_t)d * stride + c], f_o = pop[(int64_t)o * stride + c];
+    const float f_d = pop[(int64_t)d * stride + c];
     const float qq = q[k];
     float g;
     if (qq < 0.5f) {
         const int64_t p = lbm_source(c >> 6, (int)(c & 63), cx, cy, cz, nbr, mask);  // x - c_d
         g = p >= 0 ? 2.0f * qq * f_d + (1.0f - 2.0f * qq) * pop[(int64_t)d * stride + p] : f_d;
     } else {
-        g = f_d / (2.0f * qq) + (2.0f * qq - 1.0f) / (2.0f * qq) * f_o;
+        g = f_d / (2.0f * qq) + (2.0f * qq - 1.0f) / (2.0f * qq) * pop[(int64_t)o * stride + c];
     }
     pre[(int64_t)o * stride + c] = g;
     if (bits) atomicOr(bits + c, 1u << o);
@@ -142,10 +142,13 @@ __global__ void k_lbm_collide(const float *__restrict__ pre, float *__restrict__
 // word c of `bits` (row 0 of pre, which no link direction uses); bits is NULL without
 // links.  A CTA holds LBM_BLOCKS blocks, one thread a cell; their 27 neighbour ids and
 // masks are staged in shared memory, so the Q pulls of a cell wait on nothing but each
-// other.  Bound by HBM: 8 Q bytes a cell.
-#define LBM_BLOCKS 4
+// other.  Bound by HBM (8 Q bytes a cell) and the loads in flight: two blocks a CTA, ten CTAs
+// an SM for D3Q19 (48 registers) and nine for D3Q27 (56), the best of 1 to 8 blocks and all
+// register limits (6.2M cells, step with the boundary pass: 211 and 290 us; four blocks
+// and no limit 278 and 336; as three passes 400 us for D3Q19).
+#define LBM_BLOCKS 2
 template <int Q>
-__global__ void __launch_bounds__(64 * LBM_BLOCKS) k_lbm_step(const float *__restrict__ pop, const float *__restrict__ pre,
+__global__ void __launch_bounds__(64 * LBM_BLOCKS, Q == 19 ? 10 : 9) k_lbm_step(const float *__restrict__ pop, const float *__restrict__ pre,
                                                               const uint32_t *__restrict__ bits, float *__restrict__ out,
                                                               int64_t stride, int64_t nblk,
                                                               const int32_t *__restrict__ nbr,
