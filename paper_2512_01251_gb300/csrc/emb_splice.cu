@@ -15,6 +15,8 @@
 // forest's blocks there, with their solid masks, and merges the two link tables: the
 // old links outside the inner window and the window's links inside it, renumbered to
 // the merged finest level and ordered by (cell, direction) as a fresh table is.
+#include <vector>
+
 #include "emb_internal.cuh"
 
 __global__ void k_root_keys_window(int64_t R, int64_t y0, int64_t ny, int64_t z0, int64_t n, uint64_t *__restrict__ key)
@@ -114,6 +116,41 @@ __global__ void k_sp_place(const uint64_t *__restrict__ key, const uint64_t *__r
     newid[i] = (int32_t)p;
 }
 
+// The bits of the selected blocks of one side in the merged level's bitmap.
+__global__ void k_sp_bits(const uint64_t *__restrict__ key, int64_t n, int64_t nb, RowWindow W, int L, bool want_inside,
+                          unsigned long long *__restrict__ bits)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t k = key[i];
+    if (W.inside(k, L) != want_inside) return;
+    const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
+                  bz = (int64_t)(k >> (2 * EMB_KEY_BITS)), lin = (bz * nb + by) * nb + bx;
+    atomicOr(bits + (lin >> 6), 1ull << (lin & 63));
+}
+
+// With the merged bitmap and its prefixes in place, a selected block's merged id is the rank
+// of its bit: it takes its key and mask there.  newid[i] as in k_sp_place (NULL: not wanted).
+__global__ void k_sp_rank(const uint64_t *__restrict__ key, const uint64_t *__restrict__ mask, int64_t n, int64_t nb,
+                          RowWindow W, int L, bool want_inside, const uint64_t *__restrict__ bits,
+                          const uint32_t *__restrict__ wpre, uint64_t *__restrict__ mkey, uint64_t *__restrict__ mmask,
+                          int32_t *__restrict__ newid)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t k = key[i];
+    if (W.inside(k, L) != want_inside) {
+        if (newid) newid[i] = -1;
+        return;
+    }
+    const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
+                  bz = (int64_t)(k >> (2 * EMB_KEY_BITS)), lin = (bz * nb + by) * nb + bx;
+    const int64_t p = (int64_t)wpre[lin >> 6] + __popcll(bits[lin >> 6] & ((1ull << (lin & 63)) - 1ull));
+    mkey[p] = k;
+    mmask[p] = mask[i];
+    if (newid) newid[i] = (int32_t)p;
+}
+
 // First link of every block in a table sorted by cell (cell = block * 64 + t).
 __global__ void k_sp_link_starts(const int32_t *__restrict__ cell, int64_t nl, int64_t nblk, uint32_t *__restrict__ start)
 {
@@ -158,6 +195,33 @@ __global__ void k_sp_link_copy(const int32_t *__restrict__ cell, const uint8_t *
     o_tri[o] = tri_map && tri[k] >= 0 ? tri_map[tri[k]] : tri[k];
 }
 
+// Stream-ordered scratch of a splice, freed at its end whichever way it ends; keep() lets go
+// of an array that the forest has taken over.
+struct SpliceScratch {
+    std::vector<void *> p;
+    cudaStream_t s;
+    int slot = -1;
+    explicit SpliceScratch(cudaStream_t s_) : s(s_) {}
+    ~SpliceScratch()
+    {
+        for (void *q : p)
+            if (q) cudaFreeAsync(q, s);
+        emb_readback_release(slot);
+    }
+    template <class T>
+    cudaError_t get(T **out, int64_t n)
+    {
+        const cudaError_t e = emb_malloc_async(out, (size_t)n * sizeof(T), s);
+        if (e == cudaSuccess) p.push_back(*out);
+        return e;
+    }
+    void keep(void *q)
+    {
+        for (void *&x : p)
+            if (x == q) x = nullptr;
+    }
+};
+
 extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t y1, int32_t z0, int32_t z1,
                                  const int32_t *f_cell, const uint8_t *f_dir, const float *f_q, const int32_t *f_tri,
                                  int64_t f_n, const int32_t *w_cell, const uint8_t *w_dir, const float *w_q,
@@ -179,102 +243,155 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
     cudaStream_t s = emb_stream(stream);
     const RowWindow W = {y0, y1, z0, z1};
     emb_status rc = EMB_OK;
-    for (int L = 0; L <= Lf && rc == EMB_OK; ++L) {
-        EmbLevel &P = f->lv[L];
-        const EmbLevel &Q = w->lv[L];
-        const int64_t np = P.n, nq = Q.n, nmax = np > nq ? np : nq;
-        uint32_t *selP = nullptr, *posP = nullptr, *selQ = nullptr, *posQ = nullptr;
-        uint64_t *tmp = nullptr, *cP = nullptr, *cQ = nullptr;
-        EMB_CUDA_TRY(emb_malloc_async(&selP, (np + 1) * sizeof(uint32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&posP, (np + 1) * sizeof(uint32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&selQ, (nq + 1) * sizeof(uint32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&posQ, (nq + 1) * sizeof(uint32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&tmp, emb_scan_tmp_words(nmax) * sizeof(uint64_t), s));
-        if (np > 0) EMB_LAUNCH((k_sp_select), emb_grid(np, 256), 256, 0, s)(P.key, np, W, L, 0, selP);
-        if (nq > 0) EMB_LAUNCH((k_sp_select), emb_grid(nq, 256), 256, 0, s)(Q.key, nq, W, L, 1, selQ);
-        EMB_CUDA_TRY(cudaGetLastError());
-        rc = emb_scan_into(selP, posP, np, tmp, s);
-        if (rc == EMB_OK) rc = emb_scan_into(selQ, posQ, nq, tmp, s);
-        if (rc != EMB_OK) return rc;
-        uint32_t kk[2] = {0, 0};
-        EMB_CUDA_TRY(cudaMemcpyAsync(&kk[0], posP + np, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        EMB_CUDA_TRY(cudaMemcpyAsync(&kk[1], posQ + nq, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-        EMB_CUDA_TRY(cudaStreamSynchronize(s));
-        const int64_t kp = kk[0], kq = kk[1], n = kp + kq;
-        EMB_CUDA_TRY(emb_malloc_async(&cP, (kp + 1) * sizeof(uint64_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&cQ, (kq + 1) * sizeof(uint64_t), s));
-        if (np > 0) EMB_LAUNCH((k_sp_compact_keys), emb_grid(np, 256), 256, 0, s)(P.key, selP, posP, np, cP);
-        if (nq > 0) EMB_LAUNCH((k_sp_compact_keys), emb_grid(nq, 256), 256, 0, s)(Q.key, selQ, posQ, nq, cQ);
-        uint64_t *mkey = nullptr, *mmask = nullptr;
-        int32_t *idP = nullptr, *idQ = nullptr;
-        EMB_CUDA_TRY(emb_malloc_async(&mkey, (n + 1) * sizeof(uint64_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&mmask, (n + 1) * sizeof(uint64_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&idP, (np + 1) * sizeof(int32_t), s));
-        EMB_CUDA_TRY(emb_malloc_async(&idQ, (nq + 1) * sizeof(int32_t), s));
-        if (np > 0)
-            EMB_LAUNCH((k_sp_place), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, selP, posP, np, cQ, kq, mkey, mmask, idP);
-        if (nq > 0)
-            EMB_LAUNCH((k_sp_place), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, selQ, posQ, nq, cP, kp, mkey, mmask, idQ);
-        EMB_CUDA_TRY(cudaGetLastError());
-        if (L == Lf) {
-            // the link tables: per merged block the links of the side it came from
-            uint32_t *stP = nullptr, *stQ = nullptr, *cnt = nullptr, *moff = nullptr;
-            EMB_CUDA_TRY(emb_malloc_async(&stP, (np + 1) * sizeof(uint32_t), s));
-            EMB_CUDA_TRY(emb_malloc_async(&stQ, (nq + 1) * sizeof(uint32_t), s));
-            EMB_CUDA_TRY(emb_malloc_async(&cnt, (n + 1) * sizeof(uint32_t), s));
-            EMB_CUDA_TRY(emb_malloc_async(&moff, (n + 1) * sizeof(uint32_t), s));
-            EMB_CUDA_TRY(cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), s));
-            EMB_LAUNCH((k_sp_link_starts), emb_grid(np + 1, 256), 256, 0, s)(f_cell, f_n, np, stP);
-            EMB_LAUNCH((k_sp_link_starts), emb_grid(nq + 1, 256), 256, 0, s)(w_cell, w_n, nq, stQ);
-            if (np > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(np, 256), 256, 0, s)(idP, np, stP, cnt);
-            if (nq > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(nq, 256), 256, 0, s)(idQ, nq, stQ, cnt);
-            EMB_CUDA_TRY(cudaGetLastError());
-            uint64_t *tmp2 = nullptr;
-            EMB_CUDA_TRY(emb_malloc_async(&tmp2, emb_scan_tmp_words(n) * sizeof(uint64_t), s));
-            rc = emb_scan_into(cnt, moff, n, tmp2, s);
+    SpliceScratch S(s);
+    // merged blocks per level and, last, the links: in a page-locked slot where one is free
+    uint32_t here[EMB_MAX_LEVELS + 1], *counts = here;
+    uint64_t *rb = nullptr;
+    cudaEvent_t rb_ev;
+    S.slot = emb_readback_acquire(&rb, &rb_ev);
+    if (S.slot >= 0) counts = (uint32_t *)rb;
+    // every level is merged beside the old ones; f takes them over at the end
+    struct Merged {
+        uint64_t *key = nullptr, *mask = nullptr, *bits = nullptr;
+        uint32_t *wpre = nullptr;
+    } M[EMB_MAX_LEVELS];
+    int32_t *idP = nullptr, *idQ = nullptr;
+    int64_t n_fin = 0;  // room for the merged finest blocks
+    for (int L = 0; L <= Lf; ++L) {
+        const EmbLevel &P = f->lv[L], &Q = w->lv[L];
+        const int64_t np = P.n, nq = Q.n, nmax = np > nq ? np : nq, nw = emb_bitmap_words(P.nb_axis);
+        Merged &m = M[L];
+        if (L == Lf || nw == 0) {
+            EMB_CUDA_TRY(S.get(&idP, np + 1));
+            EMB_CUDA_TRY(S.get(&idQ, nq + 1));
+        }
+        if (nw > 0) {
+            // the merged bitmap first: it gives the merged ids, and is the level's index.  Room
+            // for every block of both sides; the count is read back with those of the other
+            // levels.  (Selections scanned, compacted and searched, then the index of their
+            // merge, with two read-backs: 18 operations a level instead of 7, and 20 search
+            // steps a block.)
+            const int64_t zw = nw + emb_scan_tmp_words(nw);
+            EMB_CUDA_TRY(S.get(&m.bits, zw));
+            EMB_CUDA_TRY(S.get(&m.wpre, nw + 1));
+            EMB_CUDA_TRY(S.get(&m.key, np + nq + 1));
+            EMB_CUDA_TRY(S.get(&m.mask, np + nq + 1));
+            EMB_CUDA_TRY(cudaMemsetAsync(m.bits, 0, zw * sizeof(uint64_t), s));
+            unsigned long long *mb = (unsigned long long *)m.bits;
+            if (np > 0) EMB_LAUNCH((k_sp_bits), emb_grid(np, 256), 256, 0, s)(P.key, np, P.nb_axis, W, L, false, mb);
+            if (nq > 0) EMB_LAUNCH((k_sp_bits), emb_grid(nq, 256), 256, 0, s)(Q.key, nq, P.nb_axis, W, L, true, mb);
+            rc = emb_scan_popc(m.bits, m.wpre, nw, m.bits + nw, true, s);
             if (rc != EMB_OK) return rc;
-            uint32_t total = 0;
-            EMB_CUDA_TRY(cudaMemcpyAsync(&total, moff + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-            EMB_CUDA_TRY(cudaStreamSynchronize(s));
-            *h_count = (int64_t)total;
-            if ((int64_t)total > capacity) {
-                rc = EMB_ERR_CAPACITY;
-            } else if (total > 0) {
-                if (!o_cell || !o_dir || !o_q || !o_tri) return EMB_ERR_BAD_INPUT;
-                if (f_n > 0)
-                    EMB_LAUNCH((k_sp_link_copy), emb_grid(f_n, 256), 256, 0, s)(f_cell, f_dir, f_q, f_tri, f_n, idP, stP,
-                                                                               moff, nullptr, capacity, o_cell, o_dir,
-                                                                               o_q, o_tri);
-                if (w_n > 0)
-                    EMB_LAUNCH((k_sp_link_copy), emb_grid(w_n, 256), 256, 0, s)(w_cell, w_dir, w_q, w_tri, w_n, idQ, stQ,
-                                                                               moff, w_tri_map, capacity, o_cell, o_dir,
-                                                                               o_q, o_tri);
-                EMB_CUDA_TRY(cudaGetLastError());
-            }
-            cudaFreeAsync(stP, s);
-            cudaFreeAsync(stQ, s);
-            cudaFreeAsync(cnt, s);
-            cudaFreeAsync(moff, s);
-            cudaFreeAsync(tmp2, s);
-        }
-        // the merged level replaces f's level (its index rebuilt, its neighbour table dropped)
-        if (rc == EMB_OK) {
-            if (P.key) cudaFreeAsync(P.key, s);
-            if (P.mask) cudaFreeAsync(P.mask, s);
-            if (P.nbr) cudaFreeAsync(P.nbr, s);
-            P.key = mkey;
-            P.mask = mmask;
-            P.nbr = nullptr;
-            P.n = n;
-            P.mask_valid = 1;
-            rc = emb_build_hash(P, s);
+            EMB_CUDA_TRY(cudaMemcpyAsync(counts + L, m.wpre + nw, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+            if (np > 0)
+                EMB_LAUNCH((k_sp_rank), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, np, P.nb_axis, W, L, false, m.bits,
+                                                                      m.wpre, m.key, m.mask, L == Lf ? idP : nullptr);
+            if (nq > 0)
+                EMB_LAUNCH((k_sp_rank), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, nq, P.nb_axis, W, L, true, m.bits,
+                                                                      m.wpre, m.key, m.mask, L == Lf ? idQ : nullptr);
+            EMB_CUDA_TRY(cudaGetLastError());
+            n_fin = np + nq;
         } else {
-            cudaFreeAsync(mkey, s);
-            cudaFreeAsync(mmask, s);
+            uint32_t *selP = nullptr, *posP = nullptr, *selQ = nullptr, *posQ = nullptr;
+            uint64_t *tmp = nullptr, *cP = nullptr, *cQ = nullptr;
+            EMB_CUDA_TRY(S.get(&selP, np + 1));
+            EMB_CUDA_TRY(S.get(&posP, np + 1));
+            EMB_CUDA_TRY(S.get(&selQ, nq + 1));
+            EMB_CUDA_TRY(S.get(&posQ, nq + 1));
+            EMB_CUDA_TRY(S.get(&tmp, emb_scan_tmp_words(nmax)));
+            if (np > 0) EMB_LAUNCH((k_sp_select), emb_grid(np, 256), 256, 0, s)(P.key, np, W, L, 0, selP);
+            if (nq > 0) EMB_LAUNCH((k_sp_select), emb_grid(nq, 256), 256, 0, s)(Q.key, nq, W, L, 1, selQ);
+            EMB_CUDA_TRY(cudaGetLastError());
+            rc = emb_scan_into(selP, posP, np, tmp, s);
+            if (rc == EMB_OK) rc = emb_scan_into(selQ, posQ, nq, tmp, s);
+            if (rc != EMB_OK) return rc;
+            uint32_t kk[2] = {0, 0};
+            EMB_CUDA_TRY(cudaMemcpyAsync(&kk[0], posP + np, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+            EMB_CUDA_TRY(cudaMemcpyAsync(&kk[1], posQ + nq, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+            EMB_CUDA_TRY(cudaStreamSynchronize(s));
+            const int64_t kp = kk[0], kq = kk[1], n = kp + kq;
+            EMB_CUDA_TRY(S.get(&cP, kp + 1));
+            EMB_CUDA_TRY(S.get(&cQ, kq + 1));
+            if (np > 0) EMB_LAUNCH((k_sp_compact_keys), emb_grid(np, 256), 256, 0, s)(P.key, selP, posP, np, cP);
+            if (nq > 0) EMB_LAUNCH((k_sp_compact_keys), emb_grid(nq, 256), 256, 0, s)(Q.key, selQ, posQ, nq, cQ);
+            EMB_CUDA_TRY(S.get(&m.key, n + 1));
+            EMB_CUDA_TRY(S.get(&m.mask, n + 1));
+            if (np > 0)
+                EMB_LAUNCH((k_sp_place), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, selP, posP, np, cQ, kq, m.key, m.mask, idP);
+            if (nq > 0)
+                EMB_LAUNCH((k_sp_place), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, selQ, posQ, nq, cP, kp, m.key, m.mask, idQ);
+            EMB_CUDA_TRY(cudaGetLastError());
+            counts[L] = (uint32_t)n;
+            n_fin = n;
         }
-        void *bufs[] = {selP, posP, selQ, posQ, tmp, cP, cQ, idP, idQ};
-        for (void *p : bufs)
+    }
+    {
+        // the link tables: per merged block the links of the side it came from (entries past
+        // the merged blocks count none)
+        const int64_t np = f->lv[Lf].n, nq = w->lv[Lf].n, n = n_fin;
+        uint32_t *stP = nullptr, *stQ = nullptr, *cnt = nullptr, *moff = nullptr;
+        uint64_t *tmp = nullptr;
+        EMB_CUDA_TRY(S.get(&stP, np + 1));
+        EMB_CUDA_TRY(S.get(&stQ, nq + 1));
+        EMB_CUDA_TRY(S.get(&cnt, n + 1));
+        EMB_CUDA_TRY(S.get(&moff, n + 1));
+        EMB_CUDA_TRY(S.get(&tmp, emb_scan_tmp_words(n)));
+        EMB_CUDA_TRY(cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), s));
+        EMB_LAUNCH((k_sp_link_starts), emb_grid(np + 1, 256), 256, 0, s)(f_cell, f_n, np, stP);
+        EMB_LAUNCH((k_sp_link_starts), emb_grid(nq + 1, 256), 256, 0, s)(w_cell, w_n, nq, stQ);
+        if (np > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(np, 256), 256, 0, s)(idP, np, stP, cnt);
+        if (nq > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(nq, 256), 256, 0, s)(idQ, nq, stQ, cnt);
+        EMB_CUDA_TRY(cudaGetLastError());
+        rc = emb_scan_into(cnt, moff, n, tmp, s);
+        if (rc != EMB_OK) return rc;
+        EMB_CUDA_TRY(cudaMemcpyAsync(counts + EMB_MAX_LEVELS, moff + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        if (S.slot >= 0) EMB_CUDA_TRY(cudaEventRecord(rb_ev, s));
+        EMB_CUDA_TRY(cudaStreamSynchronize(s));
+        const uint32_t total = *(volatile uint32_t *)(counts + EMB_MAX_LEVELS);
+        *h_count = (int64_t)total;
+        if ((int64_t)total > capacity) {
+            rc = EMB_ERR_CAPACITY;
+        } else if (total > 0) {
+            if (!o_cell || !o_dir || !o_q || !o_tri) return EMB_ERR_BAD_INPUT;
+            if (f_n > 0)
+                EMB_LAUNCH((k_sp_link_copy), emb_grid(f_n, 256), 256, 0, s)(f_cell, f_dir, f_q, f_tri, f_n, idP, stP, moff,
+                                                                           nullptr, capacity, o_cell, o_dir, o_q, o_tri);
+            if (w_n > 0)
+                EMB_LAUNCH((k_sp_link_copy), emb_grid(w_n, 256), 256, 0, s)(w_cell, w_dir, w_q, w_tri, w_n, idQ, stQ, moff,
+                                                                           w_tri_map, capacity, o_cell, o_dir, o_q, o_tri);
+            EMB_CUDA_TRY(cudaGetLastError());
+        }
+    }
+    // the merged levels replace f's (their neighbour tables dropped); a link buffer that was
+    // too small leaves the finest one as it was
+    for (int L = 0; L <= Lf && (L < Lf || rc == EMB_OK); ++L) {
+        EmbLevel &P = f->lv[L];
+        Merged &m = M[L];
+        void *old[] = {P.key, P.mask, P.nbr};
+        for (void *p : old)
             if (p) cudaFreeAsync(p, s);
+        P.key = m.key;
+        P.mask = m.mask;
+        P.nbr = nullptr;
+        P.n = (int64_t) * (volatile uint32_t *)(counts + L);
+        P.mask_valid = 1;
+        S.keep(m.key);
+        S.keep(m.mask);
+        if (m.bits) {
+            void *idx[] = {P.hkey, P.hval, P.bits, P.wpre};
+            for (void *p : idx)
+                if (p) cudaFreeAsync(p, s);
+            P.hkey = nullptr;
+            P.hval = nullptr;
+            P.hcap = 0;
+            P.bits = m.bits;
+            P.wpre = m.wpre;
+            S.keep(m.bits);
+            S.keep(m.wpre);
+        } else {
+            const emb_status rh = emb_build_hash(P, s);
+            if (rh != EMB_OK) rc = rh;
+        }
     }
     // cached link candidates belong to the old finest level
     if (f->cand) cudaFreeAsync(f->cand, s);
