@@ -137,12 +137,16 @@ __global__ void __launch_bounds__(CAND_BLOCK) k_link_cand(const uint64_t *__rest
 // chunk's links, which are consecutive in the table (the direction words fix each
 // cell's offset whichever warp handles it), one link per lane.  A bucket that
 // overflows sends its cell through an exact per-cell scan of the whole bin instead.
-// Sizes: 4 warps per CTA; a warp's tile of 32 triangles, 20 hit slots per cell and the
-// byte-wide best-hit indices (shared with the hit queue) take 9 KB of shared memory, so
-// six CTAs would fit on an SM.  The launch bound asks for five, which leaves 96
-// registers a thread: with the queue's shorter instruction stream the spills of the
-// 80-register build cost more than the sixth CTA gains (3.76 -> 3.43 ms on the 7.2M
-// step).  Fewer hit slots let more CTAs fit but send many more cells of a D3Q27
+// Issue-bound (62 % of the issue slots, 26 of 32 lanes).  Sizes: 4 warps per CTA; a warp's
+// tile of 32 triangles (nine words each: with box and normal staged too it took 3044 us
+// instead of 2973 on 7.2M triangles, D3Q27), 20 hit slots per cell and the byte-wide best-hit
+// indices (shared with the hit queue) take 7.4 KB of shared memory.  The launch bound asks
+// for five CTAs an SM, 96 registers a thread: six (80) take 2888 us there but 742 instead of
+// 730 on 1.0M triangles with D3Q19, and seven are slower on both.  Two ways to test fewer
+// than the 13 lines of a pair, which cost about 13 instructions each once the moments are
+// there, were slower: the lines left by the ranges of the nine linear forms that vanish
+// on them, queued and tested one a lane, 3375 us per pair and 4825 from masks over the
+// block's cells.  Fewer hit slots let more CTAs fit but send many more cells of a D3Q27
 // workload through the per-cell rescan, which costs far more than it saves.
 #define LE_WARPS 4
 #define LE_TILE 32
@@ -155,10 +159,10 @@ __global__ void __launch_bounds__(CAND_BLOCK) k_link_cand(const uint64_t *__rest
 #define LE_SPLIT_COST 16384
 #define LE_SPLIT_MAX 64
 
+// A staged triangle: nine words, so that the lanes' different triangles lie in different
+// banks (with its bounding box and normal, 22 words, two-way conflicts and twice the loads).
 struct TriT {
-    int ax, ay, az, bx, by, bz, cx, cy, cz, id;
-    int lox, loy, loz, hix, hiy, hiz;
-    long long nx, ny, nz;
+    int ax, ay, az, bx, by, bz, cx, cy, cz;
 };
 
 struct LeWarp {
@@ -407,7 +411,10 @@ __device__ __forceinline__ int side_sign64(long long X, long long nx, long long 
 __device__ __forceinline__ bool hit_segment(const TriT &T, long long px, long long py, long long pz, int d, long long h,
                                             float *q)
 {
-    const int nx = (int)T.nx, ny = (int)T.ny, nz = (int)T.nz;
+    // the normal from the edges, modulo 2^32: it fits (above), its products need not
+    const unsigned ux = T.bx - T.ax, uy = T.by - T.ay, uz = T.bz - T.az, vx = T.cx - T.ax, vy = T.cy - T.ay,
+                   vz = T.cz - T.az;
+    const int nx = (int)(uy * vz - uz * vy), ny = (int)(uz * vx - ux * vz), nz = (int)(ux * vy - uy * vx);
     const long long D = (long long)nx * (int)(T.ax - px) + (long long)ny * (int)(T.ay - py) +
                         (long long)nz * (int)(T.az - pz);
     int cx, cy, cz;
@@ -421,12 +428,22 @@ __device__ __forceinline__ bool hit_segment(const TriT &T, long long px, long lo
     return true;
 }
 
+// Normal of a staged triangle, in 64 bits (coordinates below 2^25).
+__device__ __forceinline__ void tri_normal64(const TriT &T, long long &nx, long long &ny, long long &nz)
+{
+    const int ux = T.bx - T.ax, uy = T.by - T.ay, uz = T.bz - T.az, vx = T.cx - T.ax, vy = T.cy - T.ay, vz = T.cz - T.az;
+    nx = (long long)uy * vz - (long long)uz * vy;
+    ny = (long long)uz * vx - (long long)ux * vz;
+    nz = (long long)ux * vy - (long long)uy * vx;
+}
+
 // The same for a line hit of the 64-bit path (coordinates below 2^25, so offsets fit 32
 // bits, |n| < 3 * 2^51 and c . n < 9 * 2^51): D = n . (A - P) in 128 bits.
 __device__ __noinline__ bool hit_segment_wide(const TriT &T, long long px, long long py, long long pz, int d,
                                                  long long h, float *q)
 {
-    const long long nx = T.nx, ny = T.ny, nz = T.nz;
+    long long nx, ny, nz;
+    tri_normal64(T, nx, ny, nz);
     const i128 D = mul128(nx, (int)(T.ax - px)) + mul128(ny, (int)(T.ay - py)) + mul128(nz, (int)(T.az - pz));
     int cx, cy, cz;
     emb_dir(d, cx, cy, cz);
@@ -453,10 +470,12 @@ __device__ __noinline__ bool pair_cross_wide(const TriT &T, long long px, long l
     const long long m3x = qy * az - qz * ay, m3y = qz * ax - qx * az, m3z = qx * ay - qy * ax;
     i128 D = 0;
     bool haveD = false;
-    if (!seg_cross(cx, cy, cz, h, ax, ay, az, bx, by, bz, qx, qy, qz, T.nx, T.ny, T.nz, m1x, m1y, m1z, m2x, m2y, m2z, m3x,
+    long long nx, ny, nz;
+    tri_normal64(T, nx, ny, nz);
+    if (!seg_cross(cx, cy, cz, h, ax, ay, az, bx, by, bz, qx, qy, qz, nx, ny, nz, m1x, m1y, m1z, m2x, m2y, m2z, m3x,
                    m3y, m3z, D, haveD))
         return false;
-    const long long nc = cdot(cx, cy, cz, T.nx, T.ny, T.nz);
+    const long long nc = cdot(cx, cy, cz, nx, ny, nz);
     const i128 N = nc > 0 ? D : -D;
     const long long M = nc > 0 ? nc : -nc;
     *q = __fdiv_rn(i128_to_float(N), (float)M * (float)h);
@@ -480,21 +499,21 @@ __device__ __forceinline__ void link_pair(const TriT &T, long long px, long long
     // coordinates and cell centres lie below 2^25: the offsets fit 32 bits
     const int LIM = 1 << 14;
     const int pxi = (int)px, pyi = (int)py, pzi = (int)pz;
-    const int l0 = T.lox - pxi, h0 = T.hix - pxi, l1 = T.loy - pyi, h1 = T.hiy - pyi, l2 = T.loz - pzi,
-              h2 = T.hiz - pzi;
-    const bool narrow = l0 > -LIM && h0 < LIM && l1 > -LIM && h1 < LIM && l2 > -LIM && h2 < LIM;
+    const int ax = T.ax - pxi, ay = T.ay - pyi, az = T.az - pzi;
+    const int bx = T.bx - pxi, by = T.by - pyi, bz = T.bz - pzi;
+    const int qx = T.cx - pxi, qy = T.cy - pyi, qz = T.cz - pzi;
+    const int out = (ax + LIM) | (ay + LIM) | (az + LIM) | (bx + LIM) | (by + LIM) | (bz + LIM) | (qx + LIM) | (qy + LIM) |
+                    (qz + LIM);
+    const bool narrow = !(out & ~(2 * LIM - 1));  // every offset in [-2^14, 2^14)
     if (narrow) {
-        // Every vertex offset a, b, q lies in (-2^14, 2^14), so in 32-bit integers:
-        //   moment components (a x b etc.): |a_y b_z - a_z b_y| < 2 * 2^28 = 2^29;
-        //   V_k = c . m_k over the at most three nonzero components of c: < 3 * 2^29 < 2^31;
+        // Every vertex offset a, b, q lies in [-2^14, 2^14), so in 32-bit integers:
+        //   moment components (a x b etc.): |a_y b_z - a_z b_y| <= 2 * 2^28 = 2^29;
+        //   V_k = c . m_k over the at most three nonzero components of c: <= 3 * 2^29 < 2^31;
         //   n = m1 + m2 + m3 per component: < 3 * 2^29 < 2^31.
         // c . n is NOT formed in 32 bits: for a corner direction it reaches 9 * 2^29 > 2^31.
         // The line test needs only the signs of V1, V2, V3 (n = m1 + m2 + m3, so c . n =
         // V1 + V2 + V3, which has their common sign when they agree and are nonzero, and a
         // line parallel to the face cannot have three nonzero V of one sign).
-        const int ax = (int)(T.ax - px), ay = (int)(T.ay - py), az = (int)(T.az - pz);
-        const int bx = (int)(T.bx - px), by = (int)(T.by - py), bz = (int)(T.bz - pz);
-        const int qx = (int)(T.cx - px), qy = (int)(T.cy - py), qz = (int)(T.cz - pz);
         const int m1x = ay * bz - az * by, m1y = az * bx - ax * bz, m1z = ax * by - ay * bx;
         const int m2x = by * qz - bz * qy, m2y = bz * qx - bx * qz, m2z = bx * qy - by * qx;
         const int m3x = qy * az - qz * ay, m3y = qz * ax - qx * az, m3z = qx * ay - qy * ax;
@@ -534,9 +553,6 @@ __device__ __forceinline__ void link_pair(const TriT &T, long long px, long long
     } else {
         // coordinates are below 2^25, so offsets fit 32 bits: moments (below 2^51)
         // and their signed sums in 64 bits from widening products
-        const int ax = (int)(T.ax - px), ay = (int)(T.ay - py), az = (int)(T.az - pz);
-        const int bx = (int)(T.bx - px), by = (int)(T.by - py), bz = (int)(T.bz - pz);
-        const int qx = (int)(T.cx - px), qy = (int)(T.cy - py), qz = (int)(T.cz - pz);
         const long long m1x = (long long)ay * bz - (long long)az * by,
                         m1y = (long long)az * bx - (long long)ax * bz,
                         m1z = (long long)ax * by - (long long)ay * bx;
@@ -683,23 +699,15 @@ __global__ void __launch_bounds__(LE_WARPS * 32, LE_MINB) k_link_emit(const __gr
                     s.ax = A.x; s.ay = A.y; s.az = A.z;
                     s.bx = B.x; s.by = B.y; s.bz = B.z;
                     s.cx = C.x; s.cy = C.y; s.cz = C.z;
-                    s.id = (int)id;
-                    s.lox = min(A.x, min(B.x, C.x)); s.hix = max(A.x, max(B.x, C.x));
-                    s.loy = min(A.y, min(B.y, C.y)); s.hiy = max(A.y, max(B.y, C.y));
-                    s.loz = min(A.z, min(B.z, C.z)); s.hiz = max(A.z, max(B.z, C.z));
-                    // edge vectors in 32 bits (coordinates below 2^25), products widened to 64
-                    const int ux = B.x - A.x, uy = B.y - A.y, uz = B.z - A.z;
-                    const int vx = C.x - A.x, vy = C.y - A.y, vz = C.z - A.z;
-                    s.nx = (long long)uy * vz - (long long)uz * vy;
-                    s.ny = (long long)uz * vx - (long long)ux * vz;
-                    s.nz = (long long)ux * vy - (long long)uy * vx;
                     S.tile[lane] = s;
                     // cell i (centre X0 + (2i+1) half) reaches the box iff lo - h <= centre <= hi + h
                     // in 32 bits: coordinates and block origins lie below 2^25, h below 2^19
                     int r0[3], r1[3];
                     const int hh = (int)h + (int)half;
-                    const int lo3[3] = {s.lox - (int)X0, s.loy - (int)Y0, s.loz - (int)Z0};
-                    const int hi3[3] = {s.hix - (int)X0, s.hiy - (int)Y0, s.hiz - (int)Z0};
+                    const int lo3[3] = {min(A.x, min(B.x, C.x)) - (int)X0, min(A.y, min(B.y, C.y)) - (int)Y0,
+                                        min(A.z, min(B.z, C.z)) - (int)Z0};
+                    const int hi3[3] = {max(A.x, max(B.x, C.x)) - (int)X0, max(A.y, max(B.y, C.y)) - (int)Y0,
+                                        max(A.z, max(B.z, C.z)) - (int)Z0};
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const int a_ = lo3[d] - hh;             // ceil(a / h)
@@ -1366,15 +1374,6 @@ __global__ void k_probe(int kind, const long long *__restrict__ in, int64_t n, i
             T.ax = A.x; T.ay = A.y; T.az = A.z;
             T.bx = B.x; T.by = B.y; T.bz = B.z;
             T.cx = C.x; T.cy = C.y; T.cz = C.z;
-            T.id = 0;
-            T.lox = min(A.x, min(B.x, C.x)); T.hix = max(A.x, max(B.x, C.x));
-            T.loy = min(A.y, min(B.y, C.y)); T.hiy = max(A.y, max(B.y, C.y));
-            T.loz = min(A.z, min(B.z, C.z)); T.hiz = max(A.z, max(B.z, C.z));
-            const long long ux = (long long)B.x - A.x, uy = (long long)B.y - A.y, uz = (long long)B.z - A.z;
-            const long long vx = (long long)C.x - A.x, vy = (long long)C.y - A.y, vz = (long long)C.z - A.z;
-            T.nx = uy * vz - uz * vy;
-            T.ny = uz * vx - ux * vz;
-            T.nz = ux * vy - uy * vx;
             uint32_t dm = 0;
             bool wide = false;
             link_pair(
