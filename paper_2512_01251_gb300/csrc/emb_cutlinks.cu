@@ -124,13 +124,14 @@ __global__ void __launch_bounds__(CAND_BLOCK) k_link_cand(const uint64_t *__rest
 // vertices relative to P, the moments m_i of the three edges are formed once; the
 // three Pluecker signs c . m_i test the lines of all 13 direction pairs (c and -c
 // share the line) at once.  When every vertex lies within 2^14 of P the moments fit
-// 32-bit integers; otherwise they are formed in 64 bits by widening products
-// (coarse frames, where h itself is 2^14 or more, take this path).  A pair whose
+// 32-bit integers; up to 2^24 the signs come from float values with an error bound
+// (coarse frames and odd roots, where h itself is 2^14 or more, take this path), beyond
+// that from 64-bit values by widening products.  A pair whose
 // lines hit is queued in the warp's shared memory (tile index, cell, hit
 // directions); the queue is drained 32 hits at a time, one hit per lane, which
 // checks the ends of the segment against the plane (D = n . (A - P) against
-// D - h n.c, in 64 bits, or 128 bits on the wide path) and rounds q.  A zero
-// Pluecker value sends its direction through the exact per-direction test with the
+// D - h n.c, in 64 bits, or 128 bits on the wide paths) and rounds q.  A
+// Pluecker value that is zero, or within the bound, sends its direction through the exact per-direction test with the
 // full tie-break at once.  Crossings are appended to a per-cell bucket; afterwards
 // the owner lane of each cell keeps, per direction, the nearest one (exact rational
 // comparison when a link crosses more than one face), and the warp writes the
