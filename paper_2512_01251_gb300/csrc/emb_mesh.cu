@@ -3,6 +3,7 @@
 #include <limits.h>
 #include <stdlib.h>
 
+#include "emb_edges.cuh"
 #include "emb_internal.cuh"
 
 #define MESH_ERR_ID 1         // vertex id out of range
@@ -29,6 +30,7 @@ struct EdgeTable {
     unsigned long long *slot, *over;  // V x EDGE_SLOTS (NULL: overflow only); cap (a power of two)
     uint64_t cap, probes;             // probes of the overflow table before it counts as full
     uint32_t *done;                   // EDGE_COUNTERS; NULL: no check
+    int *err;                         // the error word: nobody goes on probing a table that is full
 };
 
 // 0: p holds another edge; 1: entered or repeated; 2: completed
@@ -69,8 +71,9 @@ __device__ __forceinline__ bool edge_enter(const EdgeTable &E, uint32_t a, uint3
         const int r = edge_try(E.over + p, __ldcg(E.over + p), key, bit, bad);
         if (r) return r == 2;
         p = (p + 1) & m;
+        if ((it & 15) == 15 && (*(volatile int *)E.err & MESH_ERR_TABLE)) return false;
     }
-    bad |= MESH_ERR_TABLE;
+    atomicOr(E.err, MESH_ERR_TABLE);
     return false;
 }
 
@@ -187,21 +190,16 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
     const int slot = emb_readback_acquire(&rb, &rb_ev);
     if (slot >= 0) head = (uint32_t *)rb;
     const size_t a_head = 512;
-    // room for every edge in a small mesh's overflow table (a triangle has 3/2); in a large
-    // one for a third of them (a few percent overflow, more where a few vertices have many
-    // edges), and a second try with room for all where that is not enough.  A closed mesh
-    // has about T/2 vertices: a list with many more gets no slots for them.
-    const bool slots = check_watertight && V <= 2 * T;
-    int64_t want = !slots || T <= (1 << 16) ? 2 * T : T / 2;
     // records and scratch from the library's pool (stream-ordered on s; the
     // synchronisation below completes them before the mesh is used on any stream)
     if (emb_malloc_async(&m->rec, (size_t)T * 3 * sizeof(int4), s) != cudaSuccess) {
         rc = EMB_ERR_CUDA;
         goto done;
     }
-    for (;;) {
-        uint64_t cap = 1024;
-        while (cap < (uint64_t)want) cap <<= 1;
+    for (int attempt = 0;; ++attempt) {
+        const EdgePlan plan = emb_edge_plan(V, T, attempt);
+        const bool slots = check_watertight && plan.slots;
+        const uint64_t cap = plan.cap;
         const size_t a_slot = slots ? (size_t)V * EDGE_SLOTS * sizeof(unsigned long long) : 0,
                      a_all = a_head + a_slot + (check_watertight ? cap * sizeof(unsigned long long) : 0);
         if (emb_malloc_async(&scratch, a_all, s) != cudaSuccess) {
@@ -210,8 +208,8 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
         }
         cudaMemsetAsync(scratch, 0, a_all, s);
         const EdgeTable E = {slots ? (unsigned long long *)(scratch + a_head) : nullptr,
-                             (unsigned long long *)(scratch + a_head + a_slot), cap, want >= 2 * T ? cap : 128,
-                             check_watertight ? (uint32_t *)scratch + 1 : nullptr};
+                             (unsigned long long *)(scratch + a_head + a_slot), cap, plan.all ? cap : EDGE_PROBES,
+                             check_watertight ? (uint32_t *)scratch + 1 : nullptr, (int *)scratch};
         EMB_LAUNCH((k_mesh_records), emb_grid(T, 256), 256, 0, s)(d_verts, d_tris, V, T, r_o, m->rec, E,
                                                                       (int *)scratch + 1 + EDGE_COUNTERS, (int *)scratch);
         if (cudaGetLastError() != cudaSuccess ||
@@ -221,8 +219,7 @@ extern "C" emb_status emb_mesh_create(const float *d_verts, const int32_t *d_tri
             rc = EMB_ERR_CUDA;
             goto done;
         }
-        if (!(head[0] & MESH_ERR_TABLE) || want >= 2 * T) break;
-        want = 2 * T;
+        if (!(head[0] & MESH_ERR_TABLE) || plan.all) break;
         cudaFreeAsync(scratch, s);
         scratch = nullptr;
     }
