@@ -376,7 +376,9 @@ __global__ void __launch_bounds__(EMB_BIG_BLOCK) k_refine_big(const int4 *__rest
     }
 }
 
-// (rho_L - 1/2) h_L in frame units, or -1 if it is not an integer.
+// (rho_L - 1/2) h_L in frame units, or -1 if it is not an integer.  At most the width of the
+// domain (below 2^25): from there on every block's dilated box holds the whole of it, and
+// box corners stay within the 32 bits that the tests form them in.
 long long emb_refine_dilation(const emb_forest_s *f, int L, int band)
 {
     const int sh = 16;  // rho is kept as an integer multiple of 2^-16
@@ -388,7 +390,8 @@ long long emb_refine_dilation(const emb_forest_s *f, int L, int band)
     long long h = 1ll << (18 - f->k - L);
     long long num = (rho - (1ll << (sh - 1))) * h;
     if (num % (1ll << sh) != 0) return -1;
-    return num >> sh;
+    const long long width = (long long)f->r_o << 20;
+    return (num >> sh) < width ? num >> sh : width;
 }
 
 // The shared memory of the largest copied bitmap is above the default limit; set once a
@@ -457,10 +460,10 @@ extern "C" emb_status emb_refine_flags(emb_forest f, emb_bins b, int32_t level, 
     if (dil < 0) return EMB_ERR_RANGE;
     cudaStream_t s = emb_stream(stream);
     // the flagged bits, and the chunk queue where a triangle may meet more than
-    // EMB_BIG_ITEMS dilated blocks: [-dil, extent + dil] spans at most this many an axis
+    // EMB_BIG_ITEMS dilated blocks: [-dil, extent + dil] spans at most this many an axis, and the level has nb
     const emb_mesh m = b->m;
     const LevelGeom g = level_geom(f, level);
-    const long long span = ((m->ext + 2 * dil) >> g.lW) + 2;
+    const long long most = ((m->ext + 2 * dil) >> g.lW) + 2, span = most < g.nb ? most : g.nb;
     EmbBigQ Q = emb_bigq(m->T);
     if (emb_mesh_big(m, span, span, span)) Q.cap = (uint32_t)emb_bigq_capacity(m->T);
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
