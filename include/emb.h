@@ -492,7 +492,8 @@ emb_status emb_cutlinks_backward(emb_mesh m, emb_forest f, const int32_t *d_cell
  * headroom 0 the counts must match the plan exactly (EMB_ERR_STATE otherwise).
  * emb_batch_counts: the blocks per level (levels[j] + 1 int64) and links of mesh j in
  * the last replay (host arrays, either may be NULL); with headroom they are read from the
- * device, which synchronises `stream`.
+ * device, which synchronises `stream` (before the first replay: the root level and nothing
+ * else).
  *
  * emb_batch_info: planned blocks per level (levels[j] + 1 int64) and link count of
  * mesh j (host): the capacities of a batch with headroom.  emb_batch_results copies mesh

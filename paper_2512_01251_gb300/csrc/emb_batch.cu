@@ -180,12 +180,14 @@ static void headroom_caps(BMesh &B, int headroom)
 }
 
 // Allocates every buffer of a replay of mesh B.
-static emb_status alloc_mesh(BMesh &B, int headroom)
+static emb_status alloc_mesh(BMesh &B, int headroom, cudaStream_t s)
 {
     const int64_t T = B.m->T;
     if (headroom > 0) {
         headroom_caps(B, headroom);
         BTRY(balloc(B, &B.d_n, EMB_MAX_LEVELS + 2));
+        // until the first replay: no blocks below the root, no links
+        EMB_CUDA_TRY(cudaMemsetAsync(B.d_n, 0, (EMB_MAX_LEVELS + 2) * sizeof(uint32_t), s));
         for (int L = 1; L <= B.Lf; ++L) B.L[L].lv.d_n = B.d_n + L;
     }
     int64_t nmax = 1, wmax = 1;
@@ -344,7 +346,7 @@ extern "C" emb_status emb_batch_create_ex(const emb_mesh *meshes, const int32_t 
         B.band = bands[j];
         B.lattice = lattices[j];
         rc = plan_mesh(B, s);
-        if (rc == EMB_OK) rc = alloc_mesh(B, b->headroom);
+        if (rc == EMB_OK) rc = alloc_mesh(B, b->headroom, s);
     }
     if (rc == EMB_OK && cudaMalloc(&b->next, sizeof(unsigned int)) != cudaSuccess) rc = EMB_ERR_CUDA;
     if (rc == EMB_OK) rc = emb_link_emit_init();  // kernel attributes are set outside of any capture
@@ -748,7 +750,7 @@ static emb_status replay_counts(const BMesh &B, cudaStream_t s, int64_t *blocks,
     int64_t nl = 0;
     memcpy(&nl, h + EMB_MAX_LEVELS, sizeof(nl));
     for (int L = 1; L <= B.Lf; ++L) blocks[L] = h[L] < (uint64_t)B.L[L].lv.n ? h[L] : B.L[L].lv.n;
-    *links = nl < B.links ? nl : B.links;
+    *links = nl < 0 ? 0 : (nl < B.links ? nl : B.links);
     return EMB_OK;
 }
 
