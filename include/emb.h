@@ -433,7 +433,9 @@ emb_status emb_lbm_step(emb_forest f, int32_t lattice, const int32_t *d_cell, co
  * units): d_gverts (V x 3 float32, overwritten) = sum_k d_gq[k] dq_k/dV with
  * dq/dV_j = lambda_j n / (h n.c) for the three vertices of link k's triangle
  * (lambda: barycentric coordinates of the hit point, n: face normal, h: cell
- * size).  Summed per vertex in integers (the order does not matter: the same bits every run). */
+ * size).  The hit point is the crossing itself where d_q[k] is the value that the link
+ * table holds for it, and lies at the given d_q[k] otherwise.  Summed per vertex in
+ * integers (the order does not matter: the same bits every run). */
 emb_status emb_cutlinks_backward(emb_mesh m, emb_forest f, const int32_t *d_cell, const uint8_t *d_dir,
                                  const float *d_q, const int32_t *d_tri, int64_t n, const float *d_gq,
                                  float *d_gverts, void *stream);

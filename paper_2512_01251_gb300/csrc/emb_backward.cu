@@ -459,7 +459,7 @@ __device__ __forceinline__ long long lat_det(const int a[3], const int b[3], int
 }
 
 // The three terms of one link in FP64 with the hit point taken at the given q, for a q
-// that is not the link's crossing, a line parallel to its triangle, and a gq that is no
+// that is not the table's value of the crossing, a line parallel to its triangle, and a gq that is no
 // normal number; non-finite terms come back as flags.
 __device__ __noinline__ uint32_t qb_terms_wide(const int a[3], const int b[3], const int c3[3], const long long n[3],
                                                int cx, int cy, int cz, double s_, double f, F2 t[3], int &ex)
@@ -566,13 +566,14 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restri
         long long nn[3];
         tri_normal(A, B, C, nn);
         const float qk = q[k], gk = gq[k];
-        // the crossing of the link's line with the plane, D / (h c.n) in steps of the link: a
-        // q that is not it (within 2^-20, rounding included) takes the general path
+        // the crossing of the link's line with the plane, D / (h c.n) in steps of the link,
+        // rounded as the link table's q is: there the weights are those of the crossing itself,
+        // any other q (one ulp off, too) takes the general path with the hit point at that q
         const i128 D = mul128(nn[0], a[0]) + mul128(nn[1], a[1]) + mul128(nn[2], a[2]);
         const long long M = nc < 0 ? -nc : nc;
-        const float Nf = D < 0 ? -i128_to_float(-D) : i128_to_float(D), Mh = (float)M * (float)g.h;
+        const float Nf = D < 0 ? -i128_to_float(-D) : i128_to_float(D);
         const uint32_t ge = (__float_as_uint(gk) >> 23) & 255u;
-        const bool usual = M != 0 && fabsf(qk * Mh - (nc < 0 ? -Nf : Nf)) <= 0x1p-20f * Mh &&
+        const bool usual = M != 0 && qk == __fdiv_rn(nc < 0 ? -Nf : Nf, (float)M * (float)g.h) &&
                            (gk == 0.0f || ge - 1u < 254u);
         if (usual) {
             const int kb = 63 - __clzll(M);
