@@ -3,8 +3,8 @@
 // vertices (Sec. 2.2 cites both methods; Sec. 3.4 builds the q table they use).
 //
 // All reductions are independent of the order in which the GPU runs: the force takes
-// per-thread and per-warp sums of float pairs, per-CTA sums in FP64 and one CTA over the
-// partials in index order; the per-vertex sums are integers.  No floating-point atomics
+// per-thread and per-warp sums of three floats each, per-CTA sums in FP64 and one CTA over
+// the partials in index order; the per-vertex sums are integers.  No floating-point atomics
 // are used.
 #include <mutex>
 
@@ -65,10 +65,16 @@ __device__ __forceinline__ LinkPops link_pops(int64_t k, const int32_t *__restri
     return L;
 }
 
-// Pairs of floats (h + l, l below half an ulp of h): the terms below carry about 46 bits
-// with them, at FP32 rate.  This chip has two FP64 lanes a clock and SM against 128 FP32
-// ones: with the same terms in FP64 both kernels were bound by them (1.72 M links, D3Q19:
-// force 120 -> 14 us with the link's cells in L2, 42 us from HBM; dF/dq 92 -> 9 us).
+// Floats in pairs (h + l, l below half an ulp of h) and in threes, in place of FP64: this chip
+// has two FP64 lanes a clock and SM against 128 FP32 ones, and with the terms in FP64 the force
+// and dF/dq kernels were bound by them (1.72 M links, D3Q19: 131 and 97 us a call).  The sums and
+// products below are the error-free transformations of Knuth (two_sum) and Dekker (two_prod,
+// by fma).
+//   dF/dq, a single value a link: pairs, about 46 bits, rounded to FP32 at once (25 us).
+//   The force, a signed sum over a closed body, most of which cancels: threes, which carry a
+//   link's term to about 2^-66 of it and a thread's sums to less than FP64's 2^-53 of theirs.
+//   1.72 M links of D3Q19: 131 us with FP64, 43 now (51 from a cold L2), the call; pairs
+//   took 43 (52).
 // Bound now by the gathers of the populations.
 struct F2 {
     float h, l;
@@ -104,7 +110,30 @@ __device__ __forceinline__ F2 f2_div(F2 a, F2 b)
     const float r = __fadd_rn(__fmaf_rn(-x, b.h, a.h), __fmaf_rn(-x, b.l, a.l));
     return f2_norm(x, __fdiv_rn(r, b.h));
 }
-__device__ __forceinline__ F2 f2_neg(F2 a) { return {-a.h, -a.l}; }
+
+// a + b + c: b collects the errors of the sums in a, c those of b.
+struct F3 {
+    float a, b, c;
+};
+__device__ __forceinline__ void f3_low(F3 &s, float x)  // x of the size of s.b
+{
+    const F2 t = two_sum(s.b, x);
+    s.b = t.h;
+    s.c = __fadd_rn(s.c, t.l);
+}
+__device__ __forceinline__ void f3_add(F3 &s, float x)
+{
+    const F2 t = two_sum(s.a, x);
+    s.a = t.h;
+    f3_low(s, t.l);
+}
+__device__ __forceinline__ void f3_add(F3 &s, F3 x)
+{
+    f3_add(s, x.a);
+    f3_low(s, x.b);
+    s.c = __fadd_rn(s.c, x.c);
+}
+__device__ __forceinline__ double f3_value(F3 s) { return (double)s.a + ((double)s.b + (double)s.c); }
 
 // Zero, or a magnitude in [2^-40, 2^41): sums, products and quotients of a few such values
 // neither overflow nor lose low parts to underflow.
@@ -118,7 +147,7 @@ __device__ __forceinline__ bool link_safe(const LinkPops &L)
     return L.q >= 0.0f && L.q <= 1.0f && f2_safe(L.f_i) && f2_safe(L.f_o) && f2_safe(L.f_p);
 }
 
-// Fixed-order block reduction of three doubles; thread 0 receives the sums.
+// Fixed-order block reduction of three doubles; every thread receives the sums.
 __device__ __forceinline__ void block_sum3(double &a, double &b, double &c)
 {
     __shared__ double s[3][MEX_BLOCK];
@@ -145,31 +174,55 @@ __global__ void __launch_bounds__(MEX_BLOCK) k_mex_partial(const int32_t *__rest
                                                            const int32_t *__restrict__ nbr,
                                                            const uint64_t *__restrict__ mask, double *__restrict__ part)
 {
-    F2 ax = {0.0f, 0.0f}, ay = ax, az = ax;
-    double fx = 0, fy = 0, fz = 0;  // links outside the pairs' range (NaN and infinities too)
+    F3 ax = {0.0f, 0.0f, 0.0f}, ay = ax, az = ax;
+    double fx = 0, fy = 0, fz = 0;  // links outside the range of the threes (NaN and infinities too)
     bool wild = false;
+    int held = 0;
     for (int64_t k = (int64_t)blockIdx.x * MEX_BLOCK + threadIdx.x; k < n; k += (int64_t)gridDim.x * MEX_BLOCK) {
         const LinkPops L = link_pops(k, cell, dir, q, pop, stride, nbr, mask);
         if (link_safe(L)) {
             const float q2 = 2.0f * L.q;
-            F2 m;  // f_i plus the population returned against it
+            F3 m = {L.f_i, 0.0f, 0.0f};  // f_i plus the population returned against it
             if (L.q < 0.5f) {
                 // 2 f_i, or f_i + 2q f_i + (1 - 2q) f_p
-                m = {2.0f * L.f_i, 0.0f};
                 if (L.has) {
-                    const F2 w = two_sum(1.0f, -q2);
-                    F2 b = two_prod(w.h, L.f_p);
-                    b.l = __fmaf_rn(w.l, L.f_p, b.l);
-                    m = f2_add(f2_add(two_prod(q2, L.f_i), b), {L.f_i, 0.0f});
+                    const F2 w = two_sum(1.0f, -q2), p = two_prod(q2, L.f_i), b = two_prod(w.h, L.f_p),
+                             e = two_prod(w.l, L.f_p);
+                    f3_add(m, p.h);
+                    f3_add(m, b.h);
+                    f3_low(m, p.l);
+                    f3_low(m, b.l);
+                    f3_low(m, e.h);
+                    m.c = __fadd_rn(m.c, e.l);
+                } else {
+                    m.a = 2.0f * L.f_i;
                 }
             } else {
-                // f_i + (f_i + (2q - 1) f_o) / 2q; 2q - 1 is exact on [1/2, 1]
-                const F2 N = f2_add(two_prod(__fsub_rn(q2, 1.0f), L.f_o), {L.f_i, 0.0f});
-                m = f2_add(f2_div(N, {q2, 0.0f}), {L.f_i, 0.0f});
+                // f_i + (f_i + (2q - 1) f_o) / 2q; 2q - 1 is exact on [1/2, 1].  The quotient in
+                // three steps, each from the remainder of the ones before (the first one's exact)
+                const F2 p = two_prod(__fsub_rn(q2, 1.0f), L.f_o), N = two_sum(p.h, L.f_i);
+                const float x0 = __fdiv_rn(N.h, q2);
+                F3 r = {__fmaf_rn(-x0, q2, N.h), 0.0f, 0.0f};
+                f3_add(r, N.l);
+                f3_add(r, p.l);
+                const float inv = __frcp_rn(q2), x1 = __fmul_rn(r.a, inv);
+                const float x2 = __fmul_rn(__fadd_rn(__fmaf_rn(-x1, q2, r.a), __fadd_rn(r.b, r.c)), inv);
+                f3_add(m, x0);
+                f3_low(m, x1);
+                m.c = __fadd_rn(m.c, x2);
             }
-            if (L.cx) ax = f2_add(ax, L.cx > 0 ? m : f2_neg(m));
-            if (L.cy) ay = f2_add(ay, L.cy > 0 ? m : f2_neg(m));
-            if (L.cz) az = f2_add(az, L.cz > 0 ? m : f2_neg(m));
+            const float sx = (float)L.cx, sy = (float)L.cy, sz = (float)L.cz;  // -1, 0, 1
+            f3_add(ax, {sx * m.a, sx * m.b, sx * m.c});
+            f3_add(ay, {sy * m.a, sy * m.b, sy * m.c});
+            f3_add(az, {sz * m.a, sz * m.b, sz * m.c});
+            if (++held == 64) {  // the last float of a three rounds at each sum: few of them
+                fx += f3_value(ax);
+                fy += f3_value(ay);
+                fz += f3_value(az);
+                ax = ay = az = {0.0f, 0.0f, 0.0f};
+                held = 0;
+                wild = true;
+            }
         } else {
             const double qq = L.q, f_i = L.f_i;
             double g;
@@ -182,19 +235,25 @@ __global__ void __launch_bounds__(MEX_BLOCK) k_mex_partial(const int32_t *__rest
             wild = true;
         }
     }
-    // the warps' pairs first (FP32), then one FP64 value a warp
+    // the warps' threes first (FP32), then one FP64 value a warp: a lane keeps x and y or z of
+    // itself and the lane 16 on, then one of the three, so that the warp's sums take 6 additions
+    // and 18 exchanged floats a lane instead of 15 and 45 (x ends in lane 0, y in 8, z in 16)
     __shared__ double s_warp[3][MEX_BLOCK / 32];
+    const int lane = threadIdx.x & 31;
+    const bool hi = lane & 16, mid = lane & 8;
+    auto other = [&](const F3 &v, int o) -> F3 {
+        return {__shfl_xor_sync(0xffffffffu, v.a, o), __shfl_xor_sync(0xffffffffu, v.b, o),
+                __shfl_xor_sync(0xffffffffu, v.c, o)};
+    };
+    F3 s = hi ? az : ax;
+    f3_add(s, other(hi ? ax : az, 16));
+    f3_add(ay, other(ay, 16));
+    const F3 out = hi || mid ? s : ay, in = other(out, 8);
+    if (!hi && mid) s = ay;
+    f3_add(s, in);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        ax = f2_add(ax, {__shfl_xor_sync(0xffffffffu, ax.h, o), __shfl_xor_sync(0xffffffffu, ax.l, o)});
-        ay = f2_add(ay, {__shfl_xor_sync(0xffffffffu, ay.h, o), __shfl_xor_sync(0xffffffffu, ay.l, o)});
-        az = f2_add(az, {__shfl_xor_sync(0xffffffffu, az.h, o), __shfl_xor_sync(0xffffffffu, az.l, o)});
-    }
-    if ((threadIdx.x & 31) == 0) {
-        s_warp[0][threadIdx.x >> 5] = (double)ax.h + (double)ax.l;
-        s_warp[1][threadIdx.x >> 5] = (double)ay.h + (double)ay.l;
-        s_warp[2][threadIdx.x >> 5] = (double)az.h + (double)az.l;
-    }
+    for (int o = 4; o > 0; o >>= 1) f3_add(s, other(s, o));
+    if ((lane & 7) == 0 && lane < 24) s_warp[lane >> 3][threadIdx.x >> 5] = f3_value(s);
     if (__syncthreads_or(wild)) block_sum3(fx, fy, fz);
     if (threadIdx.x < 3) {
         double v = threadIdx.x == 0 ? s_warp[0][0] : (threadIdx.x == 1 ? s_warp[1][0] : s_warp[2][0]);
