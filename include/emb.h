@@ -370,8 +370,8 @@ emb_status emb_cutlinks(emb_forest f, emb_bins b, int32_t lattice, int32_t *d_ce
  *                                           fluid cell of the finest level.
  * d_pop: D3Q19/D3Q27 populations (post-collision), layout [Q][pop_stride]
  * indexed by finest cell id (pop_stride >= 64 * blocks).  d_F: 3 floats.
- * Terms and sums carry at least the precision of FP64 (error 2^-51 of the summed
- * magnitudes |f_i + g| before F is rounded to float).
+ * Terms and sums carry the precision of FP64 or more: an error below 2^-48 of the
+ * summed magnitudes |f_i + g| before F is rounded to float.
  * Deterministic fixed-order reduction (no float atomics). */
 emb_status emb_mex_force(emb_forest f, int32_t lattice, const int32_t *d_cell, const uint8_t *d_dir,
                          const float *d_q, int64_t n, const float *d_pop, int64_t pop_stride, float *d_F,

@@ -377,7 +377,10 @@ emb_status emb_device_view(void *p, void **dp, bool *device)
     }
     if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) {
         *dp = p;
-        if (device) *device = a.type == cudaMemoryTypeDevice;
+        if (device) {
+            int here = -1;
+            *device = cudaGetDevice(&here) == cudaSuccess && emb_plain_device(a, here);
+        }
         return EMB_OK;
     }
     if (a.type == cudaMemoryTypeHost && a.devicePointer) {

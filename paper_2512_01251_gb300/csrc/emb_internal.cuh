@@ -234,7 +234,12 @@ emb_status emb_enq_level_index(EmbLevel &lv, uint64_t *tmp, cudaStream_t s);
 emb_status emb_build_hash(EmbLevel &lv, cudaStream_t s);
 // Device address of a caller output buffer (device memory, or page-locked host memory
 // through its mapping); EMB_ERR_BAD_INPUT for pageable memory.  NULL stays NULL.  *device:
-// plain device memory.
+// plain memory of the current device, which any kernel can store to; another device's is
+// reached by copies (a kernel's stores would need peer access).
+static inline bool emb_plain_device(const cudaPointerAttributes &a, int here)
+{
+    return a.type == cudaMemoryTypeDevice && a.device == here;
+}
 emb_status emb_device_view(void *p, void **dp, bool *device = nullptr);
 #define EMB_RB_WORDS 64
 // A pinned host slot (EMB_RB_WORDS words) and its event for a count read-back; -1 when none is free.
