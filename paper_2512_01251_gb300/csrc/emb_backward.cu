@@ -555,8 +555,8 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restri
                                                          const int32_t *__restrict__ cell, const uint8_t *__restrict__ dir,
                                                          const float *__restrict__ q, const int32_t *__restrict__ tri,
                                                          const float *__restrict__ gq, int64_t n,
-                                                         const int4 *__restrict__ rec, int64_t T,
-                                                         QbEntry *__restrict__ ent, int *__restrict__ tile_n,
+                                                         const int4 *__restrict__ rec, int64_t T, int64_t nblk,
+                                                         int64_t m3, QbEntry *__restrict__ ent, int *__restrict__ tile_n,
                                                          int *__restrict__ vexp, uint32_t *__restrict__ vflag, int *st)
 {
     __shared__ int s_key[QB_HASH];                     // triangle of a hash slot (-1: free)
@@ -611,6 +611,10 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restri
         slot[u] = s;
         const int4 A = rec[3 * tr], B = rec[3 * tr + 1], C = rec[3 * tr + 2];
         const int64_t c = cell[k];
+        if (!emb_ck((uint64_t)(c >> 6), (uint64_t)nblk, st)) {
+            slot[u] = -1;
+            continue;
+        }
         const uint64_t bk = key[c >> 6];
         const int tc = (int)(c & 63), half = (int)g.half;
         const int px = (2 * (4 * (int)(bk & EMB_KEY_MASK) + (tc & 3)) + 1) * half;
@@ -699,6 +703,7 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restri
 #pragma unroll
             for (int x = 0; x < 3; ++x) {
                 const int64_t at = 3 * (int64_t)vid[j] + x;
+                if (!emb_ck((uint64_t)at, (uint64_t)m3, st)) continue;
                 if (E.m[j] != 0 && nn[x] != 0)
                     atomicMax(vexp + at, E.e[j] + mb + 64 - __clzll(nn[x] < 0 ? -nn[x] : nn[x]));
                 // an infinite term times a component of n: its sign, or NaN where that is 0
@@ -716,7 +721,8 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_tile(const uint64_t *__restri
 // below 2^63 in it.
 __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_scatter(const QbEntry *__restrict__ ent, const int *__restrict__ tile_n,
                                                             const int4 *__restrict__ rec, const int *__restrict__ vexp,
-                                                            int qbits, unsigned long long *__restrict__ vacc)
+                                                            int qbits, int64_t m3,
+                                                            unsigned long long *__restrict__ vacc, int *st)
 {
     const int cnt = tile_n[blockIdx.x];
     for (int i = threadIdx.x; i < cnt; i += QB_BLOCK) {
@@ -731,6 +737,7 @@ __global__ void __launch_bounds__(QB_BLOCK) k_qbwd_scatter(const QbEntry *__rest
             for (int x = 0; x < 3; ++x) {
                 if (E.m[j] == 0 || nn[x] == 0) continue;
                 const int64_t at = 3 * (int64_t)vid[j] + x;
+                if (!emb_ck((uint64_t)at, (uint64_t)m3, st)) continue;
                 const int sh = vexp[at] - qbits - E.e[j];  // quanta of E.e per quantum of the vertex, log2
                 const i128 P = mul128(E.m[j], nn[x]);
                 if (sh > 120) continue;
@@ -787,8 +794,8 @@ extern "C" emb_status emb_cutlinks_backward(emb_mesh m, emb_forest f, const int3
     EMB_CUDA_TRY(cudaMemsetAsync(vexp, 0x80, a_v, s));
     if (n > 0) {
         EMB_LAUNCH((k_qbwd_tile), (int)nt, QB_BLOCK, 0, s)(lv.key, g, m->r_o, d_cell, d_dir, d_q, d_tri, d_gq, n, m->rec,
-                                                           m->T, ent, tile_n, vexp, vflag, st);
-        EMB_LAUNCH((k_qbwd_scatter), (int)nt, QB_BLOCK, 0, s)(ent, tile_n, m->rec, vexp, qbits, vacc);
+                                                           m->T, lv.n, m3, ent, tile_n, vexp, vflag, st);
+        EMB_LAUNCH((k_qbwd_scatter), (int)nt, QB_BLOCK, 0, s)(ent, tile_n, m->rec, vexp, qbits, m3, vacc, st);
     }
     EMB_LAUNCH((k_qbwd_write), emb_grid(m3, 256), 256, 0, s)(vexp, vflag, vacc, m3, qbits, d_gverts);
     EMB_CUDA_TRY(cudaGetLastError());

@@ -95,7 +95,7 @@ __global__ void k_xfilter_bits(const int4 *__restrict__ rec, int64_t T, LevelGeo
 // the same launch a tile's records wait for the look-back: 139 instead of 61 us a level
 // on 7.2M triangles.)
 #define FLIST_TILE 512
-__global__ void __launch_bounds__(FLIST_TILE) k_filter_list(const uint32_t *__restrict__ word, int64_t W,
+__global__ void __launch_bounds__(FLIST_TILE) k_filter_list(const uint32_t *__restrict__ word, int64_t W, int64_t T,
                                                             uint32_t *__restrict__ flist, uint32_t *__restrict__ count,
                                                             uint64_t *__restrict__ state, uint64_t expect, int *st)
 {
@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(FLIST_TILE) k_filter_list(const uint32_t *__re
     while (m) {
         const int b = __ffs(m) - 1;
         m &= m - 1;
-        flist[o++] = (uint32_t)(32 * i + b);
+        if (emb_ck(o, (uint64_t)T, st)) flist[o] = (uint32_t)(32 * i + b);
+        ++o;
     }
 }
 
@@ -491,7 +492,7 @@ emb_status emb_enq_filter(const int4 *rec, int64_t T, LevelGeom g, uint32_t *fli
     const int bs = block < 32 ? 32 : block - block % 32;
     if (tiles > 1 && !zeroed) EMB_CUDA_TRY(cudaMemsetAsync(state, 0, emb_filter_state_words(T) * sizeof(uint64_t), s));
     if (T > 0) EMB_LAUNCH((k_xfilter_bits), emb_grid(T, bs), bs, 0, s)(rec, T, g, word);
-    EMB_LAUNCH((k_filter_list), (int)tiles, FLIST_TILE, 0, s)(word, (T + 31) / 32, flist, count, tiles > 1 ? state : nullptr,
+    EMB_LAUNCH((k_filter_list), (int)tiles, FLIST_TILE, 0, s)(word, (T + 31) / 32, T, flist, count, tiles > 1 ? state : nullptr,
                                                               expect, st);
     EMB_CUDA_TRY(cudaGetLastError());
     return EMB_OK;

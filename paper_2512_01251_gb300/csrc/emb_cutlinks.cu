@@ -1028,7 +1028,7 @@ __global__ void __launch_bounds__(LISTS_BLOCK) k_link_lists(const uint32_t *__re
         if (base + i <= n) {
             if (links > 0xFFFFFFFFull) emb_set_status(st, EMB_ERR_CAPACITY);
             blk_off[base + i] = (uint32_t)links;
-            if (v[i]) work[blocks] = (uint32_t)(base + i);
+            if (v[i] && emb_ck(blocks, (uint64_t)n, st)) work[blocks] = (uint32_t)(base + i);
             if (base + i == n) {
                 *work_n = blocks;
                 if ((expect_work != EMB_NO_EXPECT && blocks != expect_work) ||

@@ -71,6 +71,10 @@ __global__ void k_make_children(const EmbLevel P, const uint8_t *__restrict__ fl
         rh = rank_below(P.bits, P.wpre, row + nb);
         pll = rank_below(P.bits, P.wpre, plane);
         plh = rank_below(P.bits, P.wpre, plane + nb * nb);
+        // entries of rank, which holds n + 1
+        if (!emb_ck((uint64_t)rl, (uint64_t)n + 1, st) || !emb_ck((uint64_t)rh, (uint64_t)n + 1, st) ||
+            !emb_ck((uint64_t)pll, (uint64_t)n + 1, st) || !emb_ck((uint64_t)plh, (uint64_t)n + 1, st))
+            return;
     } else {
         const uint64_t row0 = k & ~EMB_KEY_MASK, row1 = row0 + (1ull << EMB_KEY_BITS);
         const uint64_t pl0 = k & ~((1ull << (2 * EMB_KEY_BITS)) - 1ull), pl1 = pl0 + (1ull << (2 * EMB_KEY_BITS));

@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(64 * LBM_BLOCKS, Q == 19 ? 10 : 9) k_lbm_step(
                                                               const uint32_t *__restrict__ bits, float *__restrict__ out,
                                                               int64_t stride, int64_t nblk,
                                                               const int32_t *__restrict__ nbr,
-                                                              const uint64_t *__restrict__ mask, float omega)
+                                                              const uint64_t *__restrict__ mask, float omega, int *st)
 {
     __shared__ uint64_t s_mask[LBM_BLOCKS * 27];
     __shared__ int32_t s_id[LBM_BLOCKS * 27];
@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(64 * LBM_BLOCKS, Q == 19 ? 10 : 9) k_lbm_step(
         const int j = threadIdx.x / 27, code = threadIdx.x - 27 * j;
         int32_t id = -1;
         if (b0 + j < nblk) id = code == 13 ? (int32_t)(b0 + j) : nbr[(b0 + j) * 26 + c_lbm_dir_of_offset[code] - 1];
+        if (id >= 0 && !emb_ck((uint64_t)id, (uint64_t)nblk, st)) id = -1;
         s_id[threadIdx.x] = id;
         s_mask[threadIdx.x] = id >= 0 ? mask[id] : 0ull;
     }
@@ -228,10 +229,10 @@ extern "C" emb_status emb_lbm_step(emb_forest f, int32_t lattice, const int32_t 
         const int grid = emb_grid(lv.n, LBM_BLOCKS);
         if (lattice == 19)
             EMB_LAUNCH((k_lbm_step<19>), grid, 64 * LBM_BLOCKS, 0, s)(d_pop, d_pre, bits, d_pop_out, pop_stride, lv.n,
-                                                                      lv.nbr, lv.mask, omega);
+                                                                      lv.nbr, lv.mask, omega, st);
         else
             EMB_LAUNCH((k_lbm_step<27>), grid, 64 * LBM_BLOCKS, 0, s)(d_pop, d_pre, bits, d_pop_out, pop_stride, lv.n,
-                                                                      lv.nbr, lv.mask, omega);
+                                                                      lv.nbr, lv.mask, omega, st);
         EMB_CUDA_TRY(cudaGetLastError());
         return EMB_OK;
     }

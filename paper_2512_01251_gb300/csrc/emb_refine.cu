@@ -56,6 +56,9 @@ __device__ __forceinline__ unsigned long long refine_items(const long long b0[3]
 struct TodoBits {
     uint32_t *w;  // null: no dense bits, look the block up and test the flag bytes
     long long nb;
+    int *st;
+    // bounds mode: position p is one of the level's
+    __device__ __forceinline__ bool in(unsigned long long p) const { return emb_ck(p, (uint64_t)nb * nb * nb, st); }
     __device__ __forceinline__ unsigned long long pos(long long bx, long long by, long long bz) const
     {
         return (unsigned long long)((bz * nb + by) * nb + bx);
@@ -63,17 +66,18 @@ struct TodoBits {
     __device__ __forceinline__ bool test(long long bx, long long by, long long bz) const
     {
         const unsigned long long p = pos(bx, by, bz);
-        return (w[p >> 5] >> (p & 31)) & 1u;
+        return in(p) && ((w[p >> 5] >> (p & 31)) & 1u);
     }
     __device__ __forceinline__ void clear(long long bx, long long by, long long bz) const
     {
         const unsigned long long p = pos(bx, by, bz);
-        atomicAnd(w + (p >> 5), ~(1u << (p & 31)));
+        if (in(p)) atomicAnd(w + (p >> 5), ~(1u << (p & 31)));
     }
     // bits [0, nx) of the row segment from (bx, by, bz), nx <= 32
     __device__ __forceinline__ uint32_t row(int bx, int by, int bz, int nx) const
     {
         const unsigned long long p = pos(bx, by, bz);
+        if (!in(p + (unsigned)(nx - 1))) return 0u;
         const int sh = (int)(p & 31);
         const uint32_t lo = w[p >> 5], hi = sh + nx > 32 ? w[(p >> 5) + 1] : 0u;
         return __funnelshift_r(lo, hi, sh) & (0xffffffffu >> (32 - nx));
@@ -184,7 +188,7 @@ __global__ void __launch_bounds__(REFINE_WARPS * 32, REFINE_MINB) k_refine(const
         for (int i = threadIdx.x; i < nw; i += REFINE_WARPS * 32) s_todo[i] = __ldcg(todo + i);
         __syncthreads();
     }
-    const TodoBits td = {SM ? s_todo : todo, g.nb};
+    const TodoBits td = {SM ? s_todo : todo, g.nb, lk.st};
     const int64_t first = (int64_t)blockIdx.x * chunk, all = (T + 31) / 32;
     const int64_t ntiles = first + chunk < all ? first + chunk : all, stride = REFINE_WARPS;
     int64_t tile = first + w;
@@ -418,7 +422,7 @@ emb_status emb_enq_refine(const int4 *rec, int64_t T, LevelGeom g, long long dil
     const emb_status ri = refine_init();
     if (ri != EMB_OK) return ri;
     const EmbLookup lk = emb_lookup_of(lv);
-    TodoBits td = {nullptr, g.nb};
+    TodoBits td = {nullptr, g.nb, lk.st};
     const int64_t nw = emb_bitmap_words(lv.nb_axis);
     if (fbits && lv.bits && nw > 0) {
         EMB_CUDA_TRY(cudaMemcpyAsync(fbits, lv.bits, nw * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));

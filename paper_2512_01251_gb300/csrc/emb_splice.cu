@@ -101,8 +101,8 @@ __global__ void k_sp_compact_keys(const uint64_t *__restrict__ key, const uint32
 // newid[i] = merged id of block i, or -1 when it is not selected.
 __global__ void k_sp_place(const uint64_t *__restrict__ key, const uint64_t *__restrict__ mask,
                            const uint32_t *__restrict__ sel, const uint32_t *__restrict__ pos, int64_t n,
-                           const uint64_t *__restrict__ other, int64_t n_other, uint64_t *__restrict__ mkey,
-                           uint64_t *__restrict__ mmask, int32_t *__restrict__ newid)
+                           const uint64_t *__restrict__ other, int64_t n_other, int64_t room, uint64_t *__restrict__ mkey,
+                           uint64_t *__restrict__ mmask, int32_t *__restrict__ newid, int *st)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -111,6 +111,7 @@ __global__ void k_sp_place(const uint64_t *__restrict__ key, const uint64_t *__r
         return;
     }
     const int64_t p = (int64_t)pos[i] + lower_bound_u64(other, n_other, key[i]);
+    if (!emb_ck((uint64_t)p, (uint64_t)room, st)) return;
     mkey[p] = key[i];
     mmask[p] = mask[i];
     newid[i] = (int32_t)p;
@@ -118,7 +119,7 @@ __global__ void k_sp_place(const uint64_t *__restrict__ key, const uint64_t *__r
 
 // The bits of the selected blocks of one side in the merged level's bitmap.
 __global__ void k_sp_bits(const uint64_t *__restrict__ key, int64_t n, int64_t nb, RowWindow W, int L, bool want_inside,
-                          unsigned long long *__restrict__ bits)
+                          unsigned long long *__restrict__ bits, int *st)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -126,6 +127,7 @@ __global__ void k_sp_bits(const uint64_t *__restrict__ key, int64_t n, int64_t n
     if (W.inside(k, L) != want_inside) return;
     const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
                   bz = (int64_t)(k >> (2 * EMB_KEY_BITS)), lin = (bz * nb + by) * nb + bx;
+    if (!emb_ck((uint64_t)lin, (uint64_t)nb * nb * nb, st)) return;
     atomicOr(bits + (lin >> 6), 1ull << (lin & 63));
 }
 
@@ -133,8 +135,8 @@ __global__ void k_sp_bits(const uint64_t *__restrict__ key, int64_t n, int64_t n
 // of its bit: it takes its key and mask there.  newid[i] as in k_sp_place (NULL: not wanted).
 __global__ void k_sp_rank(const uint64_t *__restrict__ key, const uint64_t *__restrict__ mask, int64_t n, int64_t nb,
                           RowWindow W, int L, bool want_inside, const uint64_t *__restrict__ bits,
-                          const uint32_t *__restrict__ wpre, uint64_t *__restrict__ mkey, uint64_t *__restrict__ mmask,
-                          int32_t *__restrict__ newid)
+                          const uint32_t *__restrict__ wpre, int64_t room, uint64_t *__restrict__ mkey,
+                          uint64_t *__restrict__ mmask, int32_t *__restrict__ newid, int *st)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -145,7 +147,9 @@ __global__ void k_sp_rank(const uint64_t *__restrict__ key, const uint64_t *__re
     }
     const int64_t bx = (int64_t)(k & EMB_KEY_MASK), by = (int64_t)((k >> EMB_KEY_BITS) & EMB_KEY_MASK),
                   bz = (int64_t)(k >> (2 * EMB_KEY_BITS)), lin = (bz * nb + by) * nb + bx;
+    if (!emb_ck((uint64_t)lin, (uint64_t)nb * nb * nb, st)) return;
     const int64_t p = (int64_t)wpre[lin >> 6] + __popcll(bits[lin >> 6] & ((1ull << (lin & 63)) - 1ull));
+    if (!emb_ck((uint64_t)p, (uint64_t)room, st)) return;
     mkey[p] = k;
     mmask[p] = mask[i];
     if (newid) newid[i] = (int32_t)p;
@@ -168,10 +172,10 @@ __global__ void k_sp_link_starts(const int32_t *__restrict__ cell, int64_t nl, i
 
 // Links per merged block, from the side each merged block came from.
 __global__ void k_sp_link_counts(const int32_t *__restrict__ newid, int64_t n, const uint32_t *__restrict__ start,
-                                 uint32_t *__restrict__ cnt)
+                                 int64_t room, uint32_t *__restrict__ cnt, int *st)
 {
     const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < n && newid[b] >= 0) cnt[newid[b]] = start[b + 1] - start[b];
+    if (b < n && newid[b] >= 0 && emb_ck((uint64_t)newid[b], (uint64_t)room, st)) cnt[newid[b]] = start[b + 1] - start[b];
 }
 
 // Copies the links of the selected blocks of one side to their merged place.
@@ -180,11 +184,12 @@ __global__ void k_sp_link_copy(const int32_t *__restrict__ cell, const uint8_t *
                                const int32_t *__restrict__ newid, const uint32_t *__restrict__ start,
                                const uint32_t *__restrict__ moff, const int32_t *__restrict__ tri_map, int64_t cap,
                                int32_t *__restrict__ o_cell, uint8_t *__restrict__ o_dir, float *__restrict__ o_q,
-                               int32_t *__restrict__ o_tri)
+                               int32_t *__restrict__ o_tri, int64_t nblk, int *st)
 {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= nl) return;
     const int64_t b = cell[k] >> 6;
+    if (!emb_ck((uint64_t)b, (uint64_t)nblk, st)) return;
     const int32_t nb = newid[b];
     if (nb < 0) return;
     const int64_t o = (int64_t)moff[nb] + (k - (int64_t)start[b]);
@@ -243,6 +248,8 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
     cudaStream_t s = emb_stream(stream);
     const RowWindow W = {y0, y1, z0, z1};
     emb_status rc = EMB_OK;
+    int *st = emb_status_word();
+    if (!st) return EMB_ERR_CUDA;
     SpliceScratch S(s);
     // merged blocks per level and, last, the links: in a page-locked slot where one is free
     uint32_t here[EMB_MAX_LEVELS + 1], *counts = here;
@@ -278,17 +285,17 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
             EMB_CUDA_TRY(S.get(&m.mask, np + nq + 1));
             EMB_CUDA_TRY(cudaMemsetAsync(m.bits, 0, zw * sizeof(uint64_t), s));
             unsigned long long *mb = (unsigned long long *)m.bits;
-            if (np > 0) EMB_LAUNCH((k_sp_bits), emb_grid(np, 256), 256, 0, s)(P.key, np, P.nb_axis, W, L, false, mb);
-            if (nq > 0) EMB_LAUNCH((k_sp_bits), emb_grid(nq, 256), 256, 0, s)(Q.key, nq, P.nb_axis, W, L, true, mb);
+            if (np > 0) EMB_LAUNCH((k_sp_bits), emb_grid(np, 256), 256, 0, s)(P.key, np, P.nb_axis, W, L, false, mb, st);
+            if (nq > 0) EMB_LAUNCH((k_sp_bits), emb_grid(nq, 256), 256, 0, s)(Q.key, nq, P.nb_axis, W, L, true, mb, st);
             rc = emb_scan_popc(m.bits, m.wpre, nw, m.bits + nw, true, s);
             if (rc != EMB_OK) return rc;
             EMB_CUDA_TRY(cudaMemcpyAsync(counts + L, m.wpre + nw, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
             if (np > 0)
                 EMB_LAUNCH((k_sp_rank), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, np, P.nb_axis, W, L, false, m.bits,
-                                                                      m.wpre, m.key, m.mask, L == Lf ? idP : nullptr);
+                                                                      m.wpre, np + nq, m.key, m.mask, L == Lf ? idP : nullptr, st);
             if (nq > 0)
                 EMB_LAUNCH((k_sp_rank), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, nq, P.nb_axis, W, L, true, m.bits,
-                                                                      m.wpre, m.key, m.mask, L == Lf ? idQ : nullptr);
+                                                                      m.wpre, np + nq, m.key, m.mask, L == Lf ? idQ : nullptr, st);
             EMB_CUDA_TRY(cudaGetLastError());
             n_fin = np + nq;
         } else {
@@ -317,9 +324,9 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
             EMB_CUDA_TRY(S.get(&m.key, n + 1));
             EMB_CUDA_TRY(S.get(&m.mask, n + 1));
             if (np > 0)
-                EMB_LAUNCH((k_sp_place), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, selP, posP, np, cQ, kq, m.key, m.mask, idP);
+                EMB_LAUNCH((k_sp_place), emb_grid(np, 256), 256, 0, s)(P.key, P.mask, selP, posP, np, cQ, kq, n, m.key, m.mask, idP, st);
             if (nq > 0)
-                EMB_LAUNCH((k_sp_place), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, selQ, posQ, nq, cP, kp, m.key, m.mask, idQ);
+                EMB_LAUNCH((k_sp_place), emb_grid(nq, 256), 256, 0, s)(Q.key, Q.mask, selQ, posQ, nq, cP, kp, n, m.key, m.mask, idQ, st);
             EMB_CUDA_TRY(cudaGetLastError());
             counts[L] = (uint32_t)n;
             n_fin = n;
@@ -339,8 +346,8 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
         EMB_CUDA_TRY(cudaMemsetAsync(cnt, 0, (n + 1) * sizeof(uint32_t), s));
         EMB_LAUNCH((k_sp_link_starts), emb_grid(np + 1, 256), 256, 0, s)(f_cell, f_n, np, stP);
         EMB_LAUNCH((k_sp_link_starts), emb_grid(nq + 1, 256), 256, 0, s)(w_cell, w_n, nq, stQ);
-        if (np > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(np, 256), 256, 0, s)(idP, np, stP, cnt);
-        if (nq > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(nq, 256), 256, 0, s)(idQ, nq, stQ, cnt);
+        if (np > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(np, 256), 256, 0, s)(idP, np, stP, n, cnt, st);
+        if (nq > 0) EMB_LAUNCH((k_sp_link_counts), emb_grid(nq, 256), 256, 0, s)(idQ, nq, stQ, n, cnt, st);
         EMB_CUDA_TRY(cudaGetLastError());
         rc = emb_scan_into(cnt, moff, n, tmp, s);
         if (rc != EMB_OK) return rc;
@@ -355,10 +362,10 @@ extern "C" emb_status emb_splice(emb_forest f, emb_forest w, int32_t y0, int32_t
             if (!o_cell || !o_dir || !o_q || !o_tri) return EMB_ERR_BAD_INPUT;
             if (f_n > 0)
                 EMB_LAUNCH((k_sp_link_copy), emb_grid(f_n, 256), 256, 0, s)(f_cell, f_dir, f_q, f_tri, f_n, idP, stP, moff,
-                                                                           nullptr, capacity, o_cell, o_dir, o_q, o_tri);
+                                                                           nullptr, capacity, o_cell, o_dir, o_q, o_tri, np, st);
             if (w_n > 0)
                 EMB_LAUNCH((k_sp_link_copy), emb_grid(w_n, 256), 256, 0, s)(w_cell, w_dir, w_q, w_tri, w_n, idQ, stQ, moff,
-                                                                           w_tri_map, capacity, o_cell, o_dir, o_q, o_tri);
+                                                                           w_tri_map, capacity, o_cell, o_dir, o_q, o_tri, nq, st);
             EMB_CUDA_TRY(cudaGetLastError());
         }
     }
