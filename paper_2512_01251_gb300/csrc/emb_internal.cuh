@@ -610,8 +610,9 @@ struct WuTri {
 // thread that finds the queue full walks its items itself: the queue's size
 // affects the speed only, never the result.
 // A small mesh has few warps, which leave the chip idle while each lane walks its own
-// triangle: its line lies at 8 items, and a triangle gets up to 16 chunks of 64 before
-// their size grows to EMB_BIG_CHUNK (1,103 triangles on 384 cells an axis, 35 warps: refine,
+// triangle: its line lies at 8 items (where there is a queue: the per-call path has none as
+// long as no triangle can have more than EMB_BIG_ITEMS, emb_mesh_big), and a triangle gets up
+// to 16 chunks of 64 before their size grows to EMB_BIG_CHUNK (1,103 triangles on 384 cells an axis, 35 warps: refine,
 // voxelize and bin kernels 700 -> 140 us, embed_1k_fine 1346 -> 771 us).
 #define EMB_BIG_ITEMS 64
 #define EMB_BIG_CHUNK 512

@@ -4,15 +4,17 @@
 // computation).  The paper prints neither the collision model nor Bouzidi's rule; the
 // textbook BGK collision with the D3Q19 / D3Q27 weights and the linear Bouzidi rule of
 // emb_mex_force are used.  Populations are SoA, pop[i * stride + cell], cell = block *
-// 64 + x + 4 y + 16 z on the finest level.  Three passes, each its own kernel so that
-// the cost of the boundary treatment can be timed against the rest:
-//   k_lbm_stream   pull streaming into pre-collision populations: f_i(x) = f*_i(x - c_i)
-//                  when x - c_i is a fluid cell of the level, f*_i(x) when its block is
-//                  missing (zero gradient at the edge of the level: the coupling to
-//                  coarser levels is out of scope), left for the next pass when solid;
-//   k_lbm_bouzidi  per cut link (x, d, q): the population entering x against c_d, from
-//                  f*_d(x), f*_d(x - c_d) and f*_-d(x) by the linear rule;
-//   k_lbm_collide  BGK f* = f - omega (f - f_eq(rho, u)) at fluid cells, 0 at solid ones.
+// 64 + x + 4 y + 16 z on the finest level.  The step is
+//   pull streaming  f_i(x) = f*_i(x - c_i) when x - c_i is a fluid cell of the level, f*_i(x)
+//                   when its block is missing (zero gradient at the edge of the level: the
+//                   coupling to coarser levels is out of scope), left open when solid;
+//   Bouzidi         per cut link (x, d, q): the population entering x against c_d, from
+//                   f*_d(x), f*_d(x - c_d) and f*_-d(x) by the linear rule;
+//   collision       BGK f* = f - omega (f - f_eq(rho, u)) at fluid cells, 0 at solid ones.
+// The whole step runs as k_lbm_bouzidi and then k_lbm_step, which streams and collides in one
+// pass over the cells.  Its parts by themselves (the phases of emb_lbm_step, so that the cost
+// of the boundary treatment can be timed against the rest) are k_lbm_stream, k_lbm_bouzidi and
+// k_lbm_collide.
 #include "emb_internal.cuh"
 
 // direction index of a block offset (ox, oy, oz) in {-1,0,1}^3, code (ox+1) + 3(oy+1) + 9(oz+1)

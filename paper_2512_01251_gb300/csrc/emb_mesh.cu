@@ -21,7 +21,9 @@
 // most meshes, so the slots they touch are neighbours too; a table addressed by hash alone
 // missed the L2 on every access and held every directed edge twice as sparsely (7.2M
 // triangles: records 100 us, clear + insert + look-up of the reverse 1150 us; now 434 us
-// for all, and 25 for the clear).  The mesh is closed and
+// for all, and 25 for the clear; with triangles and vertices shuffled a mesh of 7.2M takes 790
+// us in all instead of 1380, of 1.0M 160 instead of 161).  Sizes: emb_edges.cuh.  The mesh is
+// closed and
 // oriented iff no direction is seen twice and every edge is completed by its other one:
 // 3T/2 completions.
 #define EDGE_SLOTS 4

@@ -170,9 +170,11 @@ __device__ __forceinline__ void ref_drain(RefWarp &S, int &qn, int n, int lane, 
 // union is a box).  Otherwise every lane goes through the blocks left
 // among its own triangle's candidates: a vertex in the dilated block flags it, else the
 // pair waits for the separating-axis test, which the warp runs 32 at a time.
-// Latency-bound; four CTAs an SM (64 registers) over three: 5 % on 7.2M triangles.  Time over
-// the levels, before (the union's or the spread pairs' blocks looked up and tested at once,
-// global flag bits) and now: 7.2M triangles 1311 -> 899 us, 1.0M 311 -> 229, 111K 118 -> 91.
+// Latency-bound; four CTAs an SM (64 registers, which spill 188 bytes of stores and 84 of loads
+// a thread) over three: 5 % on 7.2M triangles.  Time over the levels, before (the union's or
+// the spread pairs' blocks looked up and tested at once, global flag bits) and now: 7.2M
+// triangles 1311 -> 860 us, 1.0M 311 -> 231, 111K 118 -> 91.  Triangles and vertices in any
+// order: an embedding of 7.2M shuffled ones 10.4 -> 7.2 ms, of 1.0M 2.26 -> 1.80.
 // Taking the union's blocks left one at a time for the whole warp is slower on most levels
 // (986 us, 111K: 154).
 template <bool SM>
