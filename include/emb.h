@@ -255,6 +255,7 @@ emb_status emb_voxelize_guard(emb_forest f, emb_bins b, uint64_t *d_solid_mask, 
  * closed block box dilated by (rho_L - 1/2) cells, where rho = band at level
  * max_level-1 and rho_L = max(band, rho_{L+1}/2 + 5/2) above it.  This keeps the
  * 2:1 balance of Sec. 3.2 and leaves every unrefined block free of the surface.
+ * A band as wide as the domain or wider flags every block.
  * d_flags: one uint8 per level block (1 = refine), overwritten.
  * Errors: EMB_ERR_BAD_INPUT (band < 1), EMB_ERR_STATE, EMB_ERR_RANGE. */
 emb_status emb_refine_flags(emb_forest f, emb_bins b, int32_t level, int32_t band, uint8_t *d_flags,
